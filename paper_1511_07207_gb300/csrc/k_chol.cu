@@ -22,9 +22,9 @@
 //   grid barrier per step; every read of W goes to L2 (ld.global.cg).  After
 //   the last step the panel's l's are written into W's panel columns.
 // chol_trail_kernel: the trailing lower triangle (rows k1 .. n, columns
-//   k1 .. min(i, n - 1)) in 64 x 64 tiles: each element takes the panel's 32
-//   updates in order from the panel's l's staged in shared memory (two FP64
-//   instructions an element and step: bound by the FP64 pipe).
+//   k1 .. min(i, n - 1)) in 32 x 32 tiles: each element takes the panel's 32
+//   updates in order from the panel's l's staged in shared memory, the product on
+//   the integer pipes and the difference on the FP64 pipe (ls_rank.cuh).
 // chol_backsolve_kernel (cooperative): L^T x = y by blocks of 64 rows from
 //   the bottom: CTA 0 solves the diagonal block (one warp), then every CTA
 //   subtracts the block's contribution l_ji x_j from the rows above it (a
@@ -33,11 +33,12 @@
 // forward substitution; x differs from a scalar back substitution by the
 // order of its sums.
 //
-// Work: n^3 / 6 updates of two FP64 instructions (half of the LU's).
+// Work: n^3 / 6 updates, a rounded product and a rounded difference each (half of the LU's).
 #include <cuda_runtime.h>
 
 #include "ls_device.cuh"
 #include "ls_internal.h"
+#include "ls_rank.cuh"
 
 namespace lsi {
 
@@ -46,8 +47,8 @@ constexpr int CT = 512;            // threads per CTA of the cooperative kernels
 constexpr int CW = CT / 32;
 constexpr int CH_NB = 32;          // panel width
 constexpr int CH_ROWS = 4;         // rows a warp loads before it computes
-constexpr int CTT = 64;            // trailing-update tile
 constexpr int CB = 64;             // rows per back-substitution block
+static_assert(CH_NB == RANK_NB, "panel width");
 }  // namespace
 
 __global__ void __launch_bounds__(CT, 1) chol_panel_kernel(CholArgs a, int k0, int k1) {
@@ -107,8 +108,9 @@ __global__ void __launch_bounds__(CT, 1) chol_panel_kernel(CholArgs a, int k0, i
 
 // Rows k1 .. n, columns k1 .. min(i, n - 1): w_ij -= l_it l_jt for the
 // panel's steps t in order.
-__global__ void __launch_bounds__(256) chol_trail_kernel(CholArgs a, int k0, int nb) {
-    __shared__ double Ls[CTT][CH_NB + 1], Ms[CH_NB][CTT];
+__global__ void __launch_bounds__(RANK_T, 4) chol_trail_kernel(CholArgs a, int k0, int nb) {
+    constexpr int RT = RANK_R, TT = RANK_TT, PITCH = RANK_PITCH;
+    __shared__ Op53 Ls[CH_NB * PITCH], Ms[CH_NB * PITCH];
     State *st = a.st;
     count_launch(st);
     if (*(volatile int *)&st->status == LS_BREAKDOWN) return;
@@ -117,39 +119,33 @@ __global__ void __launch_bounds__(256) chol_trail_kernel(CholArgs a, int k0, int
     double *W = a.W;
     const double *Lp = a.Lp;
     const int k1 = k0 + nb;
-    const int r0 = k1 + blockIdx.y * CTT, c0 = k1 + blockIdx.x * CTT;
-    if (c0 > r0 + CTT - 1) return;               // the tile lies above the diagonal
-    for (int e = threadIdx.x; e < CTT * CH_NB; e += blockDim.x) {
+    const int r0 = k1 + blockIdx.y * TT, c0 = k1 + blockIdx.x * TT;
+    if (c0 > r0 + TT - 1) return;                // the tile lies above the diagonal
+    // rows and columns past the block are staged as ones and not stored
+    RankRange range;
+    for (int e = threadIdx.x; e < TT * CH_NB; e += RANK_T) {
         const int r = e / CH_NB, t = e % CH_NB;
-        Ls[r][t] = (r0 + r <= n && t < nb) ? __ldcg(&Lp[(long long)(r0 + r) * CH_NB + t]) : 0.0;
-        const int tt = e / CTT, c = e % CTT;
-        Ms[tt][c] = (c0 + c < n && tt < nb) ? __ldcg(&Lp[(long long)(c0 + c) * CH_NB + tt]) : 0.0;
+        const Op53 l = op53_a((r0 + r <= n && t < nb) ? __ldcg(&Lp[(long long)(r0 + r) * CH_NB + t]) : 1.0);
+        const Op53 m = op53_b((c0 + r < n && t < nb) ? __ldcg(&Lp[(long long)(c0 + r) * CH_NB + t]) : 1.0);
+        range.a(l);
+        range.b(m);
+        Ls[t * PITCH + r] = l;
+        Ms[t * PITCH + r] = m;
     }
-    __syncthreads();
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    double acc[4][4];
+    double acc[RT][RT];
 #pragma unroll
-    for (int p = 0; p < 4; p++)
+    for (int p = 0; p < RT; p++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
+        for (int q = 0; q < RT; q++) {
             const int r = r0 + ty + 16 * p, c = c0 + tx + 16 * q;
             acc[p][q] = (r <= n && c < n && c <= r) ? W[(long long)r * ld + c] : 0.0;
         }
-    for (int t = 0; t < nb; t++) {
-        double l[4], m[4];
+    rank_tile(acc, Ls, Ms, nb, range.all_in_range(), ty, tx);
 #pragma unroll
-        for (int p = 0; p < 4; p++) l[p] = Ls[ty + 16 * p][t];
+    for (int p = 0; p < RT; p++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) m[q] = Ms[t][tx + 16 * q];
-#pragma unroll
-        for (int p = 0; p < 4; p++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) acc[p][q] = __dsub_rn(acc[p][q], __dmul_rn(l[p], m[q]));
-    }
-#pragma unroll
-    for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        for (int q = 0; q < RT; q++) {
             const int r = r0 + ty + 16 * p, c = c0 + tx + 16 * q;
             if (r <= n && c < n && c <= r) W[(long long)r * ld + c] = acc[p][q];
         }
@@ -209,7 +205,7 @@ CholKernels chol_kernels() {
     K.backsolve = reinterpret_cast<void *>(&chol_backsolve_kernel);
     K.zero_upper = reinterpret_cast<void *>(&chol_zero_upper_kernel);
     K.nb = CH_NB;
-    K.tile = CTT;
+    K.tile = RANK_TT;
     K.block = CT;
     return K;
 }

@@ -31,22 +31,22 @@
 // lu_u12_kernel: the panel's pivot rows right of the panel (the paper's
 //   triangular solve for U01): the panel's updates t = k0 .. in order, four
 //   lanes a column, each holding 8 of the 32 values in registers.
-// lu_trail_kernel: the block below and right of the panel, 64 x 64 tiles:
+// lu_trail_kernel: the block below and right of the panel, 32 x 32 tiles:
 //   each element takes the panel's 32 updates in order from the multipliers
-//   and pivot rows staged in shared memory.  This is where the time goes:
-//   two FP64 instructions per element and step (a product and a difference,
-//   not fused), so the elimination is bound by the FP64 pipe, and A crosses
-//   DRAM once per panel instead of once per step.
+//   and pivot rows staged in shared memory, the product on the integer pipes and
+//   the difference on the FP64 pipe (ls_rank.cuh).  This is where the time
+//   goes; A crosses DRAM once per panel instead of once per step.
 // lu_backsolve_kernel (cooperative): U x = y by blocks of 64 rows from the
 //   bottom: CTA 0 solves the diagonal block (one warp, column oriented),
 //   then every CTA subtracts the block's contribution from the rows above
 //   it (a warp a row).  Two grid barriers per block.
 //
-// Work: n^3 / 3 updates of two FP64 instructions; traffic about 16 n^3 / (3 LU_NB) bytes.
+// Work: n^3 / 3 updates, a rounded product and a rounded difference each; traffic about 16 n^3 / (3 LU_NB) bytes.
 #include <cuda_runtime.h>
 
 #include "ls_device.cuh"
 #include "ls_internal.h"
+#include "ls_rank.cuh"
 
 namespace lsi {
 
@@ -58,7 +58,7 @@ constexpr int U12_T = 128;         // threads per CTA of lu_u12_kernel (32 colum
 constexpr int LU_NB = 32;          // panel width
 constexpr int LW = LT / 32;        // warps per CTA
 constexpr int LB = 64;             // rows per back-substitution block
-constexpr int TT = 64;             // trailing-update tile (rows and columns)
+static_assert(LU_NB == RANK_NB, "panel width");
 
 struct Cand {
     double v;
@@ -245,8 +245,9 @@ __global__ void __launch_bounds__(U12_T) lu_u12_kernel(LuArgs a, int k0, int nb)
 
 // The block below and right of the panel (rows k0 + LU_NB .. n - 1, columns
 // k0 + LU_NB .. n): a_ij -= l_it u_tj for the panel's steps t in order.
-__global__ void __launch_bounds__(256) lu_trail_kernel(LuArgs a, int k0) {
-    __shared__ double Ls[TT][LU_NB + 1], Us[LU_NB][TT];
+__global__ void __launch_bounds__(RANK_T, 4) lu_trail_kernel(LuArgs a, int k0) {
+    constexpr int RT = RANK_R, TT = RANK_TT, PITCH = RANK_PITCH;
+    __shared__ Op53 Ls[LU_NB * PITCH], Us[LU_NB * PITCH];
     State *st = a.st;
     count_launch(st);
     if (*(volatile int *)&st->status == LS_BREAKDOWN) return;
@@ -254,38 +255,32 @@ __global__ void __launch_bounds__(256) lu_trail_kernel(LuArgs a, int k0) {
     const long long ld = a.ld;
     double *W = a.W;
     const int r0 = k0 + LU_NB + blockIdx.y * TT, c0 = k0 + LU_NB + blockIdx.x * TT;
-    for (int e = threadIdx.x; e < TT * LU_NB; e += blockDim.x) {
+    // rows and columns past the block are staged as ones and not stored
+    RankRange range;
+    for (int e = threadIdx.x; e < TT * LU_NB; e += RANK_T) {
         const int r = e / LU_NB, t = e % LU_NB;
-        Ls[r][t] = r0 + r < n ? W[(long long)(r0 + r) * ld + k0 + t] : 0.0;
+        const Op53 l = op53_a(r0 + r < n ? W[(long long)(r0 + r) * ld + k0 + t] : 1.0);
         const int tt = e / TT, c = e % TT;
-        Us[tt][c] = c0 + c <= n ? W[(long long)(k0 + tt) * ld + c0 + c] : 0.0;
+        const Op53 u = op53_b(c0 + c <= n ? W[(long long)(k0 + tt) * ld + c0 + c] : 1.0);
+        range.a(l);
+        range.b(u);
+        Ls[t * PITCH + r] = l;
+        Us[tt * PITCH + c] = u;
     }
-    __syncthreads();
     const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
-    double acc[4][4];
+    double acc[RT][RT];
 #pragma unroll
-    for (int p = 0; p < 4; p++)
+    for (int p = 0; p < RT; p++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
+        for (int q = 0; q < RT; q++) {
             const int r = r0 + ty + 16 * p, c = c0 + tx + 16 * q;
             acc[p][q] = (r < n && c <= n) ? W[(long long)r * ld + c] : 0.0;
         }
-#pragma unroll 4
-    for (int t = 0; t < LU_NB; t++) {
-        double l[4], u[4];
+    rank_tile(acc, Ls, Us, LU_NB, range.all_in_range(), ty, tx);
 #pragma unroll
-        for (int p = 0; p < 4; p++) l[p] = Ls[ty + 16 * p][t];
+    for (int p = 0; p < RT; p++)
 #pragma unroll
-        for (int q = 0; q < 4; q++) u[q] = Us[t][tx + 16 * q];
-#pragma unroll
-        for (int p = 0; p < 4; p++)
-#pragma unroll
-            for (int q = 0; q < 4; q++) acc[p][q] = __dsub_rn(acc[p][q], __dmul_rn(l[p], u[q]));
-    }
-#pragma unroll
-    for (int p = 0; p < 4; p++)
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
+        for (int q = 0; q < RT; q++) {
             const int r = r0 + ty + 16 * p, c = c0 + tx + 16 * q;
             if (r < n && c <= n) W[(long long)r * ld + c] = acc[p][q];
         }
@@ -339,8 +334,8 @@ LuKernels lu_kernels() {
     K.u12 = reinterpret_cast<void *>(&lu_u12_kernel);
     K.trail = reinterpret_cast<void *>(&lu_trail_kernel);
     K.nb = LU_NB;
+    K.tile = RANK_TT;
     K.u12_block = U12_T;
-    K.tile = TT;
     K.block = LT;
     return K;
 }
