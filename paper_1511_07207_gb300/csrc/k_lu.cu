@@ -14,18 +14,12 @@
 // t = 0, 1, ... in order, as a rounded product and a rounded difference.
 // Per panel:
 // lu_factor_kernel (cooperative, over the panel's steps, its columns only):
-//   * the pivot candidates of column k are the CTAs' partial maxima (value
-//     and first row index), formed while updating the previous column and
-//     reduced by every CTA (a total order, so all CTAs pick the same v);
-//   * rows k and v are swapped over the panel's columns by the whole grid;
-//   * each row i > k belongs to one warp: l = w_ik / w_kk (IEEE division),
-//     w_ij = w_ij - l * w_kj as a separate multiply and subtract (no fused
-//     multiply-add), so every element is bit for bit what the same
-//     elimination gives in plain FP64 arithmetic; the warp also forms the
-//     row's next pivot candidate |w_i,k+1|.
-//   Two bounded grid barriers per step.  A row is updated by different warps
-//   at different steps and swapped by any CTA, so every read of W here goes
-//   to L2 (ld.global.cg), never to a possibly stale L1 line.
+//   every CTA owns rows of the panel; per step the CTAs exchange their best
+//   pivot candidates (value, row, and that row's entries), pick the same one (a
+//   total order) and each divides and updates its rows: l = w_ik / w_kk (IEEE
+//   division), w_ij = w_ij - l * w_kj as a separate multiply and subtract (no
+//   fused multiply-add), so every element is bit for bit what the same
+//   elimination gives in plain FP64 arithmetic.
 // lu_laswp_kernel: the panel's row swaps on every other column (a thread a
 //   column, the swaps in step order).
 // lu_u12_kernel: the panel's pivot rows right of the panel (the paper's
@@ -53,124 +47,244 @@ namespace lsi {
 namespace {
 
 constexpr int LT = 512;            // threads per CTA (16 warps: enough loads in flight)
-constexpr int LU_ROWS = 4;         // rows a warp loads before it computes (panel steps)
 constexpr int U12_T = 128;         // threads per CTA of lu_u12_kernel (32 columns)
 constexpr int LU_NB = 32;          // panel width
 constexpr int LW = LT / 32;        // warps per CTA
+constexpr int FT = 256, FW = FT / 32;   // threads and warps of a panel CTA
+constexpr int SLOTS = 5;           // candidates a lane fetches at a time (152 CTAs)
 constexpr int LB = 64;             // rows per back-substitution block
 static_assert(LU_NB == RANK_NB, "panel width");
 
+// A pivot candidate: |a| as its bit pattern, which orders as the value does
+// (-1 for NaN and for no candidate at all), its row, and the place in its CTA.
+// Integer comparisons: one of doubles takes 64 cycles of a scheduler's FP64
+// unit, and a step makes dozens (473 -> 421 ms for the whole solve at n = 8192).
 struct Cand {
-    double v;
-    int i;
+    long long v;
+    int i, r;
 };
+__device__ __forceinline__ Cand make_cand(double x, int i, int r) {
+    const long long m = __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll;
+    return Cand{m > 0x7FF0000000000000ll ? -1ll : m, i, r};
+}
+__device__ __forceinline__ Cand no_cand(int n) { return Cand{-1, n, -1}; }
 
-// The better of two pivot candidates: the larger |a|, the first row on ties.
+// The better of two pivot candidates: the larger |a|, the first row on ties.  A
+// total order, so the order of a reduction does not change its result.
 __device__ __forceinline__ Cand better(Cand a, Cand b) {
-    if (b.v > a.v || (b.v == a.v && b.i < a.i)) return b;
-    return a;
+    const bool take = b.v > a.v || (b.v == a.v && b.i < a.i);
+    return Cand{take ? b.v : a.v, take ? b.i : a.i, take ? b.r : a.r};
+}
+__device__ __forceinline__ Cand warp_better(Cand c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        c = better(c, Cand{__shfl_xor_sync(0xffffffffu, c.v, o), __shfl_xor_sync(0xffffffffu, c.i, o),
+                           __shfl_xor_sync(0xffffffffu, c.r, o)});
+    return c;
 }
 
-// This CTA's candidate from its warps' candidates (fixed order) into part.
-__device__ void publish_cand(const LuArgs &a, Cand mine, Cand *red) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) red[warp] = mine;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        Cand c = red[0];
-        for (int w = 1; w < LW; w++) c = better(c, red[w]);
-        a.cand_v[blockIdx.x] = c.v;
-        a.cand_i[blockIdx.x] = c.i;
-    }
+// What the CTAs tell each other travels as 16-byte words (a value, an index and
+// the step + 1), written and read whole: a word with the expected step
+// carries its own data, so no fence separates data from a flag.
+__device__ __forceinline__ void st_word(LuWord *p, long long v, int i, unsigned seq) {
+    const unsigned long long lo = (unsigned long long)v, hi = ((unsigned long long)seq << 32) | (unsigned)i;
+    asm volatile("{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}" ::"l"(p),
+                 "l"(lo), "l"(hi)
+                 : "memory");
+}
+__device__ __forceinline__ unsigned ld_word(const LuWord *p, long long &v, int &i) {
+    unsigned long long lo, hi;
+    asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p)
+                 : "memory");
+    v = (long long)lo;
+    i = (int)(unsigned)hi;
+    return (unsigned)(hi >> 32);
+}
+// Waits for the word of step seq; false after the library's limit.
+__device__ __forceinline__ bool wait_word(const LuWord *p, unsigned seq, long long &v, int &i) {
+    if (ld_word(p, v, i) == seq) return true;
+    const unsigned long long t0 = gtimer();
+    while (ld_word(p, v, i) != seq)
+        if (gtimer() - t0 > WAIT_LIMIT_NS) return false;
+    return true;
 }
 
 }  // namespace
 
-__global__ void __launch_bounds__(LT, 1) lu_factor_kernel(LuArgs a, int k0, int k1) {
-    // k0 .. k1 - 1: the steps of one panel, whose columns are k0 .. k1 - 1
-    __shared__ Cand red[LW];
-    __shared__ int v_s;
+// The panel's steps k0 .. k1 - 1 on its own columns.  A CTA owns `R` rows of the
+// panel for all of its steps, in shared memory (or, when they do not fit, in a
+// buffer in global memory), so a row crosses HBM twice a panel.  Rows stay where
+// they are and only their positions change with the swaps; at the end each
+// row is written to its position.
+//
+// A step is one exchange, made by warp 0: it publishes the CTA's best candidate and that
+// row's entries, waits for every CTA's candidate, and fetches the winner's
+// row.  Then, a thread a row: the swap of positions, l_i = w_ik / w_kk, the
+// update of column k + 1 and the next candidate; the columns right of it are updated by
+// the other warps while warp 0 makes the next exchange (which finishes the
+// candidate's row itself).  The words are double buffered by the parity of k: a
+// CTA writes step k + 2's only after it has seen every CTA's step k + 1, which
+// each publishes after it has read step k's.
+//
+// What bounds it is the chain of a step: the exchange (two L2 round trips), a division,
+// an update and two barriers of the CTA.  Two barriers of the grid and all rows read
+// from L2 in every step took 15 us a step at n = 8192; whole solve 477 -> 393 ms,
+// n = 1500 21.8 -> 9.4 ms.
+template <bool SMEM>
+__global__ void __launch_bounds__(FT, 1) lu_factor_kernel(LuArgs a, int k0, int k1, int R) {
+    extern __shared__ __align__(16) double sm[];
+    __shared__ Cand red[FW];
+    __shared__ double prow_s[2][LU_NB];
+    __shared__ int v_s, ok_s;                    // the pivot's position (-1: no comparable candidate); no timeout
     State *st = a.st;
     count_launch(st);
-    const int n = a.n;
-    const long long ld = a.ld;
-    double *W = a.W;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gw = blockIdx.x * LW + warp, nw = gridDim.x * LW;
     if (*(volatile int *)&st->status == LS_BREAKDOWN) return;
-    {   // candidates of the panel's first column (rows k0 .. n-1)
-        Cand mine = {-1.0, n};
-        for (int i = k0 + gw; i < n; i += nw)
-            if (lane == 0) mine = better(mine, Cand{fabs(__ldcg(&W[(long long)i * ld + k0])), i});
-        publish_cand(a, mine, red);
+    constexpr int P = SMEM ? LU_NB + 1 : LU_NB;
+    const int n = a.n, nb = k1 - k0, G = gridDim.x, cta = blockIdx.x;
+    const long long ld = a.ld;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int first = k0 + cta * R, mine = max(0, min(R, n - first));
+    int *pos = reinterpret_cast<int *>(sm);                           // [R] current position of each row
+    double *w = SMEM ? sm + (R + 1) / 2 : a.rowbuf + (size_t)cta * R * LU_NB;
+    for (int e = threadIdx.x; e < mine * LU_NB; e += FT) {
+        const int r = e / LU_NB, t = e % LU_NB;
+        w[r * P + t] = t < nb ? a.W[(long long)(first + r) * ld + k0 + t] : 0.0;
     }
+    for (int r = threadIdx.x; r < mine; r += FT) pos[r] = first + r;
+    if (threadIdx.x == 0) ok_s = 1;
+    __syncthreads();
+    Cand best = no_cand(n);
+    for (int r = threadIdx.x; r < mine; r += FT) best = better(best, make_cand(w[r * P], pos[r], r));
+    best = warp_better(best);
+    if (lane == 0) red[warp] = best;
+    __syncthreads();
+
     for (int k = k0; k < k1; k++) {
-        if (!grid_sync(a.bar, st)) return;
-        // the pivot row, the same in every CTA: warp 0 reads the CTAs'
-        // candidates in parallel and reduces them by shuffles.  No NaN enters
-        // a candidate (a comparison with NaN never prefers it), so "better" is
-        // a total order and the reduction order does not change the result.
-        if (warp == 0) {
-            Cand c = {-1.0, n};
-            for (int b = lane; b < (int)gridDim.x; b += 32)
-                c = better(c, Cand{__ldcg(&a.cand_v[b]), __ldcg(&a.cand_i[b])});
+        const int t = k - k0, par = k & 1;
+        const unsigned seq = (unsigned)k + 1;
+        LuWord *slots = a.slots + (size_t)par * G;
+        LuWord *rows = a.xrows + (size_t)par * (G + 1) * LU_NB;
+        double *prow = prow_s[par];
+        const double *last = prow_s[par ^ 1];    // step k - 1's pivot row
+        Cand mycand = red[0];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1)
-                c = better(c, Cand{__shfl_xor_sync(0xffffffffu, c.v, o), __shfl_xor_sync(0xffffffffu, c.i, o)});
+        for (int i = 1; i < FW; i++) mycand = better(mycand, red[i]);
+        if (mycand.v < 0) mycand.r = -1;         // no row is left out below
+        if (warp == 0) {
+            // ---- publish the candidate, its row finished with step k - 1
+            if (mycand.v >= 0) {
+                double *wr = w + (size_t)mycand.r * P;
+                double x = wr[lane];
+                if (t > 0 && lane > t && lane < nb) {
+                    x = __dsub_rn(x, __dmul_rn(wr[t - 1], last[lane]));
+                    wr[lane] = x;
+                }
+                st_word(&rows[(size_t)cta * LU_NB + lane], __double_as_longlong(x), 0, seq);
+            }
+            if (lane == 0) st_word(&slots[cta], mycand.v, mycand.i, seq);
+            // ---- everybody's candidates; the winner's row
+            Cand c = no_cand(n);
+            bool ok = true;
+            for (int b0 = 0; b0 < G && ok; b0 += 32 * SLOTS) {
+                // a lane's words all requested before the first is looked at
+                Cand o[SLOTS];
+                unsigned got[SLOTS];
+#pragma unroll
+                for (int i = 0; i < SLOTS; i++) {
+                    o[i] = no_cand(n);
+                    got[i] = seq;
+                    const int b = b0 + 32 * i + lane;
+                    if (b < G) got[i] = ld_word(&slots[b], o[i].v, o[i].i);
+                }
+#pragma unroll
+                for (int i = 0; i < SLOTS; i++) {
+                    const int b = b0 + 32 * i + lane;
+                    if (got[i] != seq) ok = wait_word(&slots[b], seq, o[i].v, o[i].i) && ok;
+                    o[i].r = b;
+                    c = better(c, o[i]);
+                }
+            }
+            c = warp_better(c);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok && c.v >= 0) {
+                long long x;
+                int unused;
+                ok = __all_sync(0xffffffffu, wait_word(&rows[(size_t)c.r * LU_NB + lane], seq, x, unused));
+                prow[lane] = __longlong_as_double(x);
+            }
             if (lane == 0) {
-                // no comparable candidate (all NaN): row k stays the pivot, as the
-                // sequential scan that starts from it would leave it
-                v_s = c.i >= k && c.i < n ? c.i : k;
-                if (blockIdx.x == 0) a.ipiv[k] = v_s;
+                v_s = c.v >= 0 ? c.i : -1;
+                if (!ok) {
+                    set_err(st, ERRB_TIMEOUT);
+                    ok_s = 0;
+                }
+            }
+        } else if (t > 0) {
+            // ---- step k - 1 on the columns right of k
+            const int nc = nb - 1 - t;
+            for (int e = threadIdx.x - 32; e < nc * mine; e += FT - 32) {
+                const int r = e / nc, j = t + 1 + e % nc;
+                if (r != mycand.r && pos[r] > k - 1)
+                    w[r * P + j] = __dsub_rn(w[r * P + j], __dmul_rn(w[r * P + t - 1], last[j]));
             }
         }
         __syncthreads();
-        const int v = v_s;
-        if (v != k)   // the panel's columns (the others: lu_laswp_kernel)
-            for (long long j = k0 + (long long)blockIdx.x * blockDim.x + threadIdx.x; j < k1;
-                 j += (long long)gridDim.x * blockDim.x) {
-                const double t = __ldcg(&W[(long long)k * ld + j]);
-                W[(long long)k * ld + j] = __ldcg(&W[(long long)v * ld + j]);
-                W[(long long)v * ld + j] = t;
+        if (!ok_s) return;
+        int v = v_s;
+        if (v < 0) {
+            // no comparable candidate (all NaN): row k stays the pivot, as the sequential
+            // scan that starts from it would leave it; its owner publishes it now
+            v = k;
+            if (warp == 0) {
+                for (int r = 0; r < mine; r++)
+                    if (pos[r] == k)
+                        st_word(&rows[(size_t)G * LU_NB + lane], __double_as_longlong(w[r * P + lane]), 0, seq);
+                long long x;
+                int unused;
+                const bool ok = __all_sync(0xffffffffu, wait_word(&rows[(size_t)G * LU_NB + lane], seq, x, unused));
+                prow[lane] = __longlong_as_double(x);
+                if (lane == 0 && !ok) {
+                    set_err(st, ERRB_TIMEOUT);
+                    ok_s = 0;
+                }
             }
-        if (!grid_sync(a.bar, st)) return;
-        const double piv = __ldcg(&W[(long long)k * ld + k]);
-        if (piv == 0.0) {
-            if (blockIdx.x == 0 && threadIdx.x == 0) st->status = LS_BREAKDOWN;
+            __syncthreads();
+            if (!ok_s) return;
+        }
+        if (cta == 0 && threadIdx.x == 0) a.ipiv[k] = v;
+        const double piv = prow[t];
+        if ((__double_as_longlong(piv) << 1) == 0) {   // a zero pivot, the same in every CTA
+            if (cta == 0 && threadIdx.x == 0) st->status = LS_BREAKDOWN;
             return;
         }
-        // rows i > k of the panel: l, the rank-1 update, next candidates.  The
-        // panel has at most 31 columns right of k: lane c owns column k + 1 + c
-        // (lane 0 the next pivot column); a warp takes LU_ROWS rows at a time
-        // with all their loads issued before any arithmetic.
-        Cand mine = {-1.0, n};
-        const int j = k + 1 + lane;
-        const bool on = j < k1;
-        const double wkj = on ? __ldcg(&W[(long long)k * ld + j]) : 0.0;
-        for (int i0 = k + 1 + gw; i0 < n; i0 += LU_ROWS * nw) {
-            double wik[LU_ROWS], wij[LU_ROWS];
-#pragma unroll
-            for (int u = 0; u < LU_ROWS; u++) {
-                const int i = i0 + u * nw;
-                wik[u] = i < n ? __ldcg(&W[(long long)i * ld + k]) : 0.0;
-                wij[u] = (i < n && on) ? __ldcg(&W[(long long)i * ld + j]) : 0.0;
-            }
-            __syncwarp();   // every lane has read w_ik before lane 0 overwrites it with l
-#pragma unroll
-            for (int u = 0; u < LU_ROWS; u++) {
-                const int i = i0 + u * nw;
-                if (i < n) {
-                    const double l = wik[u] / piv;
-                    const double w = __dsub_rn(wij[u], __dmul_rn(l, wkj));
-                    if (on) W[(long long)i * ld + j] = w;
-                    if (lane == 0) {
-                        W[(long long)i * ld + k] = l;
-                        if (on) mine = better(mine, Cand{fabs(w), i});
-                    }
+        // ---- a thread a row: the swap (the row at position k moves to v, the pivot row to k),
+        // the multiplier, column k + 1, the next candidate
+        best = no_cand(n);
+        for (int r = threadIdx.x; r < mine; r += FT) {
+            int p = pos[r];
+            if (p == k) p = v;
+            else if (p == v) p = k;
+            pos[r] = p;
+            if (p > k) {
+                const double l = w[r * P + t] / piv;
+                w[r * P + t] = l;
+                if (t + 1 < nb) {
+                    const double x = __dsub_rn(w[r * P + t + 1], __dmul_rn(l, prow[t + 1]));
+                    w[r * P + t + 1] = x;
+                    best = better(best, make_cand(x, p, r));
                 }
             }
         }
-        publish_cand(a, mine, red);
+        best = warp_better(best);
+        if (lane == 0) red[warp] = best;
+        __syncthreads();
+    }
+    // every CTA has loaded its rows (it took part in an exchange), so they can be overwritten
+    for (int e = threadIdx.x; e < mine * LU_NB; e += FT) {
+        const int r = e / LU_NB, t = e % LU_NB;
+        if (t < nb) a.W[(long long)pos[r] * ld + k0 + t] = w[r * P + t];
     }
 }
 
@@ -328,15 +442,18 @@ __global__ void __launch_bounds__(LT, 1) lu_backsolve_kernel(LuArgs a) {
 
 LuKernels lu_kernels() {
     LuKernels K{};
-    K.factor = reinterpret_cast<void *>(&lu_factor_kernel);
+    K.factor = reinterpret_cast<void *>(&lu_factor_kernel<true>);
+    K.factor_global = reinterpret_cast<void *>(&lu_factor_kernel<false>);
     K.backsolve = reinterpret_cast<void *>(&lu_backsolve_kernel);
     K.laswp = reinterpret_cast<void *>(&lu_laswp_kernel);
     K.u12 = reinterpret_cast<void *>(&lu_u12_kernel);
     K.trail = reinterpret_cast<void *>(&lu_trail_kernel);
+    set_smem_limit(K.factor, LU_FACTOR_SMEM_MAX);
     K.nb = LU_NB;
     K.tile = RANK_TT;
     K.u12_block = U12_T;
     K.block = LT;
+    K.factor_block = FT;
     return K;
 }
 

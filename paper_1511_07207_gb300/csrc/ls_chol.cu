@@ -1,7 +1,7 @@
 // ls_chol.cu -- the host driver of the Cholesky method (ls_chol_solve,
 // ls_chol_factor): the working matrix [A; b^T] in the workspace, the
-// factorization by panels (per panel: the cooperative panel steps, then the
-// trailing lower triangle), the back substitution, the residual check.
+// factorization by panels (per panel: its columns, then the trailing lower
+// triangle), the back substitution, the residual check.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -65,9 +65,12 @@ int chol_run(ls_ctx *c, int n, const double *A, long long lda, const double *b, 
     e = cudaEventRecord(c->ev0, c->stream);
     for (int k0 = 0; k0 < n && e == cudaSuccess; k0 += K.nb) {
         int kk0 = k0, kk1 = std::min(n, k0 + K.nb), nb = kk1 - kk0;
-        void *pargs[] = {&a, &kk0, &kk1};
-        e = cudaLaunchCooperativeKernel(K.panel, dim3(c->K.coop_grid), dim3(K.block), pargs, 0, c->stream);
         const int rows = n + 1 - kk1, cols = n - kk1;   // trailing rows (b's included) and columns
+        // a CTA an SM, at least 8 and at most 128 rows each beside the diagonal block
+        int prows = std::min(128, std::max(8, (rows + c->num_sms - 1) / c->num_sms));
+        void *pargs[] = {&a, &kk0, &kk1, &prows};
+        e = cudaLaunchKernel(K.panel, dim3((rows + prows - 1) / prows), dim3(K.panel_block), pargs,
+                             (size_t)(K.nb + prows) * (K.nb + 1) * sizeof(double), c->stream);
         if (e == cudaSuccess && rows > 0 && cols > 0) {
             dim3 tg((cols + K.tile - 1) / K.tile, (rows + K.tile - 1) / K.tile);
             void *targs[] = {&a, &kk0, &nb};

@@ -267,23 +267,46 @@ struct BcgKernels {
 BcgKernels bcg_kernels();
 
 // ---- LU with partial pivoting (k_lu.cu) --------------------------------------------------
+struct alignas(16) LuWord {       // one word between the panel's CTAs: a value's bits, an index, step + 1
+    long long v;
+    int i;
+    unsigned seq;
+};
 struct LuArgs {
     int n;
     double *W;                    // [A | b], n x (n + 1), row-major, leading dimension ld
     long long ld;
     int *ipiv;                    // the row swapped with row k at step k
     double *x;                    // the solution
-    double *cand_v;               // [CTA] pivot candidates: |value| and row
-    int *cand_i;
+    LuWord *slots;                // [2][CTA] pivot candidates, by the parity of the step
+    LuWord *xrows;                // [2][CTA + 1][32] the candidates' rows, and the row at position k
+    double *rowbuf;               // the panel's rows when a CTA's do not fit in shared memory
     GridBar *bar;
     State *st;
 };
 struct LuKernels {
-    void *factor, *backsolve;     // factor takes (LuArgs, k0, k1): one panel's steps
+    // factor takes (LuArgs, k0, k1, rows a CTA): one panel's steps, its rows in shared or global memory
+    void *factor, *factor_global, *backsolve;
     void *laswp, *u12, *trail;    // (LuArgs, k0, nb), (LuArgs, k0, nb), (LuArgs, k0)
-    int block, nb, tile, u12_block;
+    int block, factor_block, nb, tile, u12_block;
 };
 LuKernels lu_kernels();
+// Shared memory of the panel kernel with R rows a CTA (in_smem: the rows themselves there too).
+inline size_t lu_factor_smem(int R, bool in_smem) {
+    return ((size_t)(R + 1) / 2 + (in_smem ? (size_t)R * 33 : 0)) * sizeof(double);
+}
+constexpr size_t LU_FACTOR_SMEM_MAX = 200 * 1024;
+// Rows of the panel a CTA takes, of `rows` over at most `grid` CTAs.  A step's exchange
+// costs more with every CTA that takes part, its updates with every row, and they
+// overlap: 64 rows at least (n = 1500: 13.9 ms with all SMs, 10 rows each; 9.8 with
+// 32, 9.4 with 64, 9.9 with 128), then about 48 CTAs (n = 8192: 393 ms; 396 with 152) up to
+// 256 rows, then all SMs.
+inline int lu_rows_per_cta(int rows, int grid) {
+    int R = (rows + 47) / 48;
+    R = R < 64 ? 64 : R > 256 ? 256 : R;
+    const int least = (rows + grid - 1) / grid;
+    return R > least ? R : least;
+}
 
 // ---- Cholesky (k_chol.cu) --------------------------------------------------------------------
 struct CholArgs {
@@ -297,8 +320,9 @@ struct CholArgs {
     State *st;                    // status LS_BREAKDOWN (iter = the failing step) on a pivot <= 0
 };
 struct CholKernels {
-    void *panel, *trail, *backsolve, *zero_upper;   // panel and trail take (CholArgs, k0, k1 / nb)
-    int block, nb, tile;
+    // panel takes (CholArgs, k0, k1, rows a CTA), trail (CholArgs, k0, nb)
+    void *panel, *trail, *backsolve, *zero_upper;
+    int block, nb, tile, panel_block;
 };
 CholKernels chol_kernels();
 size_t chol_workspace_bytes(int n, bool a_on_device);

@@ -17,10 +17,11 @@ namespace {
 
 
 struct LuLayout {
-    double *W, *x, *r, *cand_v, *Astage;
-    int *ipiv, *cand_i;
+    double *W, *x, *r, *rowbuf, *Astage;
+    LuWord *words;
+    int *ipiv;
     long long ld, lda_stage;
-    size_t bytes;
+    size_t nwords, bytes;
 };
 
 LuLayout lu_layout(void *base, int n, int grid, bool stageA) {
@@ -32,8 +33,10 @@ LuLayout lu_layout(void *base, int n, int grid, bool stageA) {
     L.x = cv.take<double>((size_t)std::max(n, 1));
     L.r = cv.take<double>((size_t)std::max(n, 1));
     L.ipiv = cv.take<int>((size_t)std::max(n, 1));
-    L.cand_v = cv.take<double>((size_t)grid);
-    L.cand_i = cv.take<int>((size_t)grid);
+    L.nwords = (size_t)2 * grid + (size_t)2 * (grid + 1) * 32;
+    L.words = cv.take<LuWord>(L.nwords);
+    const int R = lu_rows_per_cta(std::max(n, 1), grid);
+    L.rowbuf = lu_factor_smem(R, true) > LU_FACTOR_SMEM_MAX ? cv.take<double>(((size_t)n + R) * 32) : nullptr;
     L.Astage = stageA ? cv.take<double>((size_t)n * L.lda_stage) : nullptr;   // last (see ls_api.cu)
     L.bytes = align_up(cv.off, 256);
     return L;
@@ -62,16 +65,23 @@ int lu_run(ls_ctx *c, int n, const double *A, long long lda, const double *b, Lu
     a.ld = L.ld;
     a.ipiv = L.ipiv;
     a.x = L.x;
-    a.cand_v = L.cand_v;
-    a.cand_i = L.cand_i;
+    a.slots = L.words;
+    a.xrows = L.words + 2 * c->K.coop_grid;
+    a.rowbuf = L.rowbuf;
     a.bar = c->bar;
     a.st = c->st;
     const LuKernels K = lu_kernels();
-    e = cudaEventRecord(c->ev0, c->stream);
+    // no word of an earlier factorization may pass for one of this
+    e = cudaMemsetAsync(L.words, 0, sizeof(LuWord) * L.nwords, c->stream);
+    if (e == cudaSuccess) e = cudaEventRecord(c->ev0, c->stream);
     for (int k0 = 0; k0 < n && e == cudaSuccess; k0 += K.nb) {
         int kk0 = k0, kk1 = std::min(n, k0 + K.nb), nb = kk1 - kk0;
-        void *fargs[] = {&a, &kk0, &kk1};
-        e = cudaLaunchCooperativeKernel(K.factor, dim3(c->K.coop_grid), dim3(K.block), fargs, 0, c->stream);
+        int R = lu_rows_per_cta(n - kk0, c->K.coop_grid);
+        const int fgrid = (n - kk0 + R - 1) / R;
+        const bool in_smem = lu_factor_smem(R, true) <= LU_FACTOR_SMEM_MAX;
+        void *fargs[] = {&a, &kk0, &kk1, &R};
+        e = cudaLaunchCooperativeKernel(in_smem ? K.factor : K.factor_global, dim3(fgrid), dim3(K.factor_block),
+                                        fargs, lu_factor_smem(R, in_smem), c->stream);
         const int cols_right = n + 1 - kk1, rows_below = n - kk1;
         const int g = std::max(1, std::min((n + 1 + 255) / 256, 4 * c->num_sms));
         void *sargs[] = {&a, &kk0, &nb};
