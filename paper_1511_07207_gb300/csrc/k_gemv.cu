@@ -30,6 +30,7 @@
 
 #include "ls_device.cuh"
 #include "ls_ds.cuh"
+#include "ls_gemv.cuh"
 #include "ls_internal.h"
 #include "split_pair.h"
 
@@ -197,33 +198,6 @@ __device__ __forceinline__ void dot_tile(const typename Cfg<DT>::T *a,
     }
 }
 
-// Butterfly transpose-reduction of RW per-lane row accumulators over the warp:
-// each round a lane keeps half of its rows and adds the partner's copy of
-// them, so RW - 1 + (5 - log2 RW) additions replace RW full reductions.
-// Afterwards lane l holds the warp total of row (l >> (5 - log2 RW)).
-template <int N, int OFF, class V, int RW>
-__device__ __forceinline__ void butterfly(V (&acc)[RW], int lane) {
-    if constexpr (OFF >= 1) {
-        if constexpr (N > 1) {
-            constexpr int H = N / 2;
-            const bool upper = (lane & OFF) != 0;
-#pragma unroll
-            for (int i = 0; i < H; i++) {
-                const V send = upper ? acc[i] : acc[i + H];
-                const V keep = upper ? acc[i + H] : acc[i];
-                acc[i] = keep + shfl_xor_v(send, OFF);
-            }
-            butterfly<H, OFF / 2>(acc, lane);
-        } else {
-            acc[0] += shfl_xor_v(acc[0], OFF);
-            butterfly<1, OFF / 2>(acc, lane);
-        }
-    }
-}
-
-template <int RW>
-__host__ __device__ constexpr int log2i() { return RW <= 1 ? 0 : 1 + log2i<RW / 2>(); }
-
 // plain global loads (fallback when A cannot be described by a TMA map)
 template <int DT>
 __device__ __forceinline__ void dot_global(const typename Cfg<DT>::T *A, const typename Cfg<DT>::T *Alo,
@@ -259,99 +233,11 @@ __device__ __forceinline__ void dot_global(const typename Cfg<DT>::T *A, const t
     }
 }
 
-// ---- epilogue for one finished row ---------------------------------------------------
+// FP8: the row's scale
 template <int DT>
-__device__ __forceinline__ double epilogue(const GemvArgs &a, const MatDesc &M, int row,
-                                           typename Cfg<DT>::Y s) {
-    using V = typename Cfg<DT>::Y;
+__device__ __forceinline__ typename Cfg<DT>::Y scaled(const MatDesc &M, int row, typename Cfg<DT>::Y s) {
     if constexpr (DT == DT_FP8) s *= M.scale[row];
-    V *y = static_cast<V *>(a.y);
-    switch (a.epi) {
-        case EPI_STORE:
-            y[row] = s;
-            return 0.0;
-        case EPI_DOT:
-            y[row] = s;
-            return (double)(static_cast<const V *>(a.z)[row] * s);
-        case EPI_RESID: {
-            V r = (V)(a.b[row] - (double)s);
-            y[row] = r;
-            return (double)r * (double)r;
-        }
-        case EPI_JACOBI: {   // y is the next iterate; x and z are read at this row
-            const double r = a.b[row] - (double)s;
-            y[row] = (V)((double)static_cast<const V *>(a.x)[row] + static_cast<const double *>(a.z)[row] * r);
-            return r * r;
-        }
-        default:  // EPI_NRM
-            y[row] = s;
-            return (double)s * (double)s;
-    }
-}
-
-__device__ __forceinline__ void run_finaliser(const GemvArgs &a, double dot) {
-    State *st = a.st;
-    if (a.dot_out) *a.dot_out = dot;
-    switch (a.fin) {
-        case FIN_CG_ALPHA:
-            st->pq = dot;
-            if (!(dot > 0.0)) {
-                st->status = LS_BREAKDOWN;
-                st->alpha = 0.0;
-            } else {
-                st->alpha = st->rho / dot;
-            }
-            break;
-        case FIN_TRUE_RES:
-            st->true_rnorm = sqrt(dot);
-            break;
-        case FIN_WNORM0:
-            st->wnorm0 = dot;
-            break;
-        case FIN_INNER_ALPHA:
-            st->in_pq = dot;
-            if (!(dot > 0.0)) {
-                st->in_stop = 2;    // breakdown of the inner solve: keep the iterate
-                st->in_alpha = 0.0;
-            } else {
-                st->in_alpha = st->in_rho / dot;
-            }
-            break;
-        case FIN_FCG_D:
-            st->pq = dot;
-            break;
-        case FIN_BS_ALPHA:
-            st->pq = dot;
-            if (dot == 0.0 || !isfinite(dot)) {
-                st->status = LS_BREAKDOWN;
-                st->alpha = 0.0;
-            } else {
-                st->alpha = st->rho / dot;
-            }
-            break;
-        case FIN_JACOBI: {
-            // the residual of the iterate that was just multiplied; the next
-            // iterate is already in y, taken (or not) by the next kernel
-            const double rn = sqrt(dot);
-            st->rnorm = rn;
-            st->true_rnorm = rn;
-            int stop = 1;
-            if (st->status == LS_BREAKDOWN) {
-                // zero diagonal entry: this product only measured x
-            } else {
-                st->iter++;
-                if (!isfinite(dot)) set_err(st, ERRB_NAN);
-                else if (rn <= st->tol_abs) st->status = LS_OK;
-                else if (st->iter >= st->max_iter) st->status = LS_NOT_CONVERGED;
-                else stop = 0;
-            }
-            st->skip = stop;
-            break;
-        }
-        default:
-            st->dot = dot;
-            break;
-    }
+    return s;
 }
 
 // Consumer-warp-only named barrier (ids 1..; 0 is __syncthreads).
@@ -523,7 +409,7 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
 #pragma unroll
                         for (int c = 0; c < WC; c++) s += red[c][tr];
                         const int row = rt * TR + tr;
-                        if (row < rows) mydot += epilogue<DT>(args, M, row, (Y)to_double(s));
+                        if (row < rows) mydot += epilogue<Y>(args, row, scaled<DT>(M, row, (Y)to_double(s)));
                     }
                 } else {
                     // A row tile shared with neighbouring CTAs: publish the
@@ -562,7 +448,7 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
                                 s += __ldcg(&args.scr->fix[((size_t)c * 2 + sl) * TR + tr]);
                             }
                             const int row = rt * TR + tr;
-                            tdot[tr] = row < rows ? epilogue<DT>(args, M, row, (Y)s) : 0.0;
+                            tdot[tr] = row < rows ? epilogue<Y>(args, row, scaled<DT>(M, row, (Y)s)) : 0.0;
                         }
                         consumers_sync();
                         if (threadIdx.x == 0) {

@@ -369,6 +369,7 @@ struct F64Layout {
     float *gpanel;       // Gauss-Seidel: the chain CTA's M_{I,w} = T_I^-1 A_{I,I-w}, one contiguous panel
     long long npad, ldv, lda_stage, ld32;
     int nblk;
+    size_t pair_bytes;   // from Ahi on: the pair, or the packed triangle
     size_t bytes;
 };
 
@@ -391,6 +392,7 @@ F64Layout f64_layout(void *base, int n, int m, bool gmres, bool stageA, bool spl
     L.ld32 = (long long)align_up((size_t)std::max(n, 1), 4);
     L.Ahi = split ? cv.take<float>((size_t)n * L.ld32) : nullptr;
     L.Alo = split ? cv.take<float>((size_t)n * L.ld32) : nullptr;
+    L.pair_bytes = split ? 2 * (size_t)n * L.ld32 * sizeof(float) : 0;
     L.nblk = (std::max(n, 1) + 63) / 64;
     L.Thi = gs ? cv.take<float>((size_t)L.nblk * 64 * 64) : nullptr;
     L.Tlo = gs ? cv.take<float>((size_t)L.nblk * 64 * 64) : nullptr;
@@ -453,7 +455,7 @@ Vecs make_vecs(ls_ctx *c, const F64Layout &L, int n, double rtol) {
 }  // namespace lsi
 
 // Builds: [resid GEMV if x0] cg_init, while(outer){ while(inner){GEMV, update}, resid GEMV, check }
-static int build_cg_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int x0_given,
+static int build_cg_graph(ls_ctx *c, const Vecs &v, const Product &A, int x0_given,
                           const long long *key) {
     Root R;
     if (!R.create()) return LS_ERR_CUDA;
@@ -463,12 +465,11 @@ static int build_cg_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int x0_
         return LS_ERR_CUDA;
     }
     Chain top = R.chain();
-    const MatDesc *dA = c->dA;
     if (x0_given) {
         GemvArgs a{};
         a.x = v.x; a.y = v.r; a.b = v.b; a.st = v.st; a.scr = c->scr;
         a.epi = EPI_RESID; a.fin = FIN_TRUE_RES;
-        gemv_node(top, L, dA, a);
+        product_node(top, A, a);
     }
     {
         Vecs vv = v;
@@ -482,7 +483,7 @@ static int build_cg_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int x0_
         GemvArgs a{};
         a.x = v.p; a.y = v.q; a.z = v.p; a.st = v.st; a.scr = c->scr;
         a.epi = EPI_DOT; a.fin = FIN_CG_ALPHA;
-        gemv_node(inner, L, dA, a);
+        product_node(inner, A, a);
         Vecs vv = v;
         void *args[] = {&vv, &hi};
         inner.kernel(c->K.cg_update, c->K.coop_grid, c->K.block, 0, args, true);
@@ -491,7 +492,7 @@ static int build_cg_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int x0_
         GemvArgs a{};
         a.x = v.x; a.y = v.q; a.b = v.b; a.st = v.st; a.scr = c->scr;
         a.epi = EPI_RESID; a.fin = FIN_TRUE_RES;
-        gemv_node(outer, L, dA, a);
+        product_node(outer, A, a);
         Vecs vv = v;
         void *args[] = {&vv, &ho, &hi};
         outer.kernel(c->K.cg_check, c->K.coop_grid, c->K.block, 0, args, false);
@@ -744,7 +745,25 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
     Vecs v = make_vecs(c, L, n, o.rtol);
     const int dt = split ? DT_DS : DT_F64;
     GemvLaunch GL = gemv_plan(dt, hd->use_tma != 0, EPI_DOT, c->num_sms);
-    long long key[8] = {method, n, (long long)(uintptr_t)c->ws, L.ldv, o.x0_given, hd->use_tma,
+    // CG: the packed triangle takes the place of the pair when A is exactly symmetric
+    Product PR{};
+    PR.gemv = GL;
+    PR.dA = c->dA;
+    const bool want_sym = method == LS_METHOD_CG && split && n >= SYM_MIN_N &&
+                          symv_carve(DT_DS, &PR.mat, L.Ahi, n, c->num_sms) <= L.pair_bytes;
+    if (want_sym) {
+        PR.symv = symv_plan(DT_DS, c->num_sms);
+        PR.mat.bar = c->bar;
+    }
+    cudaError_t e = cudaEventRecord(c->ev0, c->stream);
+    if (e == cudaSuccess && want_sym) e = symv_pack(DT_DS, PR.mat, Ad, ldad, c->st, c->num_sms, c->stream);
+    if (e != cudaSuccess) return map_cuda(e);
+    if (want_sym) {   // one small read: which product, which graph
+        rc = read_state(c);
+        if (rc) return rc;
+        PR.sym = hs->asym == 0;
+    }
+    long long key[8] = {method, n, (long long)(uintptr_t)c->ws, L.ldv, o.x0_given, hd->use_tma + 2 * PR.sym,
                         (long long)(uintptr_t)c->stream, dt};
     GraphCache &gc = method == LS_METHOD_CG         ? c->graph_cg
                      : method == LS_METHOD_BICGSTAB ? c->graph_bs
@@ -752,14 +771,13 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
                      : gs                           ? c->graph_gs
                                                     : c->graph_gm;
     if (!gc.matches(key)) {
-        rc = method == LS_METHOD_CG         ? build_cg_graph(c, v, GL, o.x0_given, key)
+        rc = method == LS_METHOD_CG         ? build_cg_graph(c, v, PR, o.x0_given, key)
              : method == LS_METHOD_BICGSTAB ? build_bicgstab_graph(c, v, GL, o.x0_given, key)
              : method == LS_METHOD_JACOBI   ? build_jacobi_graph(c, v, GL, o.x0_given, key)
              : gs                           ? build_gs_graph(c, v, L, GL, o.x0_given, key)
                                             : build_gmres_graph(c, v, GL, o.x0_given, key);
         if (rc) return rc;
     }
-    cudaError_t e = cudaEventRecord(c->ev0, c->stream);
     if (e == cudaSuccess && method == LS_METHOD_JACOBI) {   // D^-1 into v.p (A may be borrowed per call)
         int nn = n;
         long long la = ldad;
@@ -787,7 +805,8 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
         if (e == cudaSuccess) e = cudaLaunchKernel(G.tinv, dim3(g), dim3(G.tinv_block), args, 0, c->stream);
     }
     // the FP32 pair of A: one pass over A, timed as part of the solve
-    if (e == cudaSuccess && pair) e = split_f64_launch(n, n, Ad, ldad, L.Ahi, L.Alo, L.ld32, c->num_sms, c->stream);
+    if (e == cudaSuccess && pair && !PR.sym)
+        e = split_f64_launch(n, n, Ad, ldad, L.Ahi, L.Alo, L.ld32, c->num_sms, c->stream);
     if (e == cudaSuccess && gs) {   // the chain's panel, from the pair and the T_I^-1
         const GsKernels G = gs_kernels();
         int nn = n;
@@ -831,7 +850,8 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
         sc.rnorm = s.est;   // the Givens estimate of the last step
     }
     c->launches_total += (long long)s.launches;
-    fill_info(info, sc, status, ms, passes * (double)n * n * 8.0, (long long)s.launches);
+    const double pass_bytes = PR.sym ? 4.0 * n * (n + 1.0) : 8.0 * n * (double)n;   // one triangle, or all of A
+    fill_info(info, sc, status, ms, passes * pass_bytes, (long long)s.launches);
     return status;
 }
 

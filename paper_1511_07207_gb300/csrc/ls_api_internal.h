@@ -205,6 +205,27 @@ inline void gemv_node(Chain &ch, const GemvLaunch &L, const MatDesc *dA, const G
     ch.kernel(L.func, L.grid, L.block, L.smem, args, false);
 }
 
+// The smallest n at which CG tries the product from one triangle.
+constexpr int SYM_MIN_N = 1024;
+// The product of a solver loop: the general one, or the symmetric one when A was packed.
+struct Product {
+    GemvLaunch gemv;
+    const MatDesc *dA;
+    bool sym;
+    SymLaunch symv;
+    SymMat mat;
+};
+inline void product_node(Chain &ch, const Product &P, const GemvArgs &a) {
+    if (!P.sym) {
+        gemv_node(ch, P.gemv, P.dA, a);
+        return;
+    }
+    SymMat m = P.mat;
+    GemvArgs aa = a;
+    void *args[] = {(void *)&m, (void *)&aa};
+    ch.kernel(P.symv.func, P.symv.grid, P.symv.block, P.symv.smem, args, true);
+}
+
 int finish_graph(ls_ctx *c, GraphCache &gc, Root &r, const long long *key);
 // Runs a cached solver loop on the context's stream (graph launch or host loop).
 int launch_cached(ls_ctx *c, GraphCache &gc);

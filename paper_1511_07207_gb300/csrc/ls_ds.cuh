@@ -13,7 +13,7 @@
 namespace lsi {
 
 // Double-single accumulator (hi, lo): hi + lo carries about 48 bits.
-struct DSV {
+struct alignas(8) DSV {
     float h, l;
 };
 // (hi, lo) + (hi, lo): the high parts by two-sum (Knuth), every rounding
@@ -34,6 +34,12 @@ __device__ __forceinline__ double shfl_xor_v(double v, int o) { return __shfl_xo
 __device__ __forceinline__ DSV shfl_xor_v(DSV v, int o) {
     return DSV{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)};
 }
+// Loads past L1 (values that other CTAs wrote during the launch).
+__device__ __forceinline__ DSV ldcg_v(const DSV *p) {
+    const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
+    return DSV{v.x, v.y};
+}
+__device__ __forceinline__ float ldcg_v(const float *p) { return __ldcg(p); }
 // acc += a x for a = ah + al, x = xh + xl: ah xh = p + e exactly (FMA gives
 // the product error), the cross terms ah xl + al xh and e go to lo with the
 // two-sum error of hi + p (al xl, below 2^-48 |a x|, is dropped).

@@ -81,6 +81,7 @@ struct State {
     int skip;            // BiCGSTAB: the rest of the step is skipped (s passed, or stop)
     float in_tol2;       // inner (rtol^2 * rho0), <0 = fixed count
     int launches_lo;     // kernels executed (low word; counted by block 0)
+    int asym;            // the packing found a_ij != a_ji
     int hostloop;        // 1: loop conditions go to cond[] instead of graph handles
     unsigned cond[LS_COND_SLOTS];
     unsigned long long launches;
@@ -169,6 +170,27 @@ bool encode_f32_tile_map_sw128(void *map, const float *ptr, int rows, int cols, 
 int gemv_tile_rows(int dtype);
 cudaError_t quantize_launch(int dtype, int rows, int cols, const double *A, long long lda,
                             void *Q, long long ldq, float *scale, int num_sms, cudaStream_t s);
+
+// ---- product with an exactly symmetric A, from its lower triangle (k_symv.cu) ----------
+struct SymMat {
+    int n, blocks;               // size, row blocks of 128
+    const unsigned char *tiles;  // the packed triangle
+    void *pcol, *prow;           // partial sums: of each tile's columns, of each CTA's share of a row block
+    struct GridBar *bar;
+};
+struct SymLaunch {
+    void *func;                  // takes (SymMat, GemvArgs); cooperative
+    int grid, block;
+    size_t smem;
+};
+// dtype: DT_DS, DT_BF16 or DT_F32
+SymLaunch symv_plan(int dtype, int num_sms);
+// Bytes of the packed matrix and its partial sums; places them at base when M is given.
+size_t symv_carve(int dtype, SymMat *M, void *base, int n, int num_sms);
+// Packs the lower triangle of A; DT_DS also sets State::asym unless a_ij and
+// a_ji have the same bits everywhere (the packed matrix is then incomplete).
+cudaError_t symv_pack(int dtype, const SymMat &M, const double *A, long long lda, State *st, int num_sms,
+                      cudaStream_t s);
 
 // ---- FP64 solver vectors (workspace) ---------------------------------------------
 struct GridBar;

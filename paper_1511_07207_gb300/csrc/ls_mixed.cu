@@ -18,6 +18,7 @@ struct MixLayout {
     void *Q;
     long long npad, ldp, ldq, lda_stage, ld32;
     int m;
+    size_t q_bytes, pair_bytes;   // the stored matrix and the pair, or their packed triangles
     size_t bytes;
 };
 
@@ -43,10 +44,12 @@ static MixLayout mix_layout(void *base, int n, int dtype, int m, bool fcg, bool 
     L.pf = cv.take<float>(L.npad);
     L.qf = cv.take<float>(L.npad);
     L.scale = cv.take<float>(L.npad);
-    L.Q = cv.take<unsigned char>((size_t)n * L.ldq * elt_size(dtype));
+    L.q_bytes = (size_t)n * L.ldq * elt_size(dtype);
+    L.Q = cv.take<unsigned char>(L.q_bytes);
     L.ld32 = (long long)align_up((size_t)std::max(n, 1), 4);
     L.Ahi = split ? cv.take<float>((size_t)n * L.ld32) : nullptr;
     L.Alo = split ? cv.take<float>((size_t)n * L.ld32) : nullptr;
+    L.pair_bytes = split ? 2 * (size_t)n * L.ld32 * sizeof(float) : 0;
     // last: no other pointer moves with whether A is staged or borrowed
     L.Astage = stageA ? cv.take<double>((size_t)n * L.lda_stage) : nullptr;
     L.bytes = align_up(cv.off, 256);
@@ -66,8 +69,8 @@ size_t mixed_workspace_bytes(int n, const ls_opts *o, bool a_on_device) {
                       !a_on_device).bytes;
 }
 
-static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const GemvLaunch &L64,
-                             const GemvLaunch &Llo, int x0_given, const long long *key) {
+static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const Product &A64, const Product &Alo, int x0_given,
+                             const long long *key) {
     const MixedKernels K = mixed_kernels();
     const int G = c->K.coop_grid, B = c->K.block;
     Root R;
@@ -80,14 +83,13 @@ static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const GemvLaunch &L64,
         return LS_ERR_CUDA;
     }
     if (v.mode != LS_REFINE_FCG) hs = ho;
-    const MatDesc *d64 = c->dA, *dlo = c->dA + 1;
     MixVecs vv = v;
     Chain top = R.chain();
     if (x0_given) {
         GemvArgs a{};
         a.x = v.x; a.y = v.r; a.b = v.b; a.st = v.st; a.scr = c->scr;
         a.epi = EPI_RESID; a.fin = FIN_TRUE_RES;
-        gemv_node(top, L64, d64, a);
+        product_node(top, A64, a);
     }
     {
         int x0 = x0_given;
@@ -99,7 +101,7 @@ static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const GemvLaunch &L64,
         GemvArgs a{};
         a.x = v.pf; a.y = v.qf; a.z = v.pf; a.st = v.st; a.scr = c->scr;
         a.epi = EPI_DOT; a.fin = FIN_INNER_ALPHA;
-        gemv_node(in, Llo, dlo, a);
+        product_node(in, Alo, a);
         void *args[] = {&vv, &hi};
         in.kernel(K.in_update, G, B, 0, args, true);
         return in.err;
@@ -121,7 +123,7 @@ static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const GemvLaunch &L64,
             a.x = v.P; a.y = v.W; a.kptr = &v.st->nstored; a.kstride = v.ldp; a.kyoff = 0;
             a.z_is_x = 1; a.st = v.st; a.scr = c->scr;
             a.epi = EPI_DOT; a.fin = FIN_FCG_D;
-            gemv_node(out, L64, d64, a);
+            product_node(out, A64, a);
             void *args2[] = {&vv, &ho};
             out.kernel(K.fcg_update, G, B, 0, args2, true);
         }
@@ -129,7 +131,7 @@ static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const GemvLaunch &L64,
             GemvArgs a{};
             a.x = v.x; a.y = v.q; a.b = v.b; a.st = v.st; a.scr = c->scr;
             a.epi = EPI_RESID; a.fin = FIN_TRUE_RES;
-            gemv_node(sup, L64, d64, a);
+            product_node(sup, A64, a);
             void *args[] = {&vv, &hs, &ho};
             sup.kernel(K.mx_check, G, B, 0, args, false);
         }
@@ -140,7 +142,7 @@ static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const GemvLaunch &L64,
             GemvArgs a{};
             a.x = v.x; a.y = v.r; a.b = v.b; a.st = v.st; a.scr = c->scr;
             a.epi = EPI_RESID; a.fin = FIN_TRUE_RES;
-            gemv_node(out, L64, d64, a);
+            product_node(out, A64, a);
             void *args[] = {&vv, &ho, &hi};
             out.kernel(K.ir_start, G, B, 0, args, true);
         }
@@ -193,11 +195,35 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     if (!rc && o.x0_given) rc = copy_in(c, L.x, x, n);
     if (rc) return rc;
 
+    // both products from one triangle when A is exactly symmetric (FP8's row scales
+    // make the stored matrix nonsymmetric)
+    Product P64{}, Plo{};
+    const bool want_sym = split && dtype != DT_FP8 && n >= SYM_MIN_N &&
+                          symv_carve(DT_DS, &P64.mat, L.Ahi, n, c->num_sms) <= L.pair_bytes &&
+                          symv_carve(dtype, &Plo.mat, L.Q, n, c->num_sms) <= L.q_bytes;
     cudaError_t e = cudaEventRecord(c->ev0, c->stream);
-    if (e == cudaSuccess)   // stage A: quantise once per solve
+    if (e != cudaSuccess) return map_cuda(e);
+    State *hs = c->h_st;
+    if (want_sym) {
+        state_init(hs, 0);
+        rc = upload_state(c);
+        if (!rc) rc = map_cuda(symv_pack(DT_DS, P64.mat, Ad, ldad, c->st, c->num_sms, c->stream));
+        if (!rc) rc = read_state(c);
+        if (rc) return rc;
+        P64.sym = Plo.sym = hs->asym == 0;
+    }
+    const bool sym = P64.sym;
+    if (sym) {
+        P64.symv = symv_plan(DT_DS, c->num_sms);
+        Plo.symv = symv_plan(dtype, c->num_sms);
+        P64.mat.bar = Plo.mat.bar = c->bar;
+        e = symv_pack(dtype, Plo.mat, Ad, ldad, c->st, c->num_sms, c->stream);
+    } else {
+        // stage A: quantise once per solve
         e = quantize_launch(dtype, n, n, Ad, ldad, L.Q, L.ldq, L.scale, c->num_sms, c->stream);
-    if (e == cudaSuccess && split)   // and the FP32 pair for the outer FP64 products
-        e = split_f64_launch(n, n, Ad, ldad, L.Ahi, L.Alo, L.ld32, c->num_sms, c->stream);
+        if (e == cudaSuccess && split)   // and the FP32 pair for the outer FP64 products
+            e = split_f64_launch(n, n, Ad, ldad, L.Ahi, L.Alo, L.ld32, c->num_sms, c->stream);
+    }
     if (e != cudaSuccess) return map_cuda(e);
 
     MatDesc *h64 = &c->h_desc[0], *hlo = &c->h_desc[1];
@@ -209,13 +235,12 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     hlo->scale = dtype == DT_FP8 ? L.scale : nullptr;
     rc = upload_desc(c, 0);
     if (!rc) rc = upload_desc(c, 1);
-    State *hs = c->h_st;
     state_init(hs, 0);
     hs->max_outer = max_outer;
     hs->m = m;
     hs->in_max = o.inner_iters;
     hs->in_tol2 = o.inner_rtol > 0.0 ? (float)(o.inner_rtol * o.inner_rtol) : -1.0f;
-    hs->launches = split ? 2 : 1;   // the quantisation (and split) kernels
+    hs->launches = split ? 2 : 1;   // the quantisation (and split or packing) kernels
     if (!rc) rc = upload_state(c);
     if (rc) return rc;
 
@@ -226,12 +251,14 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     v.dvals = L.dvals;
     v.rf = L.rf; v.zf = L.zf; v.pf = L.pf; v.qf = L.qf;
     v.part = c->part; v.bar = c->bar; v.st = c->st; v.rtol = o.rtol;
-    GemvLaunch L64 = gemv_plan(split ? DT_DS : DT_F64, h64->use_tma != 0, EPI_DOT, c->num_sms);
-    GemvLaunch Llo = gemv_plan(dtype, hlo->use_tma != 0, EPI_DOT, c->num_sms);
+    P64.gemv = gemv_plan(split ? DT_DS : DT_F64, h64->use_tma != 0, EPI_DOT, c->num_sms);
+    Plo.gemv = gemv_plan(dtype, hlo->use_tma != 0, EPI_DOT, c->num_sms);
+    P64.dA = c->dA;
+    Plo.dA = c->dA + 1;
     long long key[8] = {100 + o.refine, n, (long long)(uintptr_t)c->ws, dtype * 2 + (split ? 1 : 0), o.x0_given,
-                        h64->use_tma * 2 + hlo->use_tma, (long long)(uintptr_t)c->stream, m};
+                        h64->use_tma * 2 + hlo->use_tma + 4 * sym, (long long)(uintptr_t)c->stream, m};
     if (!c->graph_mx.matches(key)) {
-        rc = build_mixed_graph(c, v, L64, Llo, o.x0_given, key);
+        rc = build_mixed_graph(c, v, P64, Plo, o.x0_given, key);
         if (rc) return rc;
     }
     rc = launch_cached(c, c->graph_mx);
@@ -254,7 +281,8 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     const double nn = (double)n * n;
     const int esz = elt_size(dtype);
     const double f64_passes = (fcg ? s.outer + s.cycles : s.outer + 1) + (o.x0_given ? 1 : 0);
-    const double bytes = nn * (8.0 + esz) + f64_passes * 8.0 * nn + (double)s.iter * esz * nn;
+    const double share = sym ? 0.5 * (n + 1.0) / n : 1.0;   // one triangle, or all of A
+    const double bytes = nn * (8.0 + share * esz) + share * (f64_passes * 8.0 * nn + (double)s.iter * esz * nn);
     State sc = s;
     sc.cycles = s.outer;
     c->launches_total += (long long)s.launches;
