@@ -181,6 +181,8 @@ int upload_desc(ls_ctx *c, int which) {
 int read_state(ls_ctx *c) {
     cudaError_t e = cudaMemcpyAsync(c->h_st, c->st, sizeof(State), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    // a barrier that timed out leaves its arrivals behind
+    if (e == cudaSuccess && (c->h_st->err & ERRB_TIMEOUT)) e = cudaMemsetAsync(c->bar, 0, sizeof(GridBar), c->stream);
     return map_cuda(e);
 }
 

@@ -123,7 +123,9 @@ __device__ __forceinline__ T warp_sum(T v) {
 }
 
 // Sum over the block; every thread gets the result.  `red` needs
-// blockDim.x / 32 entries.  Fixed order, so deterministic.
+// blockDim.x / 32 entries.  Fixed order, so deterministic.  The warps' sums are added by
+// warp 0 alone: an FP64 addition takes 64 cycles of a scheduler's FP64 unit for every
+// warp that makes it, so each thread adding them all kept it busy for 0.5 us.
 template <class T>
 __device__ __forceinline__ T block_sum(T v, T *red) {
     v = warp_sum(v);
@@ -131,9 +133,17 @@ __device__ __forceinline__ T block_sum(T v, T *red) {
     __syncthreads();
     if (l == 0) red[w] = v;
     __syncthreads();
-    T s = 0;
-    for (int i = 0; i < nw; i++) s += red[i];
-    return s;
+    if (w == 0) {
+        T s = l < nw ? red[l] : T(0);
+        if (nw > 8) s += __shfl_xor_sync(0xffffffffu, s, 16);
+        if (nw > 8) s += __shfl_xor_sync(0xffffffffu, s, 8);
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        if (l == 0) red[0] = s;
+    }
+    __syncthreads();
+    return red[0];
 }
 
 // ---- launch counting -----------------------------------------------------------------
@@ -145,8 +155,7 @@ __device__ __forceinline__ void set_err(State *st, int bits) { atomicOr(&st->err
 
 // ---- bounded grid barrier (cooperative launches only) ---------------------------------
 struct GridBar {
-    unsigned count;
-    unsigned gen;
+    unsigned count;      // arrivals; cleared by the host after a barrier that timed out
 };
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned *p) {
@@ -167,30 +176,28 @@ __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
 }
 
 // All blocks of the grid meet here.  Returns false (and sets ERRB_TIMEOUT)
-// if the others did not arrive within WAIT_LIMIT_NS.
+// if the others did not arrive within WAIT_LIMIT_NS.  The arrivals of one barrier
+// add up to 2^31 whatever the grid's size, so the word's top bit flips with the last
+// of them and the waiting blocks see it in one L2 round trip (a second word, written by
+// the last block, made it two).
 __device__ __forceinline__ bool grid_sync(GridBar *b, State *st) {
     __shared__ int ok_s;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        unsigned g = ld_acquire_u32(&b->gen);
         __threadfence();
-        unsigned arrived = atomicAdd(&b->count, 1u);
-        if (arrived == gridDim.x - 1) {
-            atomicExch(&b->count, 0u);
-            __threadfence();
-            st_release_u32(&b->gen, g + 1);
-        } else {
-            unsigned long long t0 = gtimer();
-            unsigned ns = 32;
-            while (ld_acquire_u32(&b->gen) == g) {
-                __nanosleep(ns);
-                if (ns < 256) ns <<= 1;
-                if (gtimer() - t0 > WAIT_LIMIT_NS) {
-                    set_err(st, ERRB_TIMEOUT);
-                    ok = 0;
-                    break;
-                }
+        const unsigned mine = blockIdx.x == 0 ? (1u << 31) - (gridDim.x - 1) : 1u;
+        const unsigned before = atomicAdd(&b->count, mine);
+        unsigned polls = 0;
+        unsigned long long t0 = 0;
+        while (((ld_acquire_u32(&b->count) ^ before) >> 31) == 0) {
+            if (++polls < 64) continue;
+            if (t0 == 0) t0 = gtimer();
+            __nanosleep(64);
+            if (gtimer() - t0 > WAIT_LIMIT_NS) {
+                set_err(st, ERRB_TIMEOUT);
+                ok = 0;
+                break;
             }
         }
         ok_s = ok;
