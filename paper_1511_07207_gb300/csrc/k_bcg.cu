@@ -375,232 +375,273 @@ __global__ void __launch_bounds__(BK) bcg_check_kernel(BcgVecs v, cudaGraphCondi
 // the taken ones is at most 1e-8 of its norm: dependent), then P = W T with
 // T = D^-1 Pi L^-T, and a second pass (Gram of P, Cholesky, P = P L2^-T).
 // Small matrices use leading dimension BCG_MAX_S; the s x s algebra (at most
-// 16 x 16) runs on one thread.
+// 16 x 16) runs in every CTA, spread over a warp or 16 lanes a column.
 // ============================================================================
 constexpr int SL = BCG_MAX_S;              // leading dimension of the small matrices
 constexpr double BCGD_TAU2 = 1e-16;        // (1e-8)^2 on the normalized diagonal
 
+// Entry e of an nu x nv Gram matrix; sym: of its lower triangle (a >= b).
+__device__ __forceinline__ int gram_entries(int nu, int nv, bool sym) { return sym ? nu * (nu + 1) / 2 : nu * nv; }
+__device__ __forceinline__ void gram_entry(int e, int nu, bool sym, int &a, int &b) {
+    if (!sym) {
+        a = e % nu;
+        b = e / nu;
+        return;
+    }
+    a = 0;
+    while ((a + 1) * (a + 2) / 2 <= e) a++;
+    b = e - a * (a + 1) / 2;
+}
+
 // This CTA's partial U[:, :nu]^T V[:, :nv] over rows [lo, hi) into
-// buf[cta][SL*SL].  Every thread of the CTA takes part: T = BK / (nu nv)
-// threads per entry, thread q of an entry summing rows lo + q, lo + q + T,
-// ...; the T sums added in q order (a fixed order, so the result does not
-// depend on timing).  A warp's FP64 instruction takes about 64 cycles of
-// its scheduler's FP64 unit on this GPU, so shorter chains spread over all
-// warps (and all four schedulers) are what counts.
+// buf[cta][e].  Every thread of the CTA takes part: T = BK / E threads per
+// entry, thread q of an entry summing rows lo + q, lo + q + T, ...; the T sums
+// added in q order (a fixed order, so the result does not depend on timing).  A
+// warp's FP64 instruction takes about 64 cycles of its scheduler's FP64 unit on
+// this GPU, so short chains spread over all four schedulers are what counts.
 __device__ __forceinline__ void gram_partial_ld(const BcgVecs &v, double *buf, const double *U, int nu,
-                                                const double *V, int nv, long long lo, long long hi) {
+                                                const double *V, int nv, bool sym, long long lo, long long hi) {
     __shared__ double red[BK];
-    const int E = nu * nv;
+    const int E = gram_entries(nu, nv, sym);
     if (E == 0) return;
     const int T = BK / E;
     const int e = threadIdx.x / T, q = threadIdx.x - e * T;
     double acc = 0.0;
     if (e < E) {
-        const int a = e % nu, b = e / nu;
+        int a, b;
+        gram_entry(e, nu, sym, a, b);
         const double *u = U + (long long)a * v.ld, *w = V + (long long)b * v.ld;
+#pragma unroll 4
         for (long long i = lo + q; i < hi; i += T) acc += u[i] * w[i];
     }
     red[threadIdx.x] = acc;
     __syncthreads();
     if (e < E && q == 0) {
-        double sum = 0.0;
-        for (int t = 0; t < T; t++) sum += red[threadIdx.x + t];
-        const int a = e % nu, b = e / nu;
-        buf[(size_t)blockIdx.x * SL * SL + a + b * SL] = sum;
+        double sum = red[threadIdx.x];
+        for (int t = 1; t < T; t++) sum += red[threadIdx.x + t];
+        buf[(size_t)blockIdx.x * SL * SL + e] = sum;
     }
     __syncthreads();
 }
-// G = the sum of the CTAs' partials, entry by entry, by all threads of the
-// calling CTA: eight interleaved sums over the CTAs (CTA c into sum c % 8),
-// added pairwise; a fixed order.
-__device__ __forceinline__ void gram_reduce_ld(const double *buf, int nu, int nv, double *G) {
-    const int nc = (int)gridDim.x;
-    for (int e = threadIdx.x; e < nu * nv; e += blockDim.x) {
-        const int a = e % nu, b = e / nu;
-        const double *p = buf + a + b * SL;
-        double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        int c = 0;
-        for (; c + 8 <= nc; c += 8)
-#pragma unroll
-            for (int u = 0; u < 8; u++) t[u] += __ldcg(p + (size_t)(c + u) * SL * SL);
-        for (int u = 0; c + u < nc; u++) t[u] += __ldcg(p + (size_t)(c + u) * SL * SL);
-        G[a + b * SL] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+// G = the sum of the CTAs' partials, by threads t0 .. BK - 1 of the calling CTA (t0 a
+// multiple of 32; a barrier of those threads inside): T threads an entry, thread q of
+// them adding CTAs q, q + T, ..., then the T sums in q order.  The order depends on
+// nothing but the sizes, so every CTA that does this gets the same bits.
+// A lower triangle is mirrored.
+__device__ __forceinline__ void gram_reduce_ld(const double *buf, int nu, int nv, bool sym, double *G, int t0) {
+    __shared__ double red[BK];
+    const int E = gram_entries(nu, nv, sym), nt = BK - t0, nc = (int)gridDim.x;
+    if (E == 0) return;
+    const int T = max(1, nt / E), t = (int)threadIdx.x - t0;
+    for (int e0 = 0; e0 < E; e0 += nt) {              // more than one round only for 16 x 16 and t0 > 0
+        const int e = e0 + t % (T > 1 ? E : nt), q = T > 1 ? t / E : 0;
+        double acc = 0.0;
+        if (e < E && q < T) {
+#pragma unroll 8
+            for (int c = q; c < nc; c += T) acc += __ldcg(&buf[(size_t)c * SL * SL + e]);
+        }
+        red[threadIdx.x] = acc;
+        named_bar(2, nt);
+        if (e < E && q == 0) {
+            for (int i = 1; i < T; i++) acc += red[threadIdx.x + i * E];
+            int a, b;
+            gram_entry(e, nu, sym, a, b);
+            G[a + b * SL] = acc;
+            if (sym) G[b + a * SL] = acc;
+        }
+        named_bar(2, nt);
     }
 }
 
-// Cholesky of the leading r x r block (lower triangle, leading dimension SL);
-// false on a pivot that is not positive.
-__device__ bool small_chol(int r, double *G) {
-    for (int j = 0; j < r; j++) {
-        double d = G[j + j * SL];
-        for (int k = 0; k < j; k++) d -= G[j + k * SL] * G[j + k * SL];
-        if (!(d > 0.0)) return false;
-        d = sqrt(d);
-        G[j + j * SL] = d;
-        const double dinv = 1.0 / d;   // one division per column (FP64 division is slow here)
-        for (int i = j + 1; i < r; i++) {
-            double x = G[i + j * SL];
-            for (int k = 0; k < j; k++) x -= G[i + k * SL] * G[j + k * SL];
-            G[i + j * SL] = x * dinv;
+__device__ __forceinline__ bool positive(double x) {   // x > 0 and not NaN, off the FP64 pipe
+    const long long b = __double_as_longlong(x);
+    return b > 0 && b <= 0x7FF0000000000000ll;
+}
+
+// One warp: Cholesky of the leading r x r block (lower triangle, leading
+// dimension SL), right-looking, and the reciprocals of its diagonal; false on a pivot
+// that is not positive.  One reciprocal square root a column: a square root
+// and a division are 0.3 us each on the chain.
+__device__ bool warp_chol_ld(int r, double *G, double *dinv) {
+    const int lane = threadIdx.x & 31;
+    for (int k = 0; k < r; k++) {
+        const double d = G[k + k * SL];
+        if (!positive(d)) return false;                // the same in every lane
+        const double rs = rsqrt(d);
+        __syncwarp();
+        if (lane >= k && lane < r) G[lane + k * SL] = (lane == k ? d : G[lane + k * SL]) * rs;
+        if (lane == 0) dinv[k] = rs;
+        __syncwarp();
+        const int m = r - 1 - k;
+        for (int e = lane; e < m * m; e += 32) {
+            const int i = k + 1 + e % m, j = k + 1 + e / m;
+            if (i >= j) G[i + j * SL] -= G[i + k * SL] * G[j + k * SL];
         }
+        __syncwarp();
     }
     return true;
 }
-// Y (r x c) = (L L^T)^-1 Y, column j of Y by thread j of the calling CTA
-// (all threads call it), with the reciprocals of L's diagonal formed once.
-__device__ void small_chol_solve(int r, int c, const double *L, double *Y) {
-    __shared__ double dinv[SL];
-    if (threadIdx.x < r) dinv[threadIdx.x] = 1.0 / L[threadIdx.x + threadIdx.x * SL];
-    __syncthreads();
-    for (int j = threadIdx.x; j < c; j += blockDim.x) {
-        double *y = Y + j * SL;
-        for (int i = 0; i < r; i++) {
-            double x = y[i];
-            for (int k = 0; k < i; k++) x -= L[i + k * SL] * y[k];
-            y[i] = x * dinv[i];
-        }
-        for (int i = r - 1; i >= 0; i--) {
-            double x = y[i];
-            for (int k = i + 1; k < r; k++) x -= L[k + i * SL] * y[k];
-            y[i] = x * dinv[i];
-        }
-    }
-    __syncthreads();
-}
-// M = L^-T (upper triangular, r x r) for a lower-triangular L.
-__device__ void small_inv_t(int r, const double *L, double *M) {
-    for (int b = 0; b < SL; b++)
-        for (int a = 0; a < SL; a++) M[a + b * SL] = 0.0;
-    double dinv[SL];
-    for (int a = 0; a < r; a++) dinv[a] = 1.0 / L[a + a * SL];
-    for (int b = 0; b < r; b++) {                  // column b of M solves L^T m = e_b
-        for (int a = r - 1; a >= 0; a--) {
-            double x = a == b ? 1.0 : 0.0;
-            for (int k = a + 1; k < r; k++) x -= L[k + a * SL] * M[k + b * SL];
-            M[a + b * SL] = x * dinv[a];
-        }
-    }
-}
 
-// First pass of orth: from G = W^T W (s x s) the rank r and T (s x s) with
-// W T = the r orthonormal-to-first-order columns (then zero columns).
-// work: 3 SL^2 + 2 SL doubles, iwork: 2 SL ints (shared memory of the caller).
-__device__ int rr_factor(int s, const double *G, double *T, double *work, int *iwork) {
-    double *Lp = work, *M = work + SL * SL, *Lcm = work + 2 * SL * SL;
-    double *d = work + 3 * SL * SL, *rem = d + SL;
-    int *perm = iwork, *state = iwork + SL;
-#define Lc(q, t) Lcm[(q) + (t) * SL]
-    double dinv[SL];
-    for (int j = 0; j < s; j++) {
-        d[j] = sqrt(G[j + j * SL]);
-        dinv[j] = 1.0 / d[j];
-        state[j] = d[j] > 0.0 ? 0 : 2;             // 0 open, 1 taken, 2 dropped
-        rem[j] = 1.0;
+// All threads, thread (k, c) = (tid % 16, tid / 16) holding entry (k, c) of an
+// r x 16 block: y = L^-1 y, and with `both` L^-T (L^-1 y).  The 16 lanes of a column
+// hand each other the finished entries by shuffles.
+__device__ __forceinline__ double team_solve(int r, const double *L, const double *dinv, double y, bool both) {
+    const int k = threadIdx.x & 15, base = threadIdx.x & 16;
+    for (int i = 0; i < r; i++) {
+        const double yi = __shfl_sync(0xffffffffu, y, base | i) * dinv[i];
+        if (k == i) y = yi;
+        else if (k > i && k < r) y -= L[k + i * SL] * yi;
     }
+    if (both)
+        for (int i = r - 1; i >= 0; i--) {
+            const double yi = __shfl_sync(0xffffffffu, y, base | i) * dinv[i];
+            if (k == i) y = yi;
+            else if (k < i) y -= L[i + k * SL] * yi;
+        }
+    return y;
+}
+// Y (r x c, c <= 16) = (L L^T)^-1 Y.  Warps without a column of Y sit out.
+__device__ __forceinline__ void team_chol_solve(int r, int c, const double *L, const double *dinv, double *Y) {
+    const int k = threadIdx.x & 15, col = threadIdx.x >> 4;
+    if ((int)(threadIdx.x >> 5) * 2 < c) {
+        double y = k < r && col < c ? Y[k + col * SL] : 0.0;
+        y = team_solve(r, L, dinv, y, true);
+        if (k < r && col < c) Y[k + col * SL] = y;
+    }
+    __syncthreads();
+}
+// T = scale L^-T in rows perm (scale and perm may be null): T[perm[a] + b SL] = (L^-1)_ba scale[perm[a]].
+__device__ __forceinline__ void team_inv_t(int r, const double *L, const double *dinv, const int *perm,
+                                           const double *scale, double *T) {
+    const int k = threadIdx.x & 15, col = threadIdx.x >> 4;
+    T[threadIdx.x] = 0.0;                              // SL * SL = BK entries
+    __syncthreads();
+    if ((int)(threadIdx.x >> 5) * 2 < r) {
+        const double y = team_solve(r, L, dinv, k == col ? 1.0 : 0.0, false);
+        if (col < r && k >= col && k < r) {
+            const int row = perm ? perm[col] : col;
+            T[row + k * SL] = scale ? y * scale[row] : y;
+        }
+    }
+    __syncthreads();
+}
+static_assert(SL * SL == BK, "a thread an entry of the small matrices");
+
+// First pass of orth, one warp (lane q: column q): from G = W^T W (s x s) the rank r,
+// the order of the kept columns, the Cholesky factor Lp of their normalized Gram matrix
+// with the reciprocals of its diagonal, and the reciprocal column norms.
+// Lc: s x SL scratch.
+__device__ int rr_factor(int s, const double *G, double *Lc, double *Lp, double *dinv, double *scale, int *perm) {
+    const int q = threadIdx.x & 31;
+    const double gq = q < s ? G[q + q * SL] : 0.0;
+    const double sq = positive(gq) ? rsqrt(gq) : 0.0;
+    if (q < s) scale[q] = sq;
+    __syncwarp();
+    bool open = positive(gq);                          // not taken, not dropped
+    double rem = 1.0;
     int r = 0;
     for (;;) {
-        int p = -1;
-        for (int j = 0; j < s; j++) {
-            if (state[j]) continue;
-            if (!(rem[j] > BCGD_TAU2)) { state[j] = 2; continue; }
-            if (p < 0 || rem[j] > rem[p]) p = j;
+        open = open && rem > BCGD_TAU2;
+        // the open column with the most left, the first one on ties (bits order as positive values do)
+        const long long bits = open ? __double_as_longlong(rem) : -1ll;
+        long long best = bits;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = max(best, __shfl_xor_sync(0xffffffffu, best, o));
+        if (best < 0) break;
+        const int p = __ffs(__ballot_sync(0xffffffffu, bits == best)) - 1;
+        const double rp = __longlong_as_double(best), linv = rsqrt(rp);
+        const double np = scale[p];
+        double l = 0.0;
+        if (q == p) {
+            l = rp * linv;                             // sqrt(rem)
+            perm[r] = p;
+            dinv[r] = linv;
+            open = false;
+        } else if (open) {
+            double x = G[q + p * SL] * sq * np;
+            for (int t = 0; t < r; t++) x -= Lc[q + t * SL] * Lc[p + t * SL];
+            l = x * linv;
+            rem -= l * l;
         }
-        if (p < 0) break;
-        const double lpp = sqrt(rem[p]), linv = 1.0 / lpp;
-        perm[r] = p;
-        state[p] = 1;
-        Lc(p, r) = lpp;
-        for (int q = 0; q < s; q++) {
-            if (state[q]) continue;
-            double x = G[q + p * SL] * dinv[q] * dinv[p];
-            for (int t = 0; t < r; t++) x -= Lc(q, t) * Lc(p, t);
-            Lc(q, r) = x * linv;
-            rem[q] -= Lc(q, r) * Lc(q, r);
-        }
+        if (q < s) Lc[q + r * SL] = l;
+        __syncwarp();
         r++;
     }
-    for (int b = 0; b < SL; b++)
-        for (int a = 0; a < SL; a++) Lp[a + b * SL] = 0.0;
-    for (int a = 0; a < r; a++)
-        for (int t = 0; t <= a; t++) Lp[a + t * SL] = Lc(perm[a], t);
-    small_inv_t(r, Lp, M);
-    for (int e = 0; e < SL * SL; e++) T[e] = 0.0;
-    for (int a = 0; a < r; a++)
-        for (int b = 0; b < r; b++) T[perm[a] + b * SL] = M[a + b * SL] * dinv[perm[a]];
-#undef Lc
+    __syncwarp();
+    for (int e = q; e < r * r; e += 32) {
+        const int i = e % r, t = e / r;
+        Lp[i + t * SL] = t <= i ? Lc[perm[i] + t * SL] : 0.0;
+    }
+    __syncwarp();
     return r;
 }
 
+// out[i, b] = (add ? add[i, b] : 0) + sum_{c < nc} in[i, c] T[c, b] for this CTA's rows and b < nb, a thread an
+// element.  out may be `in`: a round of elements is formed before any of it is stored,
+// and a round holds whole rows.
+__device__ __forceinline__ void rows_times(const BcgVecs &v, double *out, const double *add, const double *in, int nc,
+                                           const double *T, int nb, long long lo, long long hi) {
+    if (nb == 0) return;
+    const int per = BK / nb;                           // rows a round
+    const int r = threadIdx.x % per, b = threadIdx.x / per;
+    for (long long i0 = lo; i0 < hi; i0 += per) {
+        const long long i = i0 + r;
+        const bool on = b < nb && i < hi;
+        double acc = 0.0;
+        if (on) {
+#pragma unroll 4
+            for (int c = 0; c < nc; c++) acc += in[(long long)c * v.ld + i] * T[c + b * SL];
+            if (add) acc += add[(long long)b * v.ld + i];
+        }
+        if (out == in) __syncthreads();
+        if (on) out[(long long)b * v.ld + i] = acc;
+    }
+    __syncthreads();
+}
+
 // P = orth(W) over the whole grid (cooperative launch; W and P must differ).
-// On return sm->rank holds r and sm->w2 the squared column norms of W.
-// false if a grid barrier gave up or the second pass failed.
-__device__ bool coop_orth(const BcgVecs &v, const double *W, long long lo, long long hi) {
-    __shared__ double G[SL * SL], T[SL * SL], work[3 * SL * SL + 2 * SL];
-    __shared__ int r_s, iwork[2 * SL];
+// Every CTA reduces the partial Gram matrices and factors them for itself
+// (the same operations, the same bits), so a pass has one barrier of the grid.  On
+// return `rank` holds r in every CTA, and sm->rank and sm->w2 (the squared column
+// norms of W) are set.  false if a grid barrier gave up or the second pass failed.
+__device__ bool coop_orth(const BcgVecs &v, const double *W, long long lo, long long hi, int &rank) {
+    __shared__ double G[SL * SL], T[SL * SL], Lc[SL * SL], dinv[SL], scale[SL];
+    __shared__ int r_s, perm[SL];
     BcgSmall *sm = v.sm;
     const int s = v.s;
-    gram_partial_ld(v, v.part, W, s, W, s, lo, hi);
+    gram_partial_ld(v, v.part, W, s, W, s, true, lo, hi);
     if (!grid_sync(v.bar, v.st)) return false;
-    if (blockIdx.x == 0) {
-        gram_reduce_ld(v.part, s, s, G);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int j = 0; j < s; j++) sm->w2[j] = G[j + j * SL];
-            bool nan = false;
-            for (int j = 0; j < s; j++) nan = nan || !isfinite(G[j + j * SL]);
-            const int r = nan ? 0 : rr_factor(s, G, T, work, iwork);
-            for (int e = 0; e < SL * SL; e++) sm->T[e] = T[e];
-            sm->rank = r;
-        }
-    }
-    if (!grid_sync(v.bar, v.st)) return false;
-    if (threadIdx.x == 0) r_s = *(volatile int *)&sm->rank;
-    for (int e = threadIdx.x; e < SL * SL; e += blockDim.x) T[e] = __ldcg(&sm->T[e]);
-    __syncthreads();
-    const int r = r_s;
-    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {     // P = W T
-        double w[BCG_MAX_S];
-#pragma unroll
-        for (int c = 0; c < BCG_MAX_S; c++) w[c] = c < s ? W[(long long)c * v.ld + i] : 0.0;
-        for (int b = 0; b < s; b++) {
-            double acc = 0.0;
-#pragma unroll
-            for (int c = 0; c < BCG_MAX_S; c++)
-                if (c < s) acc += w[c] * T[c + b * SL];
-            v.P[(long long)b * v.ld + i] = acc;
+    gram_reduce_ld(v.part, s, s, true, G, 0);
+    if (threadIdx.x < 32) {
+        bool nan = false;
+        for (int j = 0; j < s; j++) nan = nan || !isfinite(G[j + j * SL]);
+        const int r = nan ? 0 : rr_factor(s, G, Lc, T, dinv, scale, perm);
+        if (threadIdx.x == 0) r_s = r;
+        if (blockIdx.x == 0) {
+            if ((int)threadIdx.x < s) sm->w2[threadIdx.x] = G[threadIdx.x * (SL + 1)];
+            if (threadIdx.x == 0) sm->rank = r;
         }
     }
     __syncthreads();
-    gram_partial_ld(v, v.part, v.P, r, v.P, r, lo, hi);                 // second pass
-    if (!grid_sync(v.bar, v.st)) return false;
-    if (blockIdx.x == 0) {
-        gram_reduce_ld(v.part, r, r, G);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            const bool ok = small_chol(r, G);
-            if (ok) small_inv_t(r, G, T);
-            for (int e = 0; e < SL * SL; e++) sm->T[e] = ok ? T[e] : 0.0;
-            if (!ok) sm->rank = -1;
-        }
-    }
-    if (!grid_sync(v.bar, v.st)) return false;
-    for (int e = threadIdx.x; e < SL * SL; e += blockDim.x) T[e] = __ldcg(&sm->T[e]);
-    if (threadIdx.x == 0) r_s = *(volatile int *)&sm->rank;
+    const int r = rank = r_s;
+    G[threadIdx.x] = T[threadIdx.x];                   // the factor, so that T can take L^-T
     __syncthreads();
-    if (r_s < 0) return false;
-    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {     // P = P L2^-T (upper triangular)
-        double p[BCG_MAX_S];
-#pragma unroll
-        for (int c = 0; c < BCG_MAX_S; c++) p[c] = c < r ? v.P[(long long)c * v.ld + i] : 0.0;
-        for (int b = 0; b < r; b++) {
-            double acc = 0.0;
-#pragma unroll
-            for (int c = 0; c < BCG_MAX_S; c++)
-                if (c <= b) acc += p[c] * T[c + b * SL];
-            v.P[(long long)b * v.ld + i] = acc;
-        }
+    team_inv_t(r, G, dinv, perm, scale, T);
+    rows_times(v, v.P, nullptr, W, s, T, s, lo, hi);   // P = W T, zero past column r
+    gram_partial_ld(v, v.partb, v.P, r, v.P, r, true, lo, hi);   // second pass
+    if (!grid_sync(v.bar, v.st)) return false;
+    gram_reduce_ld(v.partb, r, r, true, G, 0);
+    if (threadIdx.x < 32) {
+        const bool ok = warp_chol_ld(r, G, dinv);
+        if (threadIdx.x == 0) r_s = ok;
     }
     __syncthreads();
+    if (!r_s) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) sm->rank = -1;
+        return false;
+    }
+    team_inv_t(r, G, dinv, nullptr, nullptr, T);
+    rows_times(v, v.P, nullptr, v.P, r, T, r, lo, hi);  // P = P L2^-T
     return true;
 }
 
@@ -641,7 +682,8 @@ __global__ void __launch_bounds__(BK) bcgd_init_kernel(BcgVecs v, int x0_given, 
         for (int c = 0; c < (int)gridDim.x; c++) t[c & 7] += __ldcg(&v.part2[(size_t)c * BCG_MAX_S + threadIdx.x]);
         sm->bn[threadIdx.x] = sqrt(((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7])));
     }
-    const bool ok = coop_orth(v, v.R, lo, hi);          // its first barrier publishes bn too
+    int rank = 0;
+    const bool ok = coop_orth(v, v.R, lo, hi, rank);    // its first barrier publishes bn too
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         bool nan = false;
         for (int j = 0; j < v.s; j++) nan = nan || !isfinite(sm->w2[j]) || !isfinite(sm->bn[j]);
@@ -653,7 +695,7 @@ __global__ void __launch_bounds__(BK) bcgd_init_kernel(BcgVecs v, int x0_given, 
         } else if (nan) {
             set_err(st, ERRB_NAN);
             go = 0;
-        } else if (pass || sm->rank == 0) {
+        } else if (pass || rank == 0) {
             go = 0;                                     // confirm on the true residual
         } else if (st->max_iter <= 0) {
             go = 0;
@@ -663,10 +705,14 @@ __global__ void __launch_bounds__(BK) bcgd_init_kernel(BcgVecs v, int x0_given, 
     }
 }
 
-// One step after Q = A P.
+// One step after Q = A P.  Four grid barriers: behind each, every CTA reduces the partial
+// sums and does the s x s algebra for itself, so nothing waits for one
+// CTA's answer.  What bounds it is latency: FP64 chains of the small matrices and
+// the barriers.  (One CTA doing the algebra, one thread of it the factorizations,
+// with eight barriers: 294 us a step at n = 8192, s = 8.)
 __global__ void __launch_bounds__(BK) bcgd_step_kernel(BcgVecs v, cudaGraphConditionalHandle h_inner) {
-    __shared__ double G[SL * SL], H[SL * SL], coef[SL * SL];
-    __shared__ int flag_s, r_s;
+    __shared__ double G[SL * SL], H[SL * SL], dinv[SL], r2[BCG_MAX_S];
+    __shared__ int flag_s;
     State *st = v.st;
     BcgSmall *sm = v.sm;
     count_launch(st);
@@ -675,133 +721,94 @@ __global__ void __launch_bounds__(BK) bcgd_step_kernel(BcgVecs v, cudaGraphCondi
         if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(st, h_inner, 0u);
         return;
     }
-    if (threadIdx.x == 0) r_s = *(volatile int *)&sm->rank;
-    __syncthreads();
-    const int r = r_s;
+    const int r = __ldcg(&sm->rank), iter = __ldcg(&st->iter), max_iter = st->max_iter;
     long long lo, hi;
     block_range(v.n, blockIdx.x, gridDim.x, lo, hi);
     // gamma = P^T Q and P^T R
-    gram_partial_ld(v, v.part, v.P, r, v.Q, r, lo, hi);
-    gram_partial_ld(v, v.partb, v.P, r, v.R, s, lo, hi);
+    gram_partial_ld(v, v.part, v.P, r, v.Q, r, true, lo, hi);
+    gram_partial_ld(v, v.partb, v.P, r, v.R, s, false, lo, hi);
     if (!grid_sync(v.bar, st)) return;
-    if (blockIdx.x == 0) {
-        gram_reduce_ld(v.part, r, r, G);
-        gram_reduce_ld(v.partb, r, s, H);
-        __syncthreads();
-        if (threadIdx.x == 0) flag_s = small_chol(r, G) ? 1 : 0;   // positive definite for SPD A
-        __syncthreads();
-        if (flag_s) small_chol_solve(r, s, G, H);       // alpha = gamma^-1 P^T R (all threads)
-        if (threadIdx.x == 0) {
-            for (int e = 0; e < SL * SL; e++) {
-                sm->Lg[e] = G[e];
-                sm->alpha[e] = H[e];
-            }
-            sm->ok = flag_s;
-            if (!flag_s) st->status = LS_BREAKDOWN;
-        }
+    gram_reduce_ld(v.part, r, r, true, G, 0);
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        const bool ok = warp_chol_ld(r, G, dinv);      // positive definite for SPD A
+        if (threadIdx.x == 0) flag_s = ok;
+    } else {
+        gram_reduce_ld(v.partb, r, s, false, H, 32);
     }
-    if (!grid_sync(v.bar, st)) return;
-    if (threadIdx.x == 0) flag_s = *(volatile int *)&sm->ok;
-    for (int e = threadIdx.x; e < SL * SL; e += blockDim.x) coef[e] = __ldcg(&sm->alpha[e]);
     __syncthreads();
     if (!flag_s) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(st, h_inner, 0u);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            st->status = LS_BREAKDOWN;
+            sm->ok = 0;
+            set_cond(st, h_inner, 0u);
+        }
         return;
     }
-    // X += P alpha, R -= Q alpha (row by row), then Q^T R and ||R_j||^2
-    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        double p[BCG_MAX_S], q[BCG_MAX_S];
-#pragma unroll
-        for (int c = 0; c < BCG_MAX_S; c++) {
-            p[c] = c < r ? v.P[(long long)c * v.ld + i] : 0.0;
-            q[c] = c < r ? v.Q[(long long)c * v.ld + i] : 0.0;
-        }
-        for (int j = 0; j < s; j++) {
-            double dx = 0.0, dr = 0.0;
-#pragma unroll
-            for (int c = 0; c < BCG_MAX_S; c++)
-                if (c < r) {
-                    dx += p[c] * coef[c + j * SL];
-                    dr += q[c] * coef[c + j * SL];
-                }
-            v.X[(long long)j * v.ld + i] += dx;
-            v.R[(long long)j * v.ld + i] -= dr;
-        }
-    }
+    team_chol_solve(r, s, G, dinv, H);                 // alpha = gamma^-1 P^T R
+    // X += P alpha, R -= Q alpha, then Q^T R and ||R_j||^2
+    rows_times(v, v.X, v.X, v.P, r, H, s, lo, hi);
+    H[threadIdx.x] = -H[threadIdx.x];
     __syncthreads();
-    gram_partial_ld(v, v.part, v.Q, r, v.R, s, lo, hi);
-    for (int j = threadIdx.x; j < s; j += blockDim.x) {
-        const double *rr = v.R + (long long)j * v.ld;
+    rows_times(v, v.R, v.R, v.Q, r, H, s, lo, hi);
+    gram_partial_ld(v, v.partc, v.Q, r, v.R, s, false, lo, hi);   // others may still read part and partb
+    {   // ||R_j||^2 over this CTA's rows: 16 lanes a column
+        const int j = threadIdx.x >> 4, q = threadIdx.x & 15;
         double acc = 0.0;
-        for (long long i = lo; i < hi; i++) acc += rr[i] * rr[i];
-        v.part2[(size_t)blockIdx.x * BCG_MAX_S + j] = acc;
+        if (j < s)
+            for (long long i = lo + q; i < hi; i += 16) {
+                const double x = v.R[(long long)j * v.ld + i];
+                acc += x * x;
+            }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (j < s && q == 0) v.part2[(size_t)blockIdx.x * BCG_MAX_S + j] = acc;
     }
     if (!grid_sync(v.bar, st)) return;
-    if (blockIdx.x == 0) {
-        __shared__ double r2[BCG_MAX_S];
-        __shared__ int nan_s, go_s;
-        // ||R_j||^2: thread j, eight interleaved sums over the CTAs
-        if (threadIdx.x < s) {
-            double t[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            const int nc = (int)gridDim.x;
-            for (int c = 0; c < nc; c++) t[c & 7] += __ldcg(&v.part2[(size_t)c * BCG_MAX_S + threadIdx.x]);
-            r2[threadIdx.x] = ((t[0] + t[1]) + (t[2] + t[3])) + ((t[4] + t[5]) + (t[6] + t[7]));
+    gram_reduce_ld(v.partc, r, s, false, H, 0);
+    {   // ||R_j||^2 over the CTAs
+        const int j = threadIdx.x >> 4, q = threadIdx.x & 15;
+        double acc = 0.0;
+        if (j < s) {
+#pragma unroll 4
+            for (int c = q; c < (int)gridDim.x; c += 16) acc += __ldcg(&v.part2[(size_t)c * BCG_MAX_S + j]);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            bool nan = false;
-            for (int j = 0; j < s; j++) nan = nan || !isfinite(r2[j]);
-            nan_s = nan;
-            go_s = !nan && !cols_pass(v, r2);
-        }
-        __syncthreads();
-        if (go_s) {
-            gram_reduce_ld(v.part, r, s, H);
-            for (int e = threadIdx.x; e < SL * SL; e += blockDim.x) G[e] = sm->Lg[e];
-            __syncthreads();
-            small_chol_solve(r, s, G, H);              // beta = -gamma^-1 Q^T R (all threads)
-        }
-        if (threadIdx.x == 0) {
-            int go = go_s;
-            if (go)
-                for (int e = 0; e < SL * SL; e++) sm->beta[e] = -H[e];
-            st->iter++;
-            if (nan_s) set_err(st, ERRB_NAN);
-            sm->update_p = go;
-            if (go && st->iter >= st->max_iter) go = 0;
-            sm->ok = go;
-        }
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (j < s && q == 0) r2[j] = acc;
     }
-    if (!grid_sync(v.bar, st)) return;
-    if (threadIdx.x == 0) flag_s = *(volatile int *)&sm->update_p;
-    for (int e = threadIdx.x; e < SL * SL; e += blockDim.x) coef[e] = __ldcg(&sm->beta[e]);
     __syncthreads();
-    if (!flag_s) {
+    // the stop test, the same in every CTA: lane j tests column j
+    if (threadIdx.x < 32) {
+        const double x = (int)threadIdx.x < s ? r2[threadIdx.x] : 0.0;
+        const bool nan = __any_sync(0xffffffffu, !isfinite(x));
+        const bool pass = __all_sync(0xffffffffu, (int)threadIdx.x >= s || sqrt(x) <= v.rtol * __ldcg(&sm->bn[threadIdx.x & 15]));
+        if (threadIdx.x == 0) flag_s = nan ? -1 : pass ? 0 : 1;
+    }
+    __syncthreads();
+    const int flag = flag_s;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        st->iter = iter + 1;
+        if (flag < 0) set_err(st, ERRB_NAN);
+    }
+    if (flag <= 0) {
         if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(st, h_inner, 0u);
         return;
     }
-    // W = R + P beta into Q's storage, then P = orth(W)
-    for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        double p[BCG_MAX_S];
-#pragma unroll
-        for (int c = 0; c < BCG_MAX_S; c++) p[c] = c < r ? v.P[(long long)c * v.ld + i] : 0.0;
-        for (int j = 0; j < s; j++) {
-            double acc = v.R[(long long)j * v.ld + i];
-#pragma unroll
-            for (int c = 0; c < BCG_MAX_S; c++)
-                if (c < r) acc += p[c] * coef[c + j * SL];
-            v.Q[(long long)j * v.ld + i] = acc;
-        }
-    }
+    team_chol_solve(r, s, G, dinv, H);                 // beta = -gamma^-1 Q^T R
+    H[threadIdx.x] = -H[threadIdx.x];
     __syncthreads();
-    const bool ok = coop_orth(v, v.Q, lo, hi);
+    // W = R + P beta into Q's storage, then P = orth(W)
+    rows_times(v, v.Q, v.R, v.P, r, H, s, lo, hi);
+    int rank = 0;
+    const bool ok = coop_orth(v, v.Q, lo, hi, rank);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        int go = *(volatile int *)&sm->ok;
+        int go = iter + 1 < max_iter;
         if (!ok) {
             go = 0;
             if (!*(volatile int *)&st->err) st->status = LS_BREAKDOWN;
-        } else if (sm->rank == 0) {
-            go = 0;                                     // nothing left to search: confirm
+        } else if (rank == 0) {
+            go = 0;                                    // nothing left to search: confirm
         }
         set_cond(st, h_inner, go ? 1u : 0u);
     }
@@ -846,13 +853,14 @@ __global__ void __launch_bounds__(BK) bcgd_check_kernel(BcgVecs v, cudaGraphCond
     }
     long long lo, hi;
     block_range(v.n, blockIdx.x, gridDim.x, lo, hi);
-    const bool ok = coop_orth(v, v.R, lo, hi);
+    int rank = 0;
+    const bool ok = coop_orth(v, v.R, lo, hi, rank);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         int go = 1;
         if (!ok) {
             go = 0;
             if (!*(volatile int *)&st->err) st->status = LS_BREAKDOWN;
-        } else if (sm->rank == 0) {
+        } else if (rank == 0) {
             go = 0;
             st->status = LS_BREAKDOWN;                  // not converged and nothing left to search
         }

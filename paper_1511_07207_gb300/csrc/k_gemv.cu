@@ -47,8 +47,7 @@ struct Cfg<DT_F64> {
     using Y = double;
     static constexpr int VEC = 2, WC = 4, WR = 1, RW = 8, PARTS = 1;
 };
-// 16 rows per warp: each lane's split x values (FP64-pipe conversions) serve
-// twice as many products as with 8
+// 16 rows per warp: each lane's split x values serve twice as many products as with 8
 template <>
 struct Cfg<DT_DS> {
     using T = float;    // hi and lo tiles of the same shape, one after the other
@@ -125,10 +124,7 @@ __device__ __forceinline__ void load_x(const typename Cfg<DT>::X *x, int c0, int
             for (int k = 0; k < VEC; k++) v[k] = (c0 + k < cols) ? x[c0 + k] : 0.0;
         }
 #pragma unroll
-        for (int k = 0; k < VEC; k++) {
-            const float h = __double2float_rn(v[k]);
-            p[k] = DSV{h, __double2float_rn(v[k] - (double)h)};
-        }
+        for (int k = 0; k < VEC; k++) split_pair(v[k], p[k].h, p[k].l);   // off the FP64 pipe
     } else if (c0 + VEC <= cols && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
         if constexpr (DT == DT_F64) {
             double2 v = __ldg(reinterpret_cast<const double2 *>(x + c0));

@@ -17,7 +17,7 @@ using namespace lsi;
 namespace {
 
 struct BcgLayout {
-    double *X, *R, *P, *Q, *B, *part, *partb, *part2, *Astage;
+    double *X, *R, *P, *Q, *B, *part, *partb, *partc, *part2, *Astage;
     BcgSmall *sm;
     float *Ahi, *Alo;
     float *Ph, *Pl;      // P split for the block product (pair path)
@@ -38,6 +38,7 @@ BcgLayout bcg_layout(void *base, int n, int s, int grid, bool stageA, bool split
     L.B = cv.take<double>((size_t)L.ld * s);
     L.part = cv.take<double>((size_t)grid * BCG_MAX_S * BCG_MAX_S);
     L.partb = cv.take<double>((size_t)grid * BCG_MAX_S * BCG_MAX_S);
+    L.partc = cv.take<double>((size_t)grid * BCG_MAX_S * BCG_MAX_S);
     L.part2 = cv.take<double>((size_t)grid * BCG_MAX_S);
     L.sm = cv.take<BcgSmall>(1);
     L.Ahi = split ? cv.take<float>((size_t)n * L.ld32) : nullptr;
@@ -206,6 +207,7 @@ extern "C" int ls_block_cg_solve(ls_ctx *c, int n, int s, const double *A, int64
     v.B = L.B;
     v.part = L.part;
     v.partb = L.partb;
+    v.partc = L.partc;
     v.part2 = L.part2;
     v.sm = L.sm;
     v.bar = c->bar;

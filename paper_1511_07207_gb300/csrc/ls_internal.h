@@ -274,7 +274,8 @@ struct BcgVecs {
     double *X, *R, *P, *Q;
     const double *B;
     double *part;                 // [CTA][BCG_MAX_S^2] partial Gram matrices
-    double *partb;                // [CTA][BCG_MAX_S^2] a second set (two Gram matrices at once)
+    double *partb, *partc;        // [CTA][BCG_MAX_S^2] more sets (a set is written again only after a
+                                  // grid barrier that follows its last read)
     double *part2;                // [CTA][BCG_MAX_S] partial ||B_j||^2
     BcgSmall *sm;
     GridBar *bar;
