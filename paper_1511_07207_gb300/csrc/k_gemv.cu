@@ -109,42 +109,36 @@ int gemv_tile_rows(int dtype) {
 }
 
 // ---- x chunk loads --------------------------------------------------------------
+// The lane's VEC entries of x from column c0 on, zero past the end.
 template <int DT>
 __device__ __forceinline__ void load_x(const typename Cfg<DT>::X *x, int c0, int cols,
-                                       typename Cfg<DT>::V (&p)[Cfg<DT>::VEC]) {
-    constexpr int VEC = Cfg<DT>::VEC;
-    if constexpr (DT == DT_DS) {        // FP64 x split into (hi, lo) floats
-        double v[VEC];
-        if (c0 + VEC <= cols && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
-            const double2 w = __ldg(reinterpret_cast<const double2 *>(x + c0));
-            v[0] = w.x;
-            v[1] = w.y;
-        } else {
+                                       typename Cfg<DT>::X (&v)[Cfg<DT>::VEC]) {
+    using X = typename Cfg<DT>::X;
+    constexpr int VEC = Cfg<DT>::VEC, W = 16 / sizeof(X);
+    if (c0 + VEC <= cols && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
 #pragma unroll
-            for (int k = 0; k < VEC; k++) v[k] = (c0 + k < cols) ? x[c0 + k] : 0.0;
-        }
-#pragma unroll
-        for (int k = 0; k < VEC; k++) split_pair(v[k], p[k].h, p[k].l);   // off the FP64 pipe
-    } else if (c0 + VEC <= cols && ((reinterpret_cast<uintptr_t>(x) & 15) == 0)) {
-        if constexpr (DT == DT_F64) {
-            double2 v = __ldg(reinterpret_cast<const double2 *>(x + c0));
-            p[0] = v.x;
-            p[1] = v.y;
-        } else {
-#pragma unroll
-            for (int k = 0; k < VEC; k += 4) {
-                float4 v = __ldg(reinterpret_cast<const float4 *>(x + c0 + k));
-                p[k] = v.x;
-                p[k + 1] = v.y;
-                p[k + 2] = v.z;
-                p[k + 3] = v.w;
+        for (int k = 0; k < VEC; k += W) {
+            if constexpr (sizeof(X) == 8) {
+                const double2 w = __ldg(reinterpret_cast<const double2 *>(x + c0 + k));
+                v[k] = w.x;
+                v[k + 1] = w.y;
+            } else {
+                const float4 w = __ldg(reinterpret_cast<const float4 *>(x + c0 + k));
+                v[k] = w.x;
+                v[k + 1] = w.y;
+                v[k + 2] = w.z;
+                v[k + 3] = w.w;
             }
         }
     } else {
 #pragma unroll
-        for (int k = 0; k < VEC; k++) p[k] = (c0 + k < cols) ? x[c0 + k] : 0;
+        for (int k = 0; k < VEC; k++) v[k] = (c0 + k < cols) ? x[c0 + k] : X(0);
     }
 }
+// ... as the operand of the products (the FP32 pair: off the FP64 pipe).
+__device__ __forceinline__ void to_operand(double x, DSV &p) { split_pair(x, p.h, p.l); }
+__device__ __forceinline__ void to_operand(double x, double &p) { p = x; }
+__device__ __forceinline__ void to_operand(float x, float &p) { p = x; }
 
 // acc0 + acc1 += a[0:VEC] . p[0:VEC] (two independent FMA chains); `a` points
 // at VEC consecutive stored elements in shared memory, aligned to the vector.
@@ -285,7 +279,12 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
     const int RT = (rows + TR - 1) / TR, CT = (cols + TC - 1) / TC;
     const long long T_all = (long long)RT * CT;
     const int G_ = gridDim.x, cta = blockIdx.x;
-    const long long t0 = tile_start(T_all, cta, G_), t1 = tile_start(T_all, cta + 1, G_);
+    // Equal pieces, except when there are at most as many row tiles as CTAs (up to n =
+    // 4864 for the FP32 pair): then a CTA takes one whole row tile, and none of them waits to
+    // add partial sums with its neighbours (2 us each time; n = 2000: half of the kernel's time).
+    const bool whole = RT <= G_;
+    const long long t0 = whole ? (long long)min(cta, RT) * CT : tile_start(T_all, cta, G_);
+    const long long t1 = whole ? (long long)min(cta + 1, RT) * CT : tile_start(T_all, cta + 1, G_);
     const int ntiles = (int)(t1 - t0);
     count_launch(args.st);
 
@@ -357,9 +356,17 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
         int rt = ntiles > 0 ? (int)(t0 / CT) : 0, ct = ntiles > 0 ? (int)(t0 % CT) : 0;
         const int first_rt = rt;
 
+        // With one CTA on most SMs (whole row tiles) x of a tile is asked for while the tile before
+        // it is worked on (Jacobi, n = 2500: 0.53 -> 0.47 ms); with two the other
+        // CTA hides that latency, and asking early costs 3 % at n = 16384.
+        X xv[VEC];
+        if (whole && ntiles > 0) load_x<DT>(x, lane_col, cols, xv);
         for (int i = 0; i < ntiles; i++) {
             V p[VEC];
-            load_x<DT>(x, ct * TC + lane_col, cols, p);
+            if (!whole) load_x<DT>(x, ct * TC + lane_col, cols, xv);
+#pragma unroll
+            for (int k = 0; k < VEC; k++) to_operand(xv[k], p[k]);
+            if (whole && i + 1 < ntiles) load_x<DT>(x, (ct + 1) * TC + lane_col, cols, xv);
             if (TMA) {
                 // On a timeout the warp stops waiting and computing but keeps
                 // walking the tile sequence, so it still meets the other

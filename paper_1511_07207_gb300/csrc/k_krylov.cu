@@ -30,7 +30,7 @@
 //                asked), h_{k+1,k} = ||w||, v_{k+1} = w / h_{k+1,k}; then one
 //                thread applies the old rotations to column k, forms the new
 //                one, updates g and tests |g_{k+1}| <= rtol ||b||;
-//     gm_finish  back-solve R y = g (one warp), x += V_k y.
+//     gm_finish  back-solve R y = g (one warp of every block), x += V_k y.
 //   Jacobi (paper, introduction: the classical stationary methods, taken from
 //   the textbooks): x(k+1) = x(k) + D^-1 (b - A x(k)).  The step itself is the
 //   GEMV's epilogue (next iterate into a second vector, ||b - A x(k)||^2
@@ -237,8 +237,11 @@ __global__ void __launch_bounds__(KB) gm_init_kernel(Vecs v, int x0_given,
     block_range(v.n, blockIdx.x, gridDim.x, lo, hi);
     double bb = 0.0;
     for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
-        if (!x0_given) v.x[i] = 0.0;
         const double bi = v.b[i];
+        if (!x0_given) {           // the first cycle's residual is b itself
+            v.x[i] = 0.0;
+            v.q[i] = bi;
+        }
         bb += bi * bi;
     }
     bb = block_sum(bb, red);
@@ -258,6 +261,7 @@ __global__ void __launch_bounds__(KB) gm_init_kernel(Vecs v, int x0_given,
             const double bn = sqrt(b2);
             st->bnorm = bn;
             st->tol_abs = v.rtol * bn;
+            if (!x0_given) st->true_rnorm = bn;
             int go = 1;
             if (!isfinite(b2)) {
                 set_err(st, ERRB_NAN);
@@ -272,7 +276,8 @@ __global__ void __launch_bounds__(KB) gm_init_kernel(Vecs v, int x0_given,
     }
 }
 
-// A cycle starts: the residual GEMV has written q = b - A x, true_rnorm = ||q||.
+// A cycle starts (or the solve ends): q = b - A x and true_rnorm = ||q|| are in place,
+// from gm_init when x = 0, else from the residual GEMV.
 __global__ void __launch_bounds__(KB) gm_start_kernel(Vecs v, cudaGraphConditionalHandle h_outer,
                                                       cudaGraphConditionalHandle h_inner) {
     State *st = v.st;
@@ -293,8 +298,6 @@ __global__ void __launch_bounds__(KB) gm_start_kernel(Vecs v, cudaGraphCondition
         if (go == -1) set_err(st, ERRB_NAN);
         if (go == 0) st->status = LS_OK;
         if (go == -2) st->status = LS_NOT_CONVERGED;
-        // no new cycle: the gm_finish node that follows in this body must not
-        // apply the previous cycle's correction a second time
         if (go != 1) st->k = 0;
         if (go == 1) {
             GmresSmall *gm = v.gm;
@@ -308,104 +311,211 @@ __global__ void __launch_bounds__(KB) gm_start_kernel(Vecs v, cudaGraphCondition
     }
 }
 
+// ---- FP64 scalars with short chains: a dependent FP64 instruction takes about 115
+// cycles here, a square root about twenty of them and a division ten ----------------
+struct RootInv {
+    double r, inv;   // sqrt(x), 1 / sqrt(x)
+};
+// One reciprocal square root, the root corrected by its remainder.
+__device__ __forceinline__ RootInv root_inv(double x) {
+    const double inv = rsqrt(x), r = x * inv;
+    if (!(x > 0.0) || !isfinite(r)) return RootInv{sqrt(x), 1.0 / sqrt(x)};
+    return RootInv{fma(0.5 * inv, fma(-r, r, x), r), inv};
+}
+// a / b with inv close to 1 / b: the quotient corrected by its remainder.
+__device__ __forceinline__ double quot(double a, double b, double inv) {
+    const double q = a * inv;
+    return fma(inv, fma(-b, q, a), q);
+}
+
+// Sums over a warp of U values at once: their shuffles and additions interleave.
+template <int U>
+__device__ __forceinline__ void warp_sums(double (&s)[U]) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < U; u++) s[u] += __shfl_xor_sync(0xffffffffu, s[u], o);
+}
+
 // One Arnoldi step after the GEMV has written w = A v_k into column k+1 and
-// ||w||^2 into wnorm0.
+// ||w||^2 into wnorm0.  What bounds it is latency: grid barriers (two, three with the
+// second pass) and chains of dependent FP64 instructions between them.  So a warp
+// takes several columns of V at once, square roots and quotients come from one
+// reciprocal square root each, and whether a second pass is needed is read from ||w||^2 -
+// ||h||^2 (V is orthonormal) instead of a norm that every block waits for.  At n = 2000,
+// k = 8, two passes: 46 k cycles before.
 __global__ void __launch_bounds__(KB) gm_arnoldi_kernel(Vecs v, cudaGraphConditionalHandle h_inner) {
     __shared__ double red[KB / 32];
     __shared__ double h[LS_MAX_RESTART + 1];
-    __shared__ double hsum[LS_MAX_RESTART + 1];
-    __shared__ double wn_s;
+    __shared__ double hsum[LS_MAX_RESTART + 1], hrot[LS_MAX_RESTART + 1];
+    __shared__ double cs[LS_MAX_RESTART], sn[LS_MAX_RESTART];
+    __shared__ double wn2_s, wn_s, winv_s, w0_s;
+    __shared__ int again_s;
+    constexpr int U = 4, NW = KB / 32;
     State *st = v.st;
     count_launch(st);
     const int k = st->k;                  // 0-based: w is column k+1, basis columns 0..k
     const double wnorm0 = st->wnorm0;
     const int always2 = st->reorth;
     const int G = gridDim.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     long long lo, hi;
     block_range(v.n, blockIdx.x, G, lo, hi);
     double *w = v.V + (long long)(k + 1) * v.ldv;
     for (int j = threadIdx.x; j <= k; j += blockDim.x) hsum[j] = 0.0;
+    if (blockIdx.x == 0)
+        for (int j = threadIdx.x; j < k; j += blockDim.x) {
+            cs[j] = v.gm->cs[j];
+            sn[j] = v.gm->sn[j];
+        }
     __syncthreads();
 
-    double wn2 = 0.0;
-    for (int pass = 0; pass < 2; pass++) {
-        // h_j = v_j . w over this block's rows (warp per column), one slot per j
-        for (int j = warp; j <= k; j += nw) {
-            const double *vj = v.V + (long long)j * v.ldv;
-            double s = 0.0;
-            for (long long i = lo + lane; i < hi; i += 32) s += vj[i] * w[i];
-            s = warp_sum(s);
-            if (lane == 0) v.part[(size_t)j * G + blockIdx.x] = s;
+    bool ok = true;
+    for (int pass = 0; pass < 2 && ok; pass++) {
+        // h_j = v_j . w over this block's rows (U columns a warp at a time), one slot per j
+        for (int j0 = warp; j0 <= k; j0 += U * NW) {
+            double s[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) s[u] = 0.0;
+            for (long long i = lo + lane; i < hi; i += 32) {
+                const double wi = w[i];
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    if (j0 + u * NW <= k) s[u] += v.V[(long long)(j0 + u * NW) * v.ldv + i] * wi;
+            }
+            warp_sums(s);
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (lane == 0 && j0 + u * NW <= k) v.part[(size_t)(j0 + u * NW) * G + blockIdx.x] = s[u];
         }
-        if (!grid_sync(v.bar, st)) break;
-        for (int j = warp; j <= k; j += nw) {
-            const double t = reduce_slot(v.part, j, G);
-            if (lane == 0) h[j] = t;
+        ok = grid_sync(v.bar, st);
+        if (!ok) break;
+        for (int j0 = warp; j0 <= k; j0 += U * NW) {
+            double s[U];
+#pragma unroll
+            for (int u = 0; u < U; u++) s[u] = 0.0;
+            for (int b = lane; b < G; b += 32)
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    if (j0 + u * NW <= k) s[u] += __ldcg(&v.part[(size_t)(j0 + u * NW) * G + b]);
+            warp_sums(s);
+#pragma unroll
+            for (int u = 0; u < U; u++)
+                if (lane == 0 && j0 + u * NW <= k) {
+                    h[j0 + u * NW] = s[u];
+                    hsum[j0 + u * NW] += s[u];
+                }
         }
         __syncthreads();
+        // a second pass only when cancellation lost accuracy (or always if asked)
+        if (warp == NW - 1 && pass == 0) {
+            double q[1] = {0.0};
+            for (int j = lane; j <= k; j += 32) q[0] += h[j] * h[j];
+            warp_sums(q);
+            if (lane == 0) again_s = always2 || wnorm0 - q[0] < 0.49 * wnorm0;
+        }
         // w -= V_k h on this block's rows, and ||w||^2
         double acc = 0.0;
         for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
             double wi = w[i];
+#pragma unroll 8
             for (int j = 0; j <= k; j++) wi -= h[j] * v.V[(long long)j * v.ldv + i];
             w[i] = wi;
             acc += wi * wi;
         }
-        for (int j = threadIdx.x; j <= k; j += blockDim.x) hsum[j] += h[j];
-        acc = block_sum(acc, red);
-        // slot k+1 is free (h used slots 0..k); keep it separate from them
-        publish(v.part, LS_MAX_RESTART + 1, acc);
-        if (!grid_sync(v.bar, st)) break;
-        if (threadIdx.x < 32) {
-            const double t = reduce_slot(v.part, LS_MAX_RESTART + 1, G);
-            if (threadIdx.x == 0) wn_s = t;
-        }
         __syncthreads();
-        wn2 = wn_s;
-        // a second pass only when cancellation lost accuracy (or always if asked)
-        if (pass == 0 && !always2 && !(wn2 < 0.49 * wnorm0)) break;
+        if (pass == 0 && again_s) continue;
+        acc = block_sum(acc, red);
+        publish(v.part, LS_MAX_RESTART + 1, acc);   // a slot that no h uses
+        const unsigned ticket = grid_arrive(v.bar);
+        if (blockIdx.x == 0 && warp == 2) {
+            // while the others arrive: the earlier rotations on the column.  a_j = -s_j a_(j-1) + c_j h_j
+            // is the chain; everything else is done for all j at once.
+            for (int j = lane; j < k; j += 32) hrot[j] = cs[j] * hsum[j + 1];
+            __syncwarp();
+            double a = hsum[0];
+            for (int j = 0; j < k; j++) {
+                const double t = hrot[j];
+                __syncwarp();
+                if (lane == 0) hrot[j] = a;
+                a = fma(-sn[j], a, t);
+            }
+            if (lane == 0) hrot[k] = a;
+            __syncwarp();
+            for (int j = lane; j < k; j += 32) hrot[j] = fma(cs[j], hrot[j], sn[j] * hsum[j + 1]);
+        }
+        if (threadIdx.x == 96) w0_s = 1e-14 * sqrt(wnorm0);
+        ok = grid_wait(v.bar, ticket, st);
+        if (ok && warp == 0) {
+            const double t = reduce_slot(v.part, LS_MAX_RESTART + 1, G);
+            if (lane == 0) wn2_s = t;
+        }
+        break;
     }
-    if (st->err) {
+    __syncthreads();
+    if (st->err || !ok) {
         if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(v.st, h_inner, 0);
         return;
     }
-    const double wn = sqrt(wn2);
-    const bool lucky = !(wn > 1e-14 * sqrt(wnorm0));
+    const double wn2 = wn2_s;
+    // block 0's warp 2 forms the new rotation while warp 0 forms ||w|| and its reciprocal
+    double den = 0.0, dinv = 0.0;
+    const bool rotates = blockIdx.x == 0 && warp == 2;
+    if (rotates) {
+        const double hk = hrot[k], d2 = fma(hk, hk, wn2);
+        if (d2 > 1e-250 && d2 < 1e250) {
+            const RootInv r = root_inv(d2);
+            den = r.r;
+            dinv = r.inv;
+        } else {
+            den = hypot(hk, sqrt(wn2));
+            dinv = 1.0 / den;
+        }
+    } else if (warp == 0) {
+        const RootInv r = root_inv(wn2);
+        if (lane == 0) {
+            wn_s = r.r;
+            winv_s = r.inv;
+        }
+    }
+    __syncthreads();
+    const double wn = wn_s, winv = winv_s;
+    const bool lucky = !(wn > w0_s);
     if (!lucky)
-        for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) w[i] = w[i] / wn;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) w[i] = isfinite(winv) ? quot(w[i], wn, winv) : w[i] / wn;
+    if (rotates) {
         GmresSmall *gm = v.gm;
         const int m1 = LS_MAX_RESTART + 1;
         double *Hk = gm->H + (size_t)k * m1;
-        for (int j = 0; j <= k; j++) Hk[j] = hsum[j];
-        Hk[k + 1] = wn;
-        for (int j = 0; j < k; j++) {          // earlier rotations
-            const double a = Hk[j], c = Hk[j + 1];
-            Hk[j] = gm->cs[j] * a + gm->sn[j] * c;
-            Hk[j + 1] = -gm->sn[j] * a + gm->cs[j] * c;
-        }
-        const double den = hypot(Hk[k], Hk[k + 1]);
-        bool stop = false;
-        if (den == 0.0 || !isfinite(den)) {
-            st->status = LS_BREAKDOWN;
-            if (!isfinite(den)) set_err(st, ERRB_NAN);
-            stop = true;
-        } else {
-            const double c = Hk[k] / den, s = Hk[k + 1] / den;
-            gm->cs[k] = c;
-            gm->sn[k] = s;
-            Hk[k] = den;
-            Hk[k + 1] = 0.0;
-            gm->g[k + 1] = -s * gm->g[k];
-            gm->g[k] = c * gm->g[k];
-            st->k = k + 1;
-            st->total += 1;
-            st->est = fabs(gm->g[k + 1]);
-            if (st->est <= st->tol_abs || lucky || k + 1 >= st->m || st->total >= st->max_iter)
+        for (int j = lane; j < k; j += 32) Hk[j] = hrot[j];
+        if (lane == 0) {
+            const double hk = hrot[k];
+            bool stop = false;
+            if (den == 0.0 || !isfinite(den)) {
+                Hk[k] = hk;
+                Hk[k + 1] = wn;
+                st->status = LS_BREAKDOWN;
+                if (!isfinite(den)) set_err(st, ERRB_NAN);
                 stop = true;
+            } else {
+                const bool fine = isfinite(dinv);
+                const double c = fine ? quot(hk, den, dinv) : hk / den, sg = fine ? quot(wn, den, dinv) : wn / den;
+                gm->cs[k] = c;
+                gm->sn[k] = sg;
+                Hk[k] = den;
+                Hk[k + 1] = 0.0;
+                const double gk = gm->g[k], gn = -sg * gk;
+                gm->g[k + 1] = gn;
+                gm->g[k] = c * gk;
+                st->k = k + 1;
+                const int total = st->total + 1;
+                st->total = total;
+                const double est = fabs(gn);
+                st->est = est;
+                if (est <= st->tol_abs || lucky || k + 1 >= st->m || total >= st->max_iter) stop = true;
+            }
+            if (stop) set_cond(v.st, h_inner, 0);
         }
-        if (stop) set_cond(v.st, h_inner, 0);
     }
 }
 
@@ -418,25 +528,54 @@ __global__ void __launch_bounds__(KB) gm_finish_kernel(Vecs v) {
     if (st->status == LS_BREAKDOWN || st->err || k == 0) return;
     GmresSmall *gm = v.gm;
     const int m1 = LS_MAX_RESTART + 1;
-    if (blockIdx.x == 0 && threadIdx.x < 32) {
-        // back substitution by one warp: row i uses y_{i+1..k-1}
+    // Back substitution by columns, one warp of every block (the same operations, the same
+    // bits, no barrier): lane holds g_j for j = lane, lane + 32, ...  The reciprocals of the
+    // diagonal are formed at once; a quotient from one is corrected by its remainder.
+    if (threadIdx.x < 32) {
+        constexpr int Q = (LS_MAX_RESTART + 31) / 32;
         const int lane = threadIdx.x;
-        for (int i = k - 1; i >= 0; i--) {
-            double s = 0.0;
-            for (int j = i + 1 + lane; j < k; j += 32) s += gm->H[(size_t)j * m1 + i] * ys[j];
-            s = warp_sum(s);
-            if (lane == 0) ys[i] = (gm->g[i] - s) / gm->H[(size_t)i * m1 + i];
-            __syncwarp();
+        double g[Q], d[Q], rinv[Q];
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            const int j = lane + 32 * q;
+            g[q] = j < k ? __ldcg(&gm->g[j]) : 0.0;
+            d[q] = j < k ? __ldcg(&gm->H[(size_t)j * m1 + j]) : 1.0;
+            rinv[q] = 1.0;
+            if (32 * q < k) rinv[q] = 1.0 / d[q];
         }
-        for (int j = lane; j < k; j += 32) gm->y[j] = ys[j];
+        for (int i = k - 1; i >= 0; i--) {
+            double col[Q];   // column i above the diagonal
+#pragma unroll
+            for (int q = 0; q < Q; q++) {
+                const int j = lane + 32 * q;
+                col[q] = j < i ? __ldcg(&gm->H[(size_t)i * m1 + j]) : 0.0;
+            }
+            double gi = 0.0, di = 1.0, ri = 1.0;
+#pragma unroll
+            for (int q = 0; q < Q; q++)
+                if (i / 32 == q) {
+                    gi = g[q];
+                    di = d[q];
+                    ri = rinv[q];
+                }
+            gi = __shfl_sync(0xffffffffu, gi, i & 31);
+            di = __shfl_sync(0xffffffffu, di, i & 31);
+            ri = __shfl_sync(0xffffffffu, ri, i & 31);
+            double y = gi * ri;
+            y = fma(ri, fma(-di, y, gi), y);
+            if (!isfinite(ri) || !isfinite(y)) y = gi / di;   // a diagonal entry near the ends of the range
+            if (lane == 0) ys[i] = y;
+#pragma unroll
+            for (int q = 0; q < Q; q++)
+                if (32 * q < i) g[q] -= col[q] * y;
+        }
     }
-    if (!grid_sync(v.bar, st)) return;
-    for (int j = threadIdx.x; j < k; j += blockDim.x) ys[j] = __ldcg(&gm->y[j]);
     __syncthreads();
     long long lo, hi;
     block_range(v.n, blockIdx.x, gridDim.x, lo, hi);
     for (long long i = lo + threadIdx.x; i < hi; i += blockDim.x) {
         double xi = v.x[i];
+#pragma unroll 4
         for (int j = 0; j < k; j++) xi += v.V[(long long)j * v.ldv + i] * ys[j];
         v.x[i] = xi;
     }

@@ -456,6 +456,11 @@ Vecs make_vecs(ls_ctx *c, const F64Layout &L, int n, double rtol) {
 
 }  // namespace lsi
 
+// CTAs of the vector kernels: one per SM, but not fewer than 32 rows each: every CTA's
+// partial sums are added by every CTA, and an FP64 instruction costs a warp the same for
+// 13 rows as for 32 (GMRES(35), n = 2000: 152 -> 63 CTAs).
+static int vec_grid(const ls_ctx *c, int n) { return std::max(1, std::min(c->K.coop_grid, (n + 31) / 32)); }
+
 // Builds: [resid GEMV if x0] cg_init, while(outer){ while(inner){GEMV, update}, resid GEMV, check }
 static int build_cg_graph(ls_ctx *c, const Vecs &v, const Product &A, int x0_given,
                           const long long *key) {
@@ -477,7 +482,7 @@ static int build_cg_graph(ls_ctx *c, const Vecs &v, const Product &A, int x0_giv
         Vecs vv = v;
         int x0 = x0_given;
         void *args[] = {&vv, &x0, &ho, &hi};
-        top.kernel(c->K.cg_init, c->K.coop_grid, c->K.block, 0, args, true);
+        top.kernel(c->K.cg_init, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
     Chain outer = top.loop(ho);
     Chain inner = outer.loop(hi);
@@ -488,7 +493,7 @@ static int build_cg_graph(ls_ctx *c, const Vecs &v, const Product &A, int x0_giv
         product_node(inner, A, a);
         Vecs vv = v;
         void *args[] = {&vv, &hi};
-        inner.kernel(c->K.cg_update, c->K.coop_grid, c->K.block, 0, args, true);
+        inner.kernel(c->K.cg_update, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
     {
         GemvArgs a{};
@@ -497,7 +502,7 @@ static int build_cg_graph(ls_ctx *c, const Vecs &v, const Product &A, int x0_giv
         product_node(outer, A, a);
         Vecs vv = v;
         void *args[] = {&vv, &ho, &hi};
-        outer.kernel(c->K.cg_check, c->K.coop_grid, c->K.block, 0, args, false);
+        outer.kernel(c->K.cg_check, vec_grid(c, v.n), c->K.block, 0, args, false);
     }
     if (top.err != cudaSuccess || inner.err != cudaSuccess || outer.err != cudaSuccess) {
         R.discard();
@@ -529,7 +534,7 @@ static int build_bicgstab_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, i
         Vecs vv = v;
         int x0 = x0_given;
         void *args[] = {&vv, &x0, &ho, &hi};
-        top.kernel(c->K.bs_init, c->K.coop_grid, c->K.block, 0, args, true);
+        top.kernel(c->K.bs_init, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
     Chain outer = top.loop(ho);
     Chain inner = outer.loop(hi);
@@ -540,13 +545,13 @@ static int build_bicgstab_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, i
         gemv_node(inner, L, dA, a);
         Vecs vv = v;
         void *args[] = {&vv, &hi};
-        inner.kernel(c->K.bs_s, c->K.coop_grid, c->K.block, 0, args, true);
+        inner.kernel(c->K.bs_s, vec_grid(c, v.n), c->K.block, 0, args, true);
         GemvArgs a2{};
         a2.x = v.s; a2.y = v.t; a2.z = v.s; a2.st = v.st; a2.scr = c->scr;
         a2.epi = EPI_DOT; a2.fin = FIN_STORE;          // st->dot = t.s
         gemv_node(inner, L, dA, a2);
         void *args2[] = {&vv, &hi};
-        inner.kernel(c->K.bs_update, c->K.coop_grid, c->K.block, 0, args2, true);
+        inner.kernel(c->K.bs_update, vec_grid(c, v.n), c->K.block, 0, args2, true);
     }
     {
         GemvArgs a{};
@@ -555,7 +560,7 @@ static int build_bicgstab_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, i
         gemv_node(outer, L, dA, a);
         Vecs vv = v;
         void *args[] = {&vv, &ho, &hi};
-        outer.kernel(c->K.bs_check, c->K.coop_grid, c->K.block, 0, args, true);
+        outer.kernel(c->K.bs_check, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
     if (top.err != cudaSuccess || inner.err != cudaSuccess || outer.err != cudaSuccess) {
         R.discard();
@@ -579,7 +584,7 @@ static int build_jacobi_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int
         Vecs vv = v;
         int x0 = x0_given;
         void *args[] = {&vv, &x0, &hl};
-        top.kernel(c->K.ja_init, c->K.coop_grid, c->K.block, 0, args, true);
+        top.kernel(c->K.ja_init, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
     Chain loop = top.loop(hl);
     {
@@ -589,7 +594,7 @@ static int build_jacobi_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int
         gemv_node(loop, L, c->dA, a);
         Vecs vv = v;
         void *args[] = {&vv, &hl};
-        loop.kernel(c->K.ja_next, c->K.coop_grid, c->K.block, 0, args, false);
+        loop.kernel(c->K.ja_next, vec_grid(c, v.n), c->K.block, 0, args, false);
     }
     if (top.err != cudaSuccess || loop.err != cudaSuccess) {
         R.discard();
@@ -613,7 +618,7 @@ static int build_gs_graph(ls_ctx *c, const Vecs &v, const F64Layout &L, const Ge
         Vecs vv = v;
         int x0 = x0_given;
         void *args[] = {&vv, &x0, &hl};
-        top.kernel(c->K.ja_init, c->K.coop_grid, c->K.block, 0, args, true);
+        top.kernel(c->K.ja_init, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
     Chain loop = top.loop(hl);
     {
@@ -644,7 +649,7 @@ static int build_gs_graph(ls_ctx *c, const Vecs &v, const F64Layout &L, const Ge
     return finish_graph(c, c->graph_gs, R, key);
 }
 
-// Builds: gm_init, while(outer){ resid GEMV, gm_start, while(inner){GEMV, arnoldi}, gm_finish }
+// Builds: gm_init, [resid GEMV if x0] gm_start, while(outer){ while(inner){GEMV, arnoldi}, gm_finish, resid GEMV, gm_start }
 static int build_gmres_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int x0_given,
                              const long long *key) {
     Root R;
@@ -656,22 +661,27 @@ static int build_gmres_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int 
     }
     const MatDesc *dA = c->dA;
     Chain top = R.chain();
+    // q = b - A x and ||q||, then the decision to start a cycle or to end
+    auto residual = [&](Chain &ch) {
+        GemvArgs a{};
+        a.x = v.x; a.y = v.q; a.b = v.b; a.st = v.st; a.scr = c->scr;
+        a.epi = EPI_RESID; a.fin = FIN_TRUE_RES;
+        gemv_node(ch, L, dA, a);
+    };
+    auto start = [&](Chain &ch) {
+        Vecs vv = v;
+        void *args[] = {&vv, &ho, &hi};
+        ch.kernel(c->K.gm_start, vec_grid(c, v.n), c->K.block, 0, args, false);
+    };
     {
         Vecs vv = v;
         int x0 = x0_given;
         void *args[] = {&vv, &x0, &ho};
-        top.kernel(c->K.gm_init, c->K.coop_grid, c->K.block, 0, args, true);
+        top.kernel(c->K.gm_init, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
+    if (x0_given) residual(top);
+    start(top);
     Chain outer = top.loop(ho);
-    {
-        GemvArgs a{};
-        a.x = v.x; a.y = v.q; a.b = v.b; a.st = v.st; a.scr = c->scr;
-        a.epi = EPI_RESID; a.fin = FIN_TRUE_RES;
-        gemv_node(outer, L, dA, a);
-        Vecs vv = v;
-        void *args[] = {&vv, &ho, &hi};
-        outer.kernel(c->K.gm_start, c->K.coop_grid, c->K.block, 0, args, false);
-    }
     Chain inner = outer.loop(hi);
     {
         GemvArgs a{};
@@ -681,13 +691,15 @@ static int build_gmres_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int 
         gemv_node(inner, L, dA, a);
         Vecs vv = v;
         void *args[] = {&vv, &hi};
-        inner.kernel(c->K.gm_arnoldi, c->K.coop_grid, c->K.block, 0, args, true);
+        inner.kernel(c->K.gm_arnoldi, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
     {
         Vecs vv = v;
         void *args[] = {&vv};
-        outer.kernel(c->K.gm_finish, c->K.coop_grid, c->K.block, 0, args, true);
+        outer.kernel(c->K.gm_finish, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
+    residual(outer);
+    start(outer);
     if (top.err != cudaSuccess || inner.err != cudaSuccess || outer.err != cudaSuccess) {
         R.discard();
         return LS_ERR_CUDA;
@@ -847,7 +859,7 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
     } else if (method == LS_METHOD_CG || method == LS_METHOD_BICGSTAB) {
         passes = s.iter + s.cycles + (o.x0_given ? 1 : 0);
     } else {
-        passes = s.total + s.cycles + 1;
+        passes = s.total + s.cycles + (o.x0_given ? 1 : 0);
         sc.iter = s.total;
         sc.rnorm = s.est;   // the Givens estimate of the last step
     }

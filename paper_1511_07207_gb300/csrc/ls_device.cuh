@@ -180,17 +180,13 @@ __device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
 // add up to 2^31 whatever the grid's size, so the word's top bit flips with the last
 // of them and the waiting blocks see it in one L2 round trip (a second word, written by
 // the last block, made it two).
-__device__ __forceinline__ bool grid_sync(GridBar *b, State *st) {
+__device__ __forceinline__ bool grid_wait(GridBar *b, unsigned ticket, State *st) {
     __shared__ int ok_s;
-    __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        __threadfence();
-        const unsigned mine = blockIdx.x == 0 ? (1u << 31) - (gridDim.x - 1) : 1u;
-        const unsigned before = atomicAdd(&b->count, mine);
         unsigned polls = 0;
         unsigned long long t0 = 0;
-        while (((ld_acquire_u32(&b->count) ^ before) >> 31) == 0) {
+        while (((ld_acquire_u32(&b->count) ^ ticket) >> 31) == 0) {
             if (++polls < 64) continue;
             if (t0 == 0) t0 = gtimer();
             __nanosleep(64);
@@ -205,6 +201,15 @@ __device__ __forceinline__ bool grid_sync(GridBar *b, State *st) {
     __syncthreads();
     return ok_s != 0;
 }
+// The arrival of a block, all of whose threads call it (after their writes); what
+// thread 0 returns goes to grid_wait.  Work that no other block waits for can stand in between.
+__device__ __forceinline__ unsigned grid_arrive(GridBar *b) {
+    __syncthreads();
+    if (threadIdx.x != 0) return 0;
+    __threadfence();
+    return atomicAdd(&b->count, blockIdx.x == 0 ? (1u << 31) - (gridDim.x - 1) : 1u);
+}
+__device__ __forceinline__ bool grid_sync(GridBar *b, State *st) { return grid_wait(b, grid_arrive(b), st); }
 
 // ---- grid-stride ranges --------------------------------------------------------------
 // Balanced contiguous range [lo, hi) of 0..n for block `b` of `nb`.
