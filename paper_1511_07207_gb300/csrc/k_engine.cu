@@ -269,13 +269,16 @@ __global__ void __launch_bounds__(RED_T) eng_red_kernel(const EngineDev *Ep, cud
 // ============================================================================
 constexpr int PC_W = P32_T / 32;                     // consumer warps
 constexpr int PROD_T = P32_T + 64;                   // + the producer warp and the MMA warp
-constexpr int PSTAGES = 3;                           // ring stages
+constexpr int PSTAGES = 4;                           // ring stages
 constexpr int PREFETCH = 4;                          // tiles of a task brought into L2 ahead of their copy
 constexpr int TILE_B = E_RB32 * E_KC32 * 4;          // 32 KB A tile
 constexpr int OPR_B = E_KC32 * 32 * 4;               // one raw operand chunk (widest slot)
 constexpr int BOP_B = E_MAXS * E_KC32 * 4;           // one K-major tensor-core B operand (4 KB)
-constexpr int TMEM_COLS = 256;                       // two 128-row halves of the tile:
-constexpr int TC_HALF_COLS = 128;                    // per half Ah [Bh | Bt] (2 sp columns), then At Bh (sp)
+constexpr int TMEM_COLS = 512;                       // all of an SM's tensor memory:
+constexpr int TC_HALF_COLS = 128;                    // accumulators of a 128-row half of the tile: Ah [Bh | Bt]
+                                                     // (2 sp columns), then At Bh (sp)
+constexpr int TC_A_COL = 2 * TC_HALF_COLS;           // A, two buffers of 128 columns: per half the 32 columns'
+                                                     // heads, then their tails
 static_assert(E_KC32 * 4 == 128, "a tile row is one 128-byte swizzle row");
 
 struct StageHdr {
@@ -289,8 +292,8 @@ enum : int { SF_FIRST = 1, SF_LAST = 2, SF_SRC2 = 4 };
 
 constexpr size_t align_c(size_t v, size_t a) { return (v + a - 1) / a * a; }
 constexpr size_t OFF_TILE = 0;                                         // 1024-aligned tiles
-constexpr size_t OFF_CVT = OFF_TILE + (size_t)PSTAGES * TILE_B;        // [2] tensor-core tail tiles
-constexpr size_t OFF_BOP = OFF_CVT + 2 * (size_t)TILE_B;               // [2] B operands [head; tail] /
+constexpr size_t OFF_CVT = OFF_TILE + (size_t)PSTAGES * TILE_B;        // the tensor-core path's staging copy
+constexpr size_t OFF_BOP = OFF_CVT + (size_t)TILE_B;                   // [2] B operands [head; tail] /
                                                                        // the FP32 path's two operand chunks
 constexpr size_t OFF_OPR = OFF_BOP + 4 * (size_t)BOP_B;                // [stage][2][OPR_B]
 constexpr size_t OFF_HDR = OFF_OPR + (size_t)PSTAGES * 2 * OPR_B;
@@ -325,9 +328,9 @@ struct ProdSmem {
     __device__ uint32_t *tslot() const { return reinterpret_cast<uint32_t *>(base + OFF_TSLOT); }
     // FP32 path: operand chunk b (32 rows x sp, row-major)
     __device__ float *ps(int b) const { return reinterpret_cast<float *>(base + OFF_BOP + (size_t)b * BOP_B); }
-    // tensor-core path, buffer parity b: the TF32 tail of the A tile (its head is written over
-    // the stage's tile) and the B operand, 2 sp rows of 128 bytes: the operand's head, then its tail
-    __device__ float *tail(int b) const { return reinterpret_cast<float *>(base + OFF_CVT + (size_t)b * TILE_B); }
+    // tensor-core path: the accumulators' staging copy, and the B operand of buffer parity b, 2 sp
+    // rows of 128 bytes: the operand's head, then its tail
+    __device__ float *staging() const { return reinterpret_cast<float *>(base + OFF_CVT); }
     __device__ float *bop(int b) const { return reinterpret_cast<float *>(base + OFF_BOP + (size_t)b * 2 * BOP_B); }
     __device__ double *red() const { return reinterpret_cast<double *>(base + OFF_RED); }
 };
@@ -559,26 +562,26 @@ __device__ bool prod_task(const EngineDev &E, const ProdSmem &M, int &seq, int *
 // build each chunk's operand as in the FP32 form; then every FP32 value v of
 // the chunk and of the 256 x 32 tile of A is split into a TF32 head h = rn(v)
 // and a TF32 tail t = rn(v - h) (v = h + t to about 2^-24 |v|): the tile's
-// head is written over the tile, its tail into the tail tile of the buffer
-// parity, the operand's head and tail as the two halves of one K-major
-// 128-byte-swizzled B operand [Bh; Bt] of 2 sp rows.  The chunk is then
-// handed to the MMA warp, which issues, per 8-column step of K and per
-// 128-row half of the tile (tcgen05.mma kind::tf32, FP32 accumulators in
-// tensor memory),
+// heads and tails go from the threads' registers into tensor memory (a thread
+// one row of the tile, 32 + 32 columns, the two 128-row halves side by side), the
+// operand's head and tail become the two halves of one K-major
+// 128-byte-swizzled B operand [Bh; Bt] of 2 sp rows in shared memory.  Both have two
+// buffers.  The chunk is then handed to the MMA warp, which issues, per 8-column
+// step of K and per 128-row half of the tile (tcgen05.mma kind::tf32, FP32
+// accumulators in tensor memory),
 //     D1 += Ah [Bh | Bt]   (N = 2 sp: A's head is read once for both)
 //     D2 += At Bh          (N = sp)
 // so that Y = D1[:, :sp] + D1[:, sp:] + D2 (the dropped At Bt is below
-// 2^-24 |A||P|), and commits twice: to the stage's "empty" barrier (the
-// stage goes back to the producer when the products that read it are done)
-// and to the parity's "done" barrier (the consumers may then overwrite that
-// parity's tail tile and B operand, two chunks later).  The consumers wait
-// for the tensor core only before reusing a buffer parity and for the task's
-// last chunk; the accumulators then come back through tcgen05.ld, summed,
-// through a shared-memory staging copy into the FP32 form's register layout,
-// and the task ends as the FP32 form does.
+// 2^-24 |A||P|), and commits to the parity's "done" barrier (the consumers may then
+// overwrite that parity's A and B, two chunks later).  A stage goes back to the
+// producer as soon as the consumers have read it.  They wait for the tensor core only
+// before reusing a buffer parity and for the task's last chunk; the accumulators then
+// come back through tcgen05.ld, summed, through a shared-memory staging copy into
+// the FP32 form's register layout, and the task ends as the FP32 form does.
+// With A's head and tail in shared memory a chunk moved 250 KB through it (the
+// copy, the split's 96 KB, the MMAs' reads of A).
 // ----------------------------------------------------------------------------
 struct TcQ {                 // a chunk handed to the MMA warp
-    int st;                  // ring stage holding the tile's head
     int sp;                  // 16 or 32
     int first;               // first chunk of its task (accumulators start from zero)
     int stop;                // no more chunks in this launch
@@ -634,9 +637,10 @@ __device__ bool prod_task_tc(const EngineDev &E, const ProdSmem &M, int &seq, in
         bool ok = ch == 0 || tc_wait(M.full(st), (seq / PSTAGES) & 1, tc.fail_s);
         const unsigned q = tc.cseq;
         const int b = q & 1;
-        // the tail tile and B operand of parity b were last read by chunk q - 2
+        // A and B of parity b were last read by chunk q - 2
         if (q >= 2) ok = tc_wait(M.mma(b), ((q - 2) >> 1) & 1, tc.fail_s) && ok;
-        if (ok) {
+        if (__all_sync(0xffffffffu, ok)) {   // the warp's stores to tensor memory are made together
+            tc_fence_after();
             const StageHdr &H = *M.hdr(st);
             const float *o1 = M.opr(st, 0), *o2 = M.opr(st, 1);
             const bool two = (H.flags & SF_SRC2) != 0;
@@ -665,19 +669,32 @@ __device__ bool prod_task_tc(const EngineDev &E, const ProdSmem &M, int &seq, in
                 *reinterpret_cast<float4 *>(Bo + pos) = make_float4(hv[0], hv[1], hv[2], hv[3]);
                 *reinterpret_cast<float4 *>(Bo + SP * KC + pos) = make_float4(tv[0], tv[1], tv[2], tv[3]);
             }
-            float4 *Ah4 = reinterpret_cast<float4 *>(M.tile(st));
-            float4 *At4 = reinterpret_cast<float4 *>(M.tail(b));
-#pragma unroll 4
-            for (int e = tid; e < TILE_B / 16; e += P32_T) {
-                const float4 a = Ah4[e];
-                const float4 h = make_float4(tf32_rn(a.x), tf32_rn(a.y), tf32_rn(a.z), tf32_rn(a.w));
-                Ah4[e] = h;
-                At4[e] = make_float4(tf32_rn(a.x - h.x), tf32_rn(a.y - h.y), tf32_rn(a.z - h.z), tf32_rn(a.w - h.w));
+            // A: a thread splits one row of the tile (warps 0 .. 3 its upper half), head and tail into
+            // its lane of tensor memory
+            const int trow = tid;
+            const float4 *Ar = reinterpret_cast<const float4 *>(M.tile(st)) + trow * (KC / 4);
+            const uint32_t ta = tc.tmem + ((uint32_t)((warp & 3) * 32) << 16) + TC_A_COL + 128 * b + 64 * (warp >> 2);
+#pragma unroll
+            for (int g = 0; g < 2; g++) {
+                float hv[16], tv[16];
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const float4 a = Ar[(4 * g + j) ^ (trow & 7)];
+                    const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+                    for (int c = 0; c < 4; c++) {
+                        hv[4 * j + c] = tf32_rn(av[c]);
+                        tv[4 * j + c] = tf32_rn(av[c] - hv[4 * j + c]);
+                    }
+                }
+                tmem_st16(ta + 16 * g, hv);
+                tmem_st16(ta + 32 + 16 * g, tv);
             }
+            tmem_wait_st();
+            tc_fence_before();
         }
         if (tid == 0) {
             TcQ &Q = M.tcq()[b];
-            Q.st = st;
             Q.sp = SP;
             Q.first = ch == 0;
             Q.stop = 0;
@@ -686,7 +703,7 @@ __device__ bool prod_task_tc(const EngineDev &E, const ProdSmem &M, int &seq, in
         __syncwarp();
         if (lane == 0) {
             mbar_arrive(M.conv(b));
-            if (warp != PC_W - 1) mbar_arrive(M.empty(st));   // the eighth arrival: the MMA warp's commit
+            mbar_arrive(M.empty(st));        // the stage's tile and operand rows have been read
         }
         tc.cseq++;
         seq++;
@@ -701,7 +718,7 @@ __device__ bool prod_task_tc(const EngineDev &E, const ProdSmem &M, int &seq, in
         const int h = warp >> 2, qw = warp & 3;
         const int row = h * 128 + qw * 32 + lane;
         const uint32_t ta = tc.tmem + ((uint32_t)(qw * 32) << 16) + (uint32_t)(TC_HALF_COLS * h);
-        float4 *Ys = reinterpret_cast<float4 *>(M.tail(0));
+        float4 *Ys = reinterpret_cast<float4 *>(M.staging());
 #pragma unroll
         for (int c0 = 0; c0 < SP; c0 += 16) {
             float v1[16], v2[16], v3[16];
@@ -723,7 +740,7 @@ __device__ bool prod_task_tc(const EngineDev &E, const ProdSmem &M, int &seq, in
     named_bar(1, P32_T);
     float acc[RPT][4];
     {
-        const float4 *Ys = reinterpret_cast<const float4 *>(M.tail(0));
+        const float4 *Ys = reinterpret_cast<const float4 *>(M.staging());
 #pragma unroll
         for (int r = 0; r < RPT; r++) {
             const int row = rg + NRG * r;
@@ -764,7 +781,7 @@ __device__ unsigned tc_mma_warp(const EngineDev &E, const ProdSmem &M, uint32_t 
         if (Q.stop) break;
         if (lane == 0) {
             tc_fence_after();
-            const uint32_t ah = smem_u32(M.tile(Q.st)), at = smem_u32(M.tail(b)), bo = smem_u32(M.bop(b));
+            const uint32_t bo = smem_u32(M.bop(b));
             const int sp = Q.sp;
             const uint32_t id1 = tc_idesc_tf32(128, 2 * sp), id2 = tc_idesc_tf32(128, sp);
 #pragma unroll
@@ -773,13 +790,12 @@ __device__ unsigned tc_mma_warp(const EngineDev &E, const ProdSmem &M, uint32_t 
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
                     const uint32_t d1 = tmem + TC_HALF_COLS * h, d2 = d1 + 2 * sp;
-                    const uint32_t ao = h * (TILE_B / 2) + kk * 32;
+                    const uint32_t ah = tmem + TC_A_COL + 128 * b + 64 * h + 8 * kk;
                     const bool acc = !Q.first || kk > 0;
-                    tc_mma_tf32(d1, tc_desc_sw128(ah + ao), db, id1, acc);
-                    tc_mma_tf32(d2, tc_desc_sw128(at + ao), db, id2, acc);
+                    tc_mma_tf32_ta(d1, ah, db, id1, acc);
+                    tc_mma_tf32_ta(d2, ah + 32, db, id2, acc);
                 }
             }
-            tc_commit(M.empty(Q.st));
             tc_commit(M.mma(b));
         }
         __syncwarp();

@@ -2,10 +2,11 @@
 //
 // Used by the block products, the only dense contractions on the solver path:
 // Y = A P with P a block of s right-hand-side directions.  One elected thread
-// issues tcgen05.mma with both operands in shared memory (K-major, 128-byte
-// swizzle, the layout a 2-D TMA copy with CU_TENSOR_MAP_SWIZZLE_128B writes);
-// the accumulator lives in tensor memory (TMEM) and is read back with
-// tcgen05.ld after a tcgen05.commit has arrived on an mbarrier.
+// issues tcgen05.mma with A in tensor memory (TMEM, written by the threads that
+// split it, tcgen05.st) and B in shared memory (K-major, 128-byte swizzle, the
+// layout a 2-D TMA copy with CU_TENSOR_MAP_SWIZZLE_128B writes); the accumulator
+// lives in tensor memory too and is read back with tcgen05.ld after a
+// tcgen05.commit has arrived on an mbarrier.
 //
 // Shared-memory matrix descriptor (64 bits):
 //   [0,14)  start address >> 4      [16,30) leading-dimension byte offset >> 4
@@ -69,14 +70,15 @@ __device__ __forceinline__ void fence_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-// D (+)= A B, A and B in shared memory, D in tensor memory (one thread).
-__device__ __forceinline__ void tc_mma_tf32(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                            bool accumulate) {
+// D (+)= A B with A and D in tensor memory (row m of A in lane m, element k in 32-bit
+// column k) and B in shared memory (one thread).
+__device__ __forceinline__ void tc_mma_tf32_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                               bool accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
         "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
+        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)accumulate)
         : "memory");
 }
 
@@ -100,6 +102,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
 #pragma unroll
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
+// This lane's row (warp quarter * 32 + lane): 16 consecutive 32-bit columns from col.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&v)[16]) {
+    uint32_t r[16];
+#pragma unroll
+    for (int i = 0; i < 16; i++) r[i] = __float_as_uint(v[i]);
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
+        "%13, %14, %15};" ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // The part of an FP32 value a TF32 operand keeps (low 13 fraction bits
