@@ -25,11 +25,11 @@
 //     (128-byte swizzle, zero fill past n); the chain's M_{I,w} sit in a
 //     contiguous panel in its threads' read order, one 32 KB bulk copy per
 //     tile;
-//   * publication is a flag per block written with release semantics after
-//     the data, polled with acquire, with the sweep's number as its value
-//     (flags are zeroed per solve, so stale ones never match); the chain's
-//     flags are written by a second lane of the producer warp, signalled by
-//     an mbarrier, so the chain never waits for its own stores;
+//   * an entry of d or u is published as one 16-byte word with the sweep's number in it
+//     (zeroed per solve, so a stale one never matches): whoever needs it polls the
+//     word itself, one L2 round trip and no fence.  With a flag per block, stored behind the
+//     data and polled before it, each hand-over took two, and the chain waited for u
+//     in every step (n = 8000: 5.46 -> 4.63 ms a solve, n = 16384 13.9 -> 12.0);
 //   * every wait is bounded (the library's time limit, ERRB_TIMEOUT) and
 //     every decision that several warps act on is combined with a
 //     barrier-reduction, so no thread is left waiting on one that gave up;
@@ -45,11 +45,11 @@ constexpr int GS_B = 64;         // rows (and columns) of a block
 constexpr int GS_W = 3;          // sub-diagonal blocks the chain CTA multiplies itself
 constexpr int GS_C = 512;        // consumer threads (16 warps)
 constexpr int GS_LPR = GS_C / 64;// consumer lanes per tile row (8)
-constexpr int GS_T = GS_C + 64;  // plus the producer warp and the chain's u-fetcher warp
+constexpr int GS_FW = 2;         // the chain's u-fetcher warps
+constexpr int GS_T = GS_C + 32 + 32 * GS_FW;   // plus the producer warp and the u-fetcher warps
 constexpr int GS_SLOTS = 6;      // tile slots in the ring
 constexpr int GS_SLOT_B = 32768; // one tile: hi and lo, two 32-column boxes each
 constexpr int GS_BOX_B = 8192;   // 32 columns x 64 rows of FP32
-constexpr int GS_PUB = 8;        // chain publication mbarriers (steps in flight, > W + 1)
 constexpr int GS_UB = 4;         // chain: u blocks staged ahead in shared memory
 constexpr int GS_KMAX = 8;       // row blocks a helper owns at most
 constexpr int GS_BAR_C = 1;      // named barrier of the consumer warps
@@ -140,32 +140,52 @@ __device__ __forceinline__ F2 tile_dot(const unsigned char *slot, const float *v
 // one of consumer thread t at index t: columns 32h + 4q .. +3 of row t / 8,
 // q = t % 8 (the same columns as tile_dot).
 constexpr int GS_PANEL_TILE = 8192;   // floats
-__device__ __forceinline__ F2 tile_dot_panel(const unsigned char *slot, const float *vh, const float *vl) {
-    F2 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+struct PanelPart {
+    float4 mh[2], ml[2];
+};
+__device__ __forceinline__ PanelPart panel_part(const unsigned char *slot) {
     const float4 *P = reinterpret_cast<const float4 *>(slot);
+    PanelPart m;
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        m.mh[h] = P[(2 * h) * GS_C + threadIdx.x];
+        m.ml[h] = P[(2 * h + 1) * GS_C + threadIdx.x];
+    }
+    return m;
+}
+// acc[h] += the thread's share of M d over column half h (the two chains stay apart, and
+// unnormalised, over the step's tiles).
+__device__ __forceinline__ void panel_mac(F2 (&acc)[2], const PanelPart &m, const float *vh, const float *vl) {
     const int q = threadIdx.x % GS_LPR;
 #pragma unroll
     for (int h = 0; h < 2; h++) {
-        const float4 mh = P[(2 * h) * GS_C + threadIdx.x];
-        const float4 ml = P[(2 * h + 1) * GS_C + threadIdx.x];
         const int col = h * 32 + q * 4;
         const float4 xh = *reinterpret_cast<const float4 *>(vh + col);
         const float4 xl = *reinterpret_cast<const float4 *>(vl + col);
-        f2_mac(acc[h], mh.x, ml.x, xh.x, xl.x);
-        f2_mac(acc[h], mh.y, ml.y, xh.y, xl.y);
-        f2_mac(acc[h], mh.z, ml.z, xh.z, xl.z);
-        f2_mac(acc[h], mh.w, ml.w, xh.w, xl.w);
+        f2_mac(acc[h], m.mh[h].x, m.ml[h].x, xh.x, xl.x);
+        f2_mac(acc[h], m.mh[h].y, m.ml[h].y, xh.y, xl.y);
+        f2_mac(acc[h], m.mh[h].z, m.ml[h].z, xh.z, xl.z);
+        f2_mac(acc[h], m.mh[h].w, m.ml[h].w, xh.w, xl.w);
     }
-    return f2_add(acc[0], acc[1]);
 }
 
-// ---- flags --------------------------------------------------------------------------------
-// Thread 0 waits until *f == ep; false (and ERRB_TIMEOUT) after the time
-// limit, or false at once when another CTA has recorded an error.
-__device__ __forceinline__ bool flag_wait(const unsigned *f, unsigned ep, State *st) {
-    if (ld_acquire_u32(f) == ep) return true;
+// ---- words between the CTAs ---------------------------------------------------------------
+// An entry of d or u travels as one 16-byte word: its FP32 pair and the sweep's number.
+__device__ __forceinline__ void gs_put(GsWord *p, F2 v, unsigned ep) {
+    st_word128(p, ((unsigned long long)__float_as_uint(v.l) << 32) | __float_as_uint(v.h), ep);
+}
+__device__ __forceinline__ bool gs_get(const GsWord *p, unsigned ep, F2 &v) {
+    unsigned long long lo, hi;
+    ld_word128(p, lo, hi);
+    v = F2{__uint_as_float((unsigned)lo), __uint_as_float((unsigned)(lo >> 32))};
+    return (unsigned)hi == ep;
+}
+// Waits for the word of sweep ep; false (and ERRB_TIMEOUT) after the time limit, or false at
+// once when another CTA has recorded an error.
+__device__ __forceinline__ bool gs_wait(const GsWord *p, unsigned ep, F2 &v, State *st) {
+    if (gs_get(p, ep, v)) return true;
     const unsigned long long t0 = gtimer();
-    while (ld_acquire_u32(f) != ep) {
+    while (!gs_get(p, ep, v)) {
         if (*(volatile int *)&st->err) return false;
         if (gtimer() - t0 > WAIT_LIMIT_NS) {
             set_err(st, ERRB_TIMEOUT);
@@ -173,13 +193,6 @@ __device__ __forceinline__ bool flag_wait(const unsigned *f, unsigned ep, State 
         }
     }
     return true;
-}
-
-// Consumer threads: thread 0 polls the flag; all agree on the outcome.
-__device__ __forceinline__ bool consumers_wait_flag(const unsigned *f, unsigned ep, State *st) {
-    bool bad = false;
-    if (threadIdx.x == 0) bad = !flag_wait(f, ep, st);
-    return !named_bar_or(GS_BAR_C, GS_C, bad);
 }
 
 // Consumer threads: every thread waits for the slot's TMA data; all agree.
@@ -242,7 +255,7 @@ __global__ void __launch_bounds__(GS_B) gs_tinv_kernel(int n, const double *__re
 
 // ---- the chain's panel (once per solve, after T_I^-1) ---------------------------------------------
 // Tile (I, w), w = 1..W: M_{I,w} = T_I^-1 A_{I,I-w} in double-single
-// arithmetic from the FP32 pairs of T_I^-1 and A, laid out as tile_dot_panel
+// arithmetic from the FP32 pairs of T_I^-1 and A, laid out as panel_part
 // reads it (zero where I - w < 0 and past n).  T_I^-1 is lower triangular,
 // so row i sums k = 0..i; each warp runs k up to its last row (the entries
 // above the diagonal are stored zeros).
@@ -304,7 +317,7 @@ struct alignas(16) GsShared {
     float vh[2][GS_B], vl[2][GS_B];                   // vectors of the tile products
     float2 ub[GS_UB][GS_B];                           // chain: u_I staged by the fetcher warp
     float sh[GS_B], sl[GS_B];                         // helper: r_I - P_I of the block being finished
-    uint64_t full[GS_SLOTS], empty[GS_SLOTS], pub[GS_PUB], uready[GS_UB], ufree[GS_UB];
+    uint64_t full[GS_SLOTS], empty[GS_SLOTS], uready[GS_UB], ufree[GS_UB];
 };
 
 // Row block owned by helper g (0 .. H-1) in round k, or -1: blocks are
@@ -367,7 +380,7 @@ __device__ void gs_produce(const GsArgs &a, int nblk, GsShared *S, unsigned char
     bool go = true;
     if (chain) {
         for (int I = 0; I < nblk && go; I++)
-            for (int w = 1; w <= GS_W && go; w++)
+            for (int w = GS_W; w >= 1 && go; w--)
                 if (I - w >= 0) go = put_panel(I * GS_W + w - 1);
     } else {
         // the order gs_helper takes them: blocks without tiles first, then
@@ -391,63 +404,38 @@ __device__ void gs_produce(const GsArgs &a, int nblk, GsShared *S, unsigned char
         if (!mbar_wait(&S->full[k % GS_SLOTS], (k / GS_SLOTS) & 1)) set_err(st, ERRB_TIMEOUT);
 }
 
-// Publisher lane of the chain CTA: flagD[I] once the consumer warps have
-// stored d_I (they arrive on pub[I % GS_PUB]).
-__device__ void gs_publish(const GsArgs &a, unsigned ep, int nblk, GsShared *S) {
-    for (int I = 0; I < nblk; I++) {
-        if (!mbar_wait(&S->pub[I % GS_PUB], (I / GS_PUB) & 1)) {
-            set_err(a.st, ERRB_TIMEOUT);
-            return;
-        }
-        st_release_u32(&a.flagD[I], ep);
-    }
-}
-
-// Consumer thread 0 of a helper: wait until d_j is published.  The chain
-// publishes in order, so one acquire of flagD[J] covers every j <= J; the
-// furthest published flag among the next few is remembered in *known.
-__device__ __forceinline__ bool helper_wait_d(const GsArgs &a, unsigned ep, int j, int nblk, int *known) {
-    if (j < *known) return true;
-    if (!flag_wait(&a.flagD[j], ep, a.st)) return false;
-    int k = j + 1;
-#pragma unroll
-    for (int t = 0; t < 7; t++) {
-        if (k >= nblk) break;
-        unsigned v;
-        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&a.flagD[k]) : "memory");
-        if (v != ep) break;
-        k++;
-    }
-    asm volatile("fence.acq_rel.gpu;" ::: "memory");
-    *known = k;
-    return true;
-}
-
-// u-fetcher warp of the chain CTA: for I = 0, 1, ... wait until u_I is
-// published, copy it into ub[I % GS_UB] and signal uready; a buffer is
-// reused once the consumers have signalled ufree.
-__device__ void gs_fetch_u(const GsArgs &a, unsigned ep, int nblk, GsShared *S) {
+// u-fetcher warps of the chain CTA, warp f of GS_FW: for I = f, f + GS_FW, ... wait for
+// the words of u_I into ub[I % GS_UB] and signal uready; a buffer is
+// reused once the consumers have signalled ufree.  Two warps: one block's round
+// trip to L2 would otherwise be a step's least time.
+__device__ void gs_fetch_u(const GsArgs &a, unsigned ep, int nblk, GsShared *S, int f) {
     const int lane = threadIdx.x & 31;
-    for (int I = 0; I < nblk; I++) {
+    for (int I = f; I < nblk; I += GS_FW) {
         const int b = I % GS_UB;
         bool ok = I < GS_UB || mbar_wait(&S->ufree[b], ((I / GS_UB) - 1) & 1);
-        if (lane == 0 && ok) ok = flag_wait(&a.flagU[I], ep, a.st);
-        ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-        if (!ok) {
+        F2 v[2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+        for (int k = 0; k < 2; k++) {
+            const int gr = I * GS_B + lane + 32 * k;
+            if (gr < a.n && ok) ok = gs_wait(&a.u[gr], ep, v[k], a.st);
+        }
+        if (!__all_sync(0xffffffffu, ok)) {
             set_err(a.st, ERRB_TIMEOUT);
             return;
         }
-        __syncwarp();
-        for (int r = lane; r < GS_B; r += 32) {
-            const int gr = I * GS_B + r;
-            S->ub[b][r] = gr < a.n ? __ldcg(&a.u[gr]) : make_float2(0.f, 0.f);
-        }
+        S->ub[b][lane] = make_float2(v[0].h, v[0].l);
+        S->ub[b][lane + 32] = make_float2(v[1].h, v[1].l);
         __syncwarp();
         if (lane == 0) mbar_arrive(&S->uready[b]);
     }
 }
 
-// Chain consumers (CTA 0): d_I = u_I - sum_w M_{I,w} d_{I-w}.
+// Chain consumers (CTA 0): d_I = u_I - sum_w M_{I,w} d_{I-w}, the oldest d first: the
+// products with d_{I-W} .. d_{I-2} are made before the step's one barrier, behind
+// which d_{I-1} is known.  Each warp waits for its tiles itself; after a failed
+// wait (the error is recorded) a warp stops waiting and computing but keeps meeting the
+// others at the barriers.  A slot of the d ring (W + 1 of them) is written again only behind
+// a barrier that follows its last read.
 __device__ void gs_chain(const GsArgs &a, unsigned ep, int nblk, GsShared *S, const unsigned char *ring) {
     State *st = a.st;
     const int n = a.n, row = threadIdx.x / GS_LPR, q = threadIdx.x % GS_LPR;
@@ -457,40 +445,45 @@ __device__ void gs_chain(const GsArgs &a, unsigned ep, int nblk, GsShared *S, co
     }
     named_bar(GS_BAR_C, GS_C);
     int seq = 0;
+    bool ok = true;
+    auto wait = [&](uint64_t *bar, unsigned parity) {
+        ok = ok && mbar_wait(bar, parity);
+        if (!__all_sync(0xffffffffu, ok)) {
+            if (ok) ok = false;
+            set_err(st, ERRB_TIMEOUT);
+        }
+    };
     for (int I = 0; I < nblk; I++) {
         const int gr = I * GS_B + row;
-        F2 acc = {0.f, 0.f};
-        for (int w = 1; w <= GS_W; w++) {
+        F2 acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+        for (int w = GS_W; w >= 1; w--) {
             if (I - w < 0) continue;
             const int sl = seq % GS_SLOTS;
-            if (!consumers_wait_full(&S->full[sl], seq, st)) return;
+            wait(&S->full[sl], (seq / GS_SLOTS) & 1);
             const int dslot = (I - w) % (GS_W + 1);
-            acc = f2_add(acc, tile_dot_panel(ring + (size_t)sl * GS_SLOT_B, S->dh[dslot], S->dl[dslot]));
+            const PanelPart m = panel_part(ring + (size_t)sl * GS_SLOT_B);
+            if (w == 1) named_bar(GS_BAR_C, GS_C);   // d_{I-1} in shared memory
+            if (ok) panel_mac(acc, m, S->dh[dslot], S->dl[dslot]);
             consumers_release(&S->empty[sl]);
             seq++;
         }
-        const F2 t = f2_row_sum(acc);
+        const F2 t = f2_row_sum(f2_add(acc[0], acc[1]));
         // u_I, staged by the fetcher warp
         const int ubi = I % GS_UB;
-        const bool bad = !mbar_wait(&S->uready[ubi], (I / GS_UB) & 1);
-        if (bad) set_err(st, ERRB_TIMEOUT);
-        if (named_bar_or(GS_BAR_C, GS_C, bad)) return;
+        wait(&S->uready[ubi], (I / GS_UB) & 1);
         if (q == 0) {
             F2 d = {0.f, 0.f};
-            if (gr < n) {
+            if (gr < n && ok) {
                 const float2 u = S->ub[ubi][row];
                 d = f2_add(F2{u.x, u.y}, F2{-t.h, -t.l});
-                a.delta[gr] = make_float2(d.h, d.l);
+                gs_put(&a.delta[gr], d, ep);
             }
             S->dh[I % (GS_W + 1)][row] = d.h;
             S->dl[I % (GS_W + 1)][row] = d.l;
         }
         __syncwarp();
-        if ((threadIdx.x & 31) == 0) {
-            mbar_arrive(&S->pub[I % GS_PUB]);
-            mbar_arrive(&S->ufree[ubi]);
-        }
-        named_bar(GS_BAR_C, GS_C);   // d_I in shared memory before the next step
+        if ((threadIdx.x & 31) == 0) mbar_arrive(&S->ufree[ubi]);
     }
 }
 
@@ -514,9 +507,8 @@ __device__ bool gs_helper_finish(const GsArgs &a, unsigned ep, int I, double acc
     const F2 t = f2_row_sum(tile_dot(ring + (size_t)sl * GS_SLOT_B, S->sh, S->sl));
     consumers_release(&S->empty[sl]);
     (*seq)++;
-    if (q == 0 && r0 + row < n) a.u[r0 + row] = make_float2(t.h, t.l);
-    named_bar(GS_BAR_C, GS_C);
-    if (threadIdx.x == 0) st_release_u32(&a.flagU[I], ep);
+    if (q == 0 && r0 + row < n) gs_put(&a.u[r0 + row], t, ep);
+    named_bar(GS_BAR_C, GS_C);   // sh and sl are free
     return true;
 }
 
@@ -532,21 +524,26 @@ __device__ void gs_helper(const GsArgs &a, unsigned ep, int nblk, GsShared *S, c
         acc[m] = 0.0;
         if (m < K) jmax = max(jmax, Iown[m] - GS_W);
     }
-    int seq = 0, known = 0;
+    int seq = 0;
 #pragma unroll
     for (int m = 0; m < GS_KMAX; m++)
         if (m < K && Iown[m] - GS_W <= 0 && !gs_helper_finish(a, ep, Iown[m], 0.0, S, ring, &seq)) return;
+    // thread r < 64 brings entry r of d_j, asked for a column ahead
+    F2 next = {0.f, 0.f};
+    bool have = false;
     for (int j = 0; j < jmax; j++) {
         bool bad = false;
-        if (threadIdx.x == 0) bad = !helper_wait_d(a, ep, j, nblk, &known);
-        if (named_bar_or(GS_BAR_C, GS_C, bad)) return;
         const int buf = j & 1;
         if (threadIdx.x < GS_B) {
             const int gc = j * GS_B + threadIdx.x;
-            const float2 v = gc < n ? __ldcg(&a.delta[gc]) : make_float2(0.f, 0.f);
-            S->vh[buf][threadIdx.x] = v.x;
-            S->vl[buf][threadIdx.x] = v.y;
+            if (!have) bad = gc < n && !gs_wait(&a.delta[gc], ep, next, st);
+            S->vh[buf][threadIdx.x] = next.h;
+            S->vl[buf][threadIdx.x] = next.l;
+            const int gn = gc + GS_B;
+            next = F2{0.f, 0.f};
+            have = j + 1 < jmax && (gn >= n || gs_get(&a.delta[gn], ep, next));
         }
+        if (named_bar_or(GS_BAR_C, GS_C, bad)) return;
 #pragma unroll
         for (int m = 0; m < GS_KMAX; m++) {
             if (m >= K || j >= Iown[m] - GS_W) continue;
@@ -583,7 +580,6 @@ __global__ void __launch_bounds__(GS_T, 1) gs_trsv_kernel(const GsArgs a, cudaGr
             mbar_init(&S.full[i], 1);
             mbar_init(&S.empty[i], GS_C / 32);
         }
-        for (int i = 0; i < GS_PUB; i++) mbar_init(&S.pub[i], GS_C / 32);
         for (int i = 0; i < GS_UB; i++) {
             mbar_init(&S.uready[i], 1);
             mbar_init(&S.ufree[i], GS_C / 32);
@@ -592,11 +588,9 @@ __global__ void __launch_bounds__(GS_T, 1) gs_trsv_kernel(const GsArgs a, cudaGr
     }
     __syncthreads();
     if (threadIdx.x >= GS_C + 32) {
-        if (chain) gs_fetch_u(a, ep, nblk, &S);
+        if (chain) gs_fetch_u(a, ep, nblk, &S, (threadIdx.x - GS_C - 32) / 32);
     } else if (threadIdx.x >= GS_C) {
-        const int lane = threadIdx.x & 31;
-        if (lane == 0) gs_produce(a, nblk, &S, ring, chain);
-        else if (lane == 1 && chain) gs_publish(a, ep, nblk, &S);
+        if ((threadIdx.x & 31) == 0) gs_produce(a, nblk, &S, ring, chain);
     } else if (chain) {
         gs_chain(a, ep, nblk, &S, ring);
     } else {
@@ -612,8 +606,9 @@ __global__ void __launch_bounds__(GS_T, 1) gs_trsv_kernel(const GsArgs a, cudaGr
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x)
     {
-        const float2 d = __ldcg(&a.delta[i]);
-        a.x[i] += (double)d.x + (double)d.y;
+        F2 d;
+        gs_get(&a.delta[i], ep, d);
+        a.x[i] += (double)d.h + (double)d.l;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) set_cond(st, h_loop, 1u);
 }

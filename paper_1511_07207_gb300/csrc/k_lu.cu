@@ -83,21 +83,14 @@ __device__ __forceinline__ Cand warp_better(Cand c) {
     return c;
 }
 
-// What the CTAs tell each other travels as 16-byte words (a value, an index and
-// the step + 1), written and read whole: a word with the expected step
-// carries its own data, so no fence separates data from a flag.
+// What the CTAs tell each other travels as 16-byte words: a value, an index and
+// the step + 1.
 __device__ __forceinline__ void st_word(LuWord *p, long long v, int i, unsigned seq) {
-    const unsigned long long lo = (unsigned long long)v, hi = ((unsigned long long)seq << 32) | (unsigned)i;
-    asm volatile("{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}" ::"l"(p),
-                 "l"(lo), "l"(hi)
-                 : "memory");
+    st_word128(p, (unsigned long long)v, ((unsigned long long)seq << 32) | (unsigned)i);
 }
 __device__ __forceinline__ unsigned ld_word(const LuWord *p, long long &v, int &i) {
     unsigned long long lo, hi;
-    asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
-                 : "=l"(lo), "=l"(hi)
-                 : "l"(p)
-                 : "memory");
+    ld_word128(p, lo, hi);
     v = (long long)lo;
     i = (int)(unsigned)hi;
     return (unsigned)(hi >> 32);

@@ -366,7 +366,7 @@ struct F64Layout {
     double *rh, *vv, *s, *t;   // BiCGSTAB
     float *Ahi, *Alo;    // the FP32 pair of A (double-single products)
     float *Thi, *Tlo;    // Gauss-Seidel: inverses of the 64 x 64 diagonal blocks (FP32 pairs)
-    unsigned *gflags;    // Gauss-Seidel: 2 x nblk publication flags
+    GsWord *gwords;      // Gauss-Seidel: the entries of d and of u, npad each
     void *gmaps;         // Gauss-Seidel: 4 tensor maps (pair of A, pair of the T_I^-1)
     float *gpanel;       // Gauss-Seidel: the chain CTA's M_{I,w} = T_I^-1 A_{I,I-w}, one contiguous panel
     long long npad, ldv, lda_stage, ld32;
@@ -398,7 +398,7 @@ F64Layout f64_layout(void *base, int n, int m, bool gmres, bool stageA, bool spl
     L.nblk = (std::max(n, 1) + 63) / 64;
     L.Thi = gs ? cv.take<float>((size_t)L.nblk * 64 * 64) : nullptr;
     L.Tlo = gs ? cv.take<float>((size_t)L.nblk * 64 * 64) : nullptr;
-    L.gflags = gs ? cv.take<unsigned>((size_t)2 * L.nblk) : nullptr;
+    L.gwords = gs ? cv.take<GsWord>((size_t)2 * L.npad) : nullptr;
     L.gmaps = gs ? static_cast<void *>(cv.take<CUtensorMap>(4)) : nullptr;
     if (gs) {
         const GsKernels G = gs_kernels();
@@ -630,12 +630,10 @@ static int build_gs_graph(ls_ctx *c, const Vecs &v, const F64Layout &L, const Ge
         g.n = v.n;
         g.r = v.r;
         g.x = v.x;
-        g.delta = reinterpret_cast<float2 *>(v.p);   // n FP32 pairs in an n-double vector
-        g.u = reinterpret_cast<float2 *>(v.q);
+        g.delta = L.gwords;
+        g.u = L.gwords + L.npad;
         g.tmaps = static_cast<const CUtensorMap *>(L.gmaps);
         g.panel = L.gpanel;
-        g.flagD = L.gflags;
-        g.flagU = L.gflags + L.nblk;
         g.bar = v.bar;
         g.st = v.st;
         const GsKernels G = gs_kernels();
@@ -802,12 +800,12 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
         const int g = std::min((n + c->K.block - 1) / c->K.block, 4 * c->num_sms);
         e = cudaLaunchKernel(c->K.ja_diag, dim3(g), dim3(c->K.block), args, 0, c->stream);
     }
-    if (e == cudaSuccess && gs) {   // flags zeroed; T_I^-1 of the diagonal blocks (A may be borrowed per call)
+    if (e == cudaSuccess && gs) {   // words zeroed (no sweep's number); T_I^-1 of the diagonal blocks (A may be borrowed per call)
         alignas(64) CUtensorMap maps[4];
         if (!gs_encode_maps(maps, L.Ahi, L.Alo, n, L.ld32, L.Thi, L.Tlo, L.nblk)) return LS_ERR_UNSUPPORTED;
         e = cudaMemcpyAsync(L.gmaps, maps, sizeof(maps), cudaMemcpyHostToDevice, c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);   // maps is on this stack frame
-        if (e == cudaSuccess) e = cudaMemsetAsync(L.gflags, 0, sizeof(unsigned) * 2 * L.nblk, c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(L.gwords, 0, sizeof(GsWord) * 2 * L.npad, c->stream);
         const GsKernels G = gs_kernels();
         int nn = n;
         long long la = ldad;

@@ -211,6 +211,21 @@ __device__ __forceinline__ unsigned grid_arrive(GridBar *b) {
 }
 __device__ __forceinline__ bool grid_sync(GridBar *b, State *st) { return grid_wait(b, grid_arrive(b), st); }
 
+// ---- 16-byte words between CTAs -------------------------------------------------------
+// Written and read whole: a word that carries the expected tag carries its own
+// data, so no fence and no flag separate data from its announcement.
+__device__ __forceinline__ void st_word128(void *p, unsigned long long lo, unsigned long long hi) {
+    asm volatile("{\n\t.reg .b128 q;\n\tmov.b128 q, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], q;\n\t}" ::"l"(p),
+                 "l"(lo), "l"(hi)
+                 : "memory");
+}
+__device__ __forceinline__ void ld_word128(const void *p, unsigned long long &lo, unsigned long long &hi) {
+    asm volatile("{\n\t.reg .b128 q;\n\tld.relaxed.gpu.global.b128 q, [%2];\n\tmov.b128 {%0, %1}, q;\n\t}"
+                 : "=l"(lo), "=l"(hi)
+                 : "l"(p)
+                 : "memory");
+}
+
 // ---- grid-stride ranges --------------------------------------------------------------
 // Balanced contiguous range [lo, hi) of 0..n for block `b` of `nb`.
 __device__ __forceinline__ void block_range(long long n, int b, int nb, long long &lo,

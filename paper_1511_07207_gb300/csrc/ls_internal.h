@@ -231,14 +231,17 @@ MixedKernels mixed_kernels();
 
 // ---- Krylov launchers (k_krylov.cu) -----------------------------------------------
 // ---- Gauss-Seidel triangular solve (k_gs.cu) -----------------------------------------
+struct alignas(16) GsWord {      // an entry of d or u between CTAs: the FP32 pair, the sweep's number
+    float h, l;
+    unsigned ep, pad_;
+};
 struct GsArgs {
     int n;
     const double *r;         // b - A x(k), from the residual GEMV
     double *x;               // x(k) -> x(k+1) = x(k) + d
-    float2 *delta, *u;       // d, and u_I = T_I^-1 (r_I - sum_{j < I - W} A_Ij d_j), as FP32 pairs
+    GsWord *delta, *u;       // d, and u_I = T_I^-1 (r_I - sum_{j < I - W} A_Ij d_j)
     const CUtensorMap *tmaps;// device: A hi, A lo (n x n), T hi, T lo (nblk*64 x 64), 32 x 64 boxes
     const float *panel;      // the chain's tiles per block, in its read order (gs_panel_kernel)
-    unsigned *flagD, *flagU; // per row block: d_I / u_I published (value = sweep number)
     GridBar *bar;            // the final x += d waits for the whole chain
     State *st;
 };
