@@ -282,7 +282,9 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
     // Equal pieces, except when there are at most as many row tiles as CTAs (up to n =
     // 4864 for the FP32 pair): then a CTA takes one whole row tile, and none of them waits to
     // add partial sums with its neighbours (2 us each time; n = 2000: half of the kernel's time).
-    const bool whole = RT <= G_;
+    // The native FP64 product is bound by the FP64 pipe and keeps the equal pieces, which
+    // use every SM.
+    const bool whole = DT != DT_F64 && RT <= G_;
     const long long t0 = whole ? (long long)min(cta, RT) * CT : tile_start(T_all, cta, G_);
     const long long t1 = whole ? (long long)min(cta + 1, RT) * CT : tile_start(T_all, cta + 1, G_);
     const int ntiles = (int)(t1 - t0);
