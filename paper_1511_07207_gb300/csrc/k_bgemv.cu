@@ -1,8 +1,8 @@
 // k_bgemv.cu -- Q = A P for an n x s block P (the block product of block CG),
 // A read once as its FP32 pair hi + lo, double-single arithmetic.
 //
-// One CTA per SM: a producer lane streams, for each of the CTA's 16-row
-// blocks and each 256-column tile, the A tile (hi and lo, the solvers' 2-D
+// One CTA per SM: a producer lane streams, for each of the CTA's 16-row x
+// 256-column tiles, the A tile (hi and lo, the solvers' 2-D
 // TMA map) and the matching 256-row chunk of P (pre-split into FP32 pairs,
 // column panels padded with zeros to a multiple of 256, one 1-D bulk copy
 // per column and part) through a ring of shared-memory stages (mbarrier
@@ -13,8 +13,10 @@
 // tile.  A thread accumulates all S columns of P for its rows in
 // double-single (two-sum of the high parts, the low parts and rounding
 // errors summed apart, as the GEMV does), and the 32 lanes of a row add
-// their sums by shuffles at the end of the row block.  Every row block
-// belongs to one CTA and is summed in column order, so results are
+// their sums by shuffles at the end of the row block.  The (row block, column
+// tile) sequence is cut into equal pieces, one per CTA (whole row blocks left up to
+// a fifth of the SMs idle in the last round: n = 8192 has 512 of them); the last
+// of the CTAs that share a row block adds their sums in CTA order, so results are
 // deterministic.  Work per element of A is 12 FP32 operations per column of
 // P: compute-bound for S >= 4 (HBM-bound below).
 #include <cuda_runtime.h>
@@ -77,6 +79,11 @@ template <int S>
 __host__ __device__ constexpr int stages() {
     return S >= 16 ? 3 : 4;
 }
+__device__ __forceinline__ long long bg_start(long long T, int c, int G) { return T * c / G; }
+__device__ __forceinline__ int bg_owner(long long t, long long T, int G) {
+    return (int)(((long long)G * (t + 1) + T - 1) / T) - 1;
+}
+
 template <int S>
 __host__ __device__ constexpr size_t stage_bytes() {
     return (size_t)2 * BG_A_B + (size_t)2 * S * BG_TC * 4;
@@ -116,6 +123,16 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
     count_launch(st);
     const int n = a.n;
     const int RB = (n + BG_TR - 1) / BG_TR, CT = (n + BG_TC - 1) / BG_TC;
+    // Equal pieces of the (row block, column tile) sequence, or whole row blocks where
+    // those leave less idle time than adding shared ones up takes: a tile is about 0.3 S
+    // us, the sums 4 (n = 2000, s = 3: 5.6 ms a solve with whole blocks, 6.1 with pieces).
+    const long long T = (long long)RB * CT;
+    const int G = gridDim.x, cta = blockIdx.x;
+    const bool whole = ((long long)((RB + G - 1) / G) * CT - T / G) * S < 16;
+    const long long t0 = whole ? bg_start(RB, cta, G) * CT : bg_start(T, cta, G);
+    const long long t1 = whole ? bg_start(RB, cta + 1, G) * CT : bg_start(T, cta + 1, G);
+    const int ntiles = (int)(t1 - t0), first_rb = (int)(t0 / CT);
+    __shared__ int ca_s, cb_s, fin_s;
     if (threadIdx.x == 0) {
         for (int i = 0; i < NST; i++) {
             mbar_init(&full[i], 1);
@@ -132,13 +149,12 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
         tmap_acquire(&M.tmap);
         tmap_acquire(&M.tmap_lo);
         int seq = 0;
-        bool go = true;
-        for (int rb = blockIdx.x; rb < RB && go; rb += gridDim.x)
-            for (int t = 0; t < CT && go; t++) {
+        int rb = first_rb, t = (int)(t0 - (long long)rb * CT);
+        {
+            for (int i = 0; i < ntiles; i++) {
                 const int sl = seq % NST;
                 if (seq >= NST && !mbar_wait(&empty[sl], ((seq / NST) - 1) & 1)) {
                     set_err(st, ERRB_TIMEOUT);
-                    go = false;
                     break;
                 }
                 unsigned char *dst = ring + (size_t)sl * SB;
@@ -151,7 +167,12 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
                     bulk_load_1d(dst + 2 * BG_A_B + (size_t)(S + j) * BG_TC * 4, a.Pl + off, BG_TC * 4, &full[sl]);
                 }
                 seq++;
+                if (++t == CT) {
+                    t = 0;
+                    rb++;
+                }
             }
+        }
         // no copy may be in flight when the CTA exits
         for (int k = seq > NST ? seq - NST : 0; k < seq; k++)
             if (!mbar_wait(&full[k % NST], (k / NST) & 1)) set_err(st, ERRB_TIMEOUT);
@@ -162,23 +183,26 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
     // warp w: rows w, w + WS, ... of the block (RPW of them); lane g: the
     // 4-column chunks g and g + 32 of each tile
     const int w = threadIdx.x >> 5, g = threadIdx.x & 31;
-    int seq = 0;
     // one row per warp (S <= 8): the two column chunks accumulate apart (two
     // independent chains per column of P), added at the end of the row block
     constexpr int NA = RPW == 1 ? 2 : 1;
-    for (int rb = blockIdx.x; rb < RB; rb += gridDim.x) {
-        F2 acc[RPW * NA][S];
+    F2 acc[RPW * NA][S];
 #pragma unroll
-        for (int q = 0; q < RPW * NA; q++)
+    for (int q = 0; q < RPW * NA; q++)
 #pragma unroll
-            for (int j = 0; j < S; j++) acc[q][j] = {0.f, 0.f};
-        for (int t = 0; t < CT; t++) {
-            const int sl = seq % NST;
-            const bool ok = mbar_wait(&full[sl], (seq / NST) & 1);
-            if (!__all_sync(0xffffffffu, ok)) {   // the warp leaves together
-                set_err(st, ERRB_TIMEOUT);
-                return;
-            }
+        for (int j = 0; j < S; j++) acc[q][j] = {0.f, 0.f};
+    int rb = first_rb, t = (int)(t0 - (long long)rb * CT);
+    bool ok = true;
+    for (int seq = 0; seq < ntiles; seq++) {
+        const int sl = seq % NST;
+        // on a timeout the warp stops waiting and computing but keeps walking
+        // its tiles, so it still meets the others where a row block is shared
+        ok = ok && mbar_wait(&full[sl], (seq / NST) & 1);
+        if (!__all_sync(0xffffffffu, ok)) {
+            set_err(st, ERRB_TIMEOUT);
+            ok = false;
+        }
+        if (ok) {
             const unsigned char *base = ring + (size_t)sl * SB;
             const float *Ah = reinterpret_cast<const float *>(base);
             const float *Al = reinterpret_cast<const float *>(base + BG_A_B);
@@ -207,35 +231,84 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
                     }
                 }
             }
-            __syncwarp();
-            if (g == 0) mbar_arrive(&empty[sl]);
-            seq++;
         }
-        if constexpr (NA == 2)
+        __syncwarp();
+        if (g == 0) mbar_arrive(&empty[sl]);
+        if (t == CT - 1 || seq == ntiles - 1) {
+            // this CTA's share of row block rb
+            if constexpr (NA == 2)
 #pragma unroll
-            for (int j = 0; j < S; j++) acc[0][j] = f2_add(acc[0][j], acc[1][j]);
-        // the 32 lanes of a row
+                for (int j = 0; j < S; j++) acc[0][j] = f2_add(acc[0][j], acc[1][j]);
+            // the 32 lanes of a row
 #pragma unroll
-        for (int q = 0; q < RPW; q++)
+            for (int q = 0; q < RPW; q++)
 #pragma unroll
-            for (int j = 0; j < S; j++) {
+                for (int j = 0; j < S; j++) {
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    F2 b;
-                    b.h = __shfl_xor_sync(0xffffffffu, acc[q][j].h, o);
-                    b.l = __shfl_xor_sync(0xffffffffu, acc[q][j].l, o);
-                    acc[q][j] = f2_add(acc[q][j], b);
+                    for (int o = 1; o < 32; o <<= 1) {
+                        F2 b;
+                        b.h = __shfl_xor_sync(0xffffffffu, acc[q][j].h, o);
+                        b.l = __shfl_xor_sync(0xffffffffu, acc[q][j].l, o);
+                        acc[q][j] = f2_add(acc[q][j], b);
+                    }
+                }
+            const long long rfirst = (long long)rb * CT;
+            if (t0 <= rfirst && rfirst + CT <= t1) {
+                if (g == 0)
+#pragma unroll
+                    for (int q = 0; q < RPW; q++) {
+                        const int row = rb * BG_TR + w + WS * q;
+                        if (row < n)
+#pragma unroll
+                            for (int j = 0; j < S; j++)
+                                if (j < a.s) a.Q[(long long)j * a.ldq + row] = (double)acc[q][j].h + (double)acc[q][j].l;
+                    }
+            } else {
+                // shared with neighbouring CTAs: publish the partial sums; the last of
+                // the sharing CTAs adds them in CTA order
+                double *fix = a.scr->fix + (size_t)(2 * blockIdx.x + (rb == first_rb ? 0 : 1)) * BG_TR * S;
+                if (g == 0) {
+#pragma unroll
+                    for (int q = 0; q < RPW; q++)
+#pragma unroll
+                        for (int j = 0; j < S; j++)
+                            fix[(w + WS * q) * S + j] = (double)acc[q][j].h + (double)acc[q][j].l;
+                    __threadfence();
+                }
+                named_bar(1, BG_C);
+                if (threadIdx.x == 0) {
+                    ca_s = bg_owner(rfirst, T, gridDim.x);
+                    cb_s = bg_owner(rfirst + CT - 1, T, gridDim.x);
+                    int ncov = 0;
+                    for (int c = ca_s; c <= cb_s; c++) ncov += bg_start(T, c, gridDim.x) < bg_start(T, c + 1, gridDim.x);
+                    fin_s = atomicAdd(&a.scr->bticket[ca_s], 1u) == (unsigned)ncov - 1;
+                    if (fin_s) atomicExch(&a.scr->bticket[ca_s], 0u);
+                }
+                named_bar(1, BG_C);
+                if (fin_s) {
+                    __threadfence();
+                    for (int e = threadIdx.x; e < BG_TR * S; e += BG_C) {
+                        const int row = rb * BG_TR + e / S, j = e % S;
+                        double sum = 0.0;
+                        for (int c = ca_s; c <= cb_s; c++) {
+                            const long long a0 = bg_start(T, c, gridDim.x);
+                            if (bg_start(T, c + 1, gridDim.x) <= a0) continue;   // empty CTA
+                            const int slot = rb == (int)(a0 / CT) ? 0 : 1;
+                            sum += __ldcg(&a.scr->fix[(size_t)(2 * c + slot) * BG_TR * S + e]);
+                        }
+                        if (row < n && j < a.s) a.Q[(long long)j * a.ldq + row] = sum;
+                    }
                 }
             }
-        if (g == 0)
 #pragma unroll
-            for (int q = 0; q < RPW; q++) {
-                const int row = rb * BG_TR + w + WS * q;
-                if (row < n)
+            for (int q = 0; q < RPW * NA; q++)
 #pragma unroll
-                    for (int j = 0; j < S; j++)
-                        if (j < a.s) a.Q[(long long)j * a.ldq + row] = (double)acc[q][j].h + (double)acc[q][j].l;
-            }
+                for (int j = 0; j < S; j++) acc[q][j] = {0.f, 0.f};
+        }
+        if (++t == CT) {
+            t = 0;
+            rb++;
+        }
     }
 }
 

@@ -109,6 +109,7 @@ int build_bcg_graph(ls_ctx *c, const BcgVecs &v, const BcgLayout &L, const GemvL
         ba.Q = v.Q;
         ba.ldq = v.ld;
         ba.st = v.st;
+        ba.scr = c->scr;
         const MatDesc *pA = c->dA;
         void *bargs[] = {&pA, &ba};
         inner.kernel(BL.func, BL.grid, BL.block, BL.smem, bargs, false);

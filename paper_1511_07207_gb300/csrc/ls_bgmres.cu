@@ -100,6 +100,7 @@ int build_bgm_graph(ls_ctx *c, const BgmVecs &v, const BgmLayout &L, int x0_give
         ba.Q = v.V;
         ba.ldq = v.ld;
         ba.st = v.st;
+        ba.scr = c->scr;
         const MatDesc *pA = c->dA;
         void *bargs[] = {&pA, &ba};
         outer.kernel(BL.func, BL.grid, BL.block, BL.smem, bargs, false);
@@ -129,6 +130,7 @@ int build_bgm_graph(ls_ctx *c, const BgmVecs &v, const BgmLayout &L, int x0_give
         ba.Q = v.W;
         ba.ldq = v.ld;
         ba.st = v.st;
+        ba.scr = c->scr;
         const MatDesc *pA = c->dA;
         void *bargs[] = {&pA, &ba};
         inner.kernel(BL.func, BL.grid, BL.block, BL.smem, bargs, false);

@@ -400,6 +400,7 @@ struct BgemvArgs {
     double *Q;                    // column-major n x s, column stride ldq
     long long ldq;
     State *st;
+    GemvScratch *scr;             // partial sums and tickets of shared row blocks
 };
 struct BgemvLaunch {
     void *func, *split;           // the product (takes the A descriptor) and the P splitter
