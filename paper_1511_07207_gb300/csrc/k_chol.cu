@@ -23,8 +23,8 @@
 //   the integer pipes and the difference on the FP64 pipe (ls_rank.cuh).
 // chol_backsolve_kernel (cooperative): L^T x = y by blocks of 64 rows from
 //   the bottom: CTA 0 solves the diagonal block (one warp), then every CTA
-//   subtracts the block's contribution l_ji x_j from the rows above it (a
-//   thread a row, reading the block's rows of L, which are contiguous).
+//   subtracts the block's contribution l_ji x_j from the rows above it (32
+//   rows a CTA, reading the block's rows of L, which are contiguous).
 // So L and y are bit for bit those of the plain column factorization and
 // forward substitution; x differs from a scalar back substitution by the
 // order of its sums.
@@ -43,7 +43,7 @@ constexpr int CT = 512;            // threads per CTA of the cooperative kernels
 constexpr int CW = CT / 32;
 constexpr int CH_NB = 32;          // panel width
 constexpr int CP_T = 256;           // threads of a panel CTA
-constexpr int CB = 64;             // rows per back-substitution block
+constexpr int CB = BACK_B;         // rows per back-substitution block
 static_assert(CH_NB == RANK_NB, "panel width");
 }  // namespace
 
@@ -157,7 +157,8 @@ __global__ void __launch_bounds__(RANK_T, 4) chol_trail_kernel(CholArgs a, int k
 }
 
 __global__ void __launch_bounds__(CT, 1) chol_backsolve_kernel(CholArgs a) {
-    __shared__ double s[CB], xs[CB];
+    __shared__ double s[CB], xs[CB], T[CB][CB + 1];
+    __shared__ double part[CW][33];
     State *st = a.st;
     count_launch(st);
     const int n = a.n;
@@ -168,26 +169,39 @@ __global__ void __launch_bounds__(CT, 1) chol_backsolve_kernel(CholArgs a) {
     double *y = a.y;                             // a copy of row n: y, then the updated right sides
     for (int r1 = n; r1 > 0; r1 -= CB) {
         const int r0 = r1 > CB ? r1 - CB : 0, nb = r1 - r0;
-        if (blockIdx.x == 0 && warp == 0) {
-            // the diagonal block, column oriented: x_i = s_i / l_ii, then s_r -= l_ir x_i (r < i)
-            for (int r = lane; r < nb; r += 32) s[r] = __ldcg(&y[r0 + r]);
-            __syncwarp();
-            for (int i = nb - 1; i >= 0; i--) {
-                const double xi = s[i] / W[(long long)(r0 + i) * ld + r0 + i];
-                __syncwarp();
-                for (int r = lane; r < i; r += 32) s[r] -= W[(long long)(r0 + i) * ld + r0 + r] * xi;
-                if (lane == 0) xs[i] = xi;
-                __syncwarp();
+        if (blockIdx.x == 0) {                   // the diagonal block, transposed: t_rc = l_cr
+            for (int e = threadIdx.x; e < CB * CB; e += CT) {
+                const int c = e / CB, r = e % CB;
+                T[r][c] = r <= c && c < nb ? W[(long long)(r0 + c) * ld + r0 + r] : 0.0;
             }
-            for (int r = lane; r < nb; r += 32) a.x[r0 + r] = xs[r];
+            for (int r = threadIdx.x; r < nb; r += CT) s[r] = __ldcg(&y[r0 + r]);
+            __syncthreads();
+            if (warp == 0) back_solve_block(nb, T, s, xs);
+            __syncthreads();
+            for (int r = threadIdx.x; r < nb; r += CT) a.x[r0 + r] = xs[r];
         }
         if (!grid_sync(a.bar, st)) return;
-        // rows above the block: y_i -= sum_{j in block} l_ji x_j, a thread a row i
-        // (the block's rows of L are contiguous in i)
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < r0; i += gridDim.x * blockDim.x) {
+        // rows above the block: y_i -= sum_{j in block} l_ji x_j.  A CTA takes 32 rows i (the
+        // block's rows of L are contiguous in i), a warp four of the block's rows;
+        // the warps' sums are added pairwise.
+        for (int i0 = blockIdx.x * 32; i0 < r0; i0 += gridDim.x * 32) {
+            const int i = i0 + lane;
             double acc = 0.0;
-            for (int jj = 0; jj < nb; jj++) acc += W[(long long)(r0 + jj) * ld + i] * __ldcg(&a.x[r0 + jj]);
-            y[i] = __ldcg(&y[i]) - acc;
+            if (i < r0) {
+#pragma unroll
+                for (int u = 0; u < CB / CW; u++) {
+                    const int jj = warp * (CB / CW) + u;
+                    if (jj < nb) acc += W[(long long)(r0 + jj) * ld + i] * __ldcg(&a.x[r0 + jj]);
+                }
+            }
+            part[warp][lane] = acc;
+            __syncthreads();
+            for (int o = CW / 2; o > 0; o >>= 1) {
+                if (warp < o) part[warp][lane] += part[warp + o][lane];
+                __syncthreads();
+            }
+            if (warp == 0 && i < r0) y[i] = __ldcg(&y[i]) - part[0][lane];
+            __syncthreads();
         }
         if (!grid_sync(a.bar, st)) return;
     }

@@ -52,7 +52,7 @@ constexpr int LU_NB = 32;          // panel width
 constexpr int LW = LT / 32;        // warps per CTA
 constexpr int FT = 256, FW = FT / 32;   // threads and warps of a panel CTA
 constexpr int SLOTS = 5;           // candidates a lane fetches at a time (152 CTAs)
-constexpr int LB = 64;             // rows per back-substitution block
+constexpr int LB = BACK_B;         // rows per back-substitution block
 static_assert(LU_NB == RANK_NB, "panel width");
 
 // A pivot candidate: |a| as its bit pattern, which orders as the value does
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(RANK_T, 4) lu_trail_kernel(LuArgs a, int k0) {
 }
 
 __global__ void __launch_bounds__(LT, 1) lu_backsolve_kernel(LuArgs a) {
-    __shared__ double s[LB], xs[LB];
+    __shared__ double s[LB], xs[LB], T[LB][LB + 1];
     State *st = a.st;
     count_launch(st);
     const int n = a.n;
@@ -406,18 +406,16 @@ __global__ void __launch_bounds__(LT, 1) lu_backsolve_kernel(LuArgs a) {
 #define Y(i) W[(long long)(i) * ld + n]   // y = L^-1 P b, column n of the working matrix
     for (int r1 = n; r1 > 0; r1 -= LB) {
         const int r0 = r1 > LB ? r1 - LB : 0, nb = r1 - r0;
-        if (blockIdx.x == 0 && warp == 0) {
-            // the diagonal block, column oriented: x_i = s_i / u_ii, then s_r -= u_ri x_i
-            for (int r = lane; r < nb; r += 32) s[r] = __ldcg(&Y(r0 + r));
-            __syncwarp();
-            for (int i = nb - 1; i >= 0; i--) {
-                const double xi = s[i] / W[(long long)(r0 + i) * ld + r0 + i];
-                __syncwarp();
-                for (int r = lane; r < i; r += 32) s[r] -= W[(long long)(r0 + r) * ld + r0 + i] * xi;
-                if (lane == 0) xs[i] = xi;
-                __syncwarp();
+        if (blockIdx.x == 0) {   // the diagonal block
+            for (int e = threadIdx.x; e < LB * LB; e += LT) {
+                const int r = e / LB, c = e % LB;
+                T[r][c] = r < nb && c < nb ? W[(long long)(r0 + r) * ld + r0 + c] : 0.0;
             }
-            for (int r = lane; r < nb; r += 32) a.x[r0 + r] = xs[r];
+            for (int r = threadIdx.x; r < nb; r += LT) s[r] = __ldcg(&Y(r0 + r));
+            __syncthreads();
+            if (warp == 0) back_solve_block(nb, T, s, xs);
+            __syncthreads();
+            for (int r = threadIdx.x; r < nb; r += LT) a.x[r0 + r] = xs[r];
         }
         if (!grid_sync(a.bar, st)) return;
         // rows above the block: y_i -= sum_{j in block} u_ij x_j (a warp a row)

@@ -118,4 +118,39 @@ __device__ __forceinline__ void rank_tile(double (&acc)[RANK_R][RANK_R], const O
     }
 }
 
+// ---- back substitution: one diagonal block -----------------------------------------------
+constexpr int BACK_B = 64;           // rows of a block
+
+// One warp: T x = s for the upper triangular nb x nb block T (shared memory), column
+// oriented: x_i = s_i / t_ii, then s_r -= t_ri x_i for r < i.  The chain is 64 of those, so
+// the block is in shared memory, the reciprocals of its diagonal are formed
+// at once and a quotient from one is corrected by its remainder (three dependent FP64
+// instructions instead of a division's ten).
+__device__ __forceinline__ void back_solve_block(int nb, const double (*T)[BACK_B + 1], const double *s, double *x) {
+    const int lane = threadIdx.x & 31;
+    double sv[2], d[2], inv[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+        const int r = lane + 32 * h;
+        sv[h] = r < nb ? s[r] : 0.0;
+        d[h] = r < nb ? T[r][r] : 1.0;
+        inv[h] = 1.0 / d[h];
+    }
+    for (int i = nb - 1; i >= 0; i--) {
+        const int h = i >> 5, src = i & 31;
+        const double si = __shfl_sync(0xffffffffu, h ? sv[1] : sv[0], src);
+        const double di = __shfl_sync(0xffffffffu, h ? d[1] : d[0], src);
+        const double ri = __shfl_sync(0xffffffffu, h ? inv[1] : inv[0], src);
+        const double t0 = T[lane][i], t1 = T[lane + 32][i];
+        double xi = si * ri;
+        xi = fma(ri, fma(-di, xi, si), xi);
+        // a diagonal entry or a quotient near the ends of the range: the division itself
+        const int er = (__double2hiint(ri) >> 20) & 0x7FF, ex = (__double2hiint(xi) >> 20) & 0x7FF;
+        if (er < 64 || er > 1982 || ex < 64 || ex > 1982) xi = si / di;
+        if (lane < i) sv[0] -= t0 * xi;
+        if (lane + 32 < i) sv[1] -= t1 * xi;
+        if (lane == 0) x[i] = xi;
+    }
+}
+
 }  // namespace lsi
