@@ -2,8 +2,7 @@
 // A read once as its FP32 pair hi + lo, double-single arithmetic.
 //
 // One CTA per SM: a producer lane streams, for each of the CTA's 16-row x
-// 256-column tiles, the A tile (hi and lo, the solvers' 2-D
-// TMA map) and the matching 256-row chunk of P (pre-split into FP32 pairs,
+// 256-column tiles, the A tile (hi and lo, the solvers' 2-D TMA map) and the matching 256-row chunk of P (pre-split into FP32 pairs,
 // column panels padded with zeros to a multiple of 256, one 1-D bulk copy
 // per column and part) through a ring of shared-memory stages (mbarrier
 // full/empty).  Consumer warps: for S <= 8 sixteen warps, warp w owning row
@@ -15,9 +14,9 @@
 // errors summed apart, as the GEMV does), and the 32 lanes of a row add
 // their sums by shuffles at the end of the row block.  The (row block, column
 // tile) sequence is cut into equal pieces, one per CTA (whole row blocks left up to
-// a fifth of the SMs idle in the last round: n = 8192 has 512 of them); the last
-// of the CTAs that share a row block adds their sums in CTA order, so results are
-// deterministic.  Work per element of A is 12 FP32 operations per column of
+// a fifth of the SMs idle in the last round: n = 8192 has 512 of them; S = 16 and
+// small products keep them); the last of the CTAs that share a row block adds
+// their sums in CTA order, so results are deterministic.  Work per element of A is 12 FP32 operations per column of
 // P: compute-bound for S >= 4 (HBM-bound below).
 #include <cuda_runtime.h>
 
@@ -66,6 +65,12 @@ template <int S>
 __host__ __device__ constexpr int bg_rows_per_warp() {
     return S <= 8 ? 1 : 2;
 }
+// Accumulators a column: one row per warp (S <= 8) keeps the two column chunks apart (two
+// independent chains per column of P), added at the end of the row block.
+template <int S>
+__host__ __device__ constexpr int bg_accs() {
+    return 2;
+}
 template <int S>
 __host__ __device__ constexpr int bg_consumers() {
     return 32 * 16 / bg_rows_per_warp<S>();
@@ -87,6 +92,39 @@ __device__ __forceinline__ int bg_owner(long long t, long long T, int G) {
 template <int S>
 __host__ __device__ constexpr size_t stage_bytes() {
     return (size_t)2 * BG_A_B + (size_t)2 * S * BG_TC * 4;
+}
+
+// A warp's share of one 16 x 256 tile in a ring stage: rows w, w + WS, ..., lane g's 4-column chunks.
+template <int S>
+__device__ __forceinline__ void bg_tile(F2 (&acc)[bg_accs<S>()][S], const unsigned char *base, int w, int g) {
+    constexpr int RPW = bg_rows_per_warp<S>(), WS = 16 / RPW, NA = bg_accs<S>() / RPW;
+    const float *Ah = reinterpret_cast<const float *>(base);
+    const float *Al = reinterpret_cast<const float *>(base + BG_A_B);
+    const float *Xh = reinterpret_cast<const float *>(base + 2 * BG_A_B);
+    const float *Xl = Xh + S * BG_TC;
+#pragma unroll
+    for (int k = 0; k < 2; k++) {
+        const int c0 = (k * 32 + g) * 4;
+        float4 ah[RPW], al[RPW];
+#pragma unroll
+        for (int q = 0; q < RPW; q++) {
+            ah[q] = *reinterpret_cast<const float4 *>(Ah + (w + WS * q) * BG_TC + c0);
+            al[q] = *reinterpret_cast<const float4 *>(Al + (w + WS * q) * BG_TC + c0);
+        }
+#pragma unroll
+        for (int j = 0; j < S; j++) {
+            const float4 xh = *reinterpret_cast<const float4 *>(Xh + j * BG_TC + c0);
+            const float4 xl = *reinterpret_cast<const float4 *>(Xl + j * BG_TC + c0);
+#pragma unroll
+            for (int q = 0; q < RPW; q++) {
+                F2 &a2 = acc[NA == 2 ? k : q][j];
+                f2_mac(a2, ah[q].x, al[q].x, xh.x, xl.x);
+                f2_mac(a2, ah[q].y, al[q].y, xh.y, xl.y);
+                f2_mac(a2, ah[q].z, al[q].z, xh.z, xl.z);
+                f2_mac(a2, ah[q].w, al[q].w, xh.w, xl.w);
+            }
+        }
+    }
 }
 
 }  // namespace
@@ -123,15 +161,17 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
     count_launch(st);
     const int n = a.n;
     const int RB = (n + BG_TR - 1) / BG_TR, CT = (n + BG_TC - 1) / BG_TC;
-    // Equal pieces of the (row block, column tile) sequence, or whole row blocks where
-    // those leave less idle time than adding shared ones up takes: a tile is about 0.3 S
-    // us, the sums 4 (n = 2000, s = 3: 5.6 ms a solve with whole blocks, 6.1 with pieces).
+    // Equal pieces of the (row block, column tile) sequence, or whole row blocks (CTA c: c, c + G,
+    // ...) where those leave less idle time than adding shared ones up takes: a tile is about
+    // 0.3 S us, the sums 4 (n = 2000, s = 3: 5.6 ms a solve with whole blocks, 6.1 with pieces).
+    // Sixteen columns keep whole row blocks, by measurement (block GMRES, s = 16: n = 8192
+    // 40.4 ms a solve with whole blocks, 42.1 with pieces; n = 6000, s = 12 24.7 and 26.5).
     const long long T = (long long)RB * CT;
     const int G = gridDim.x, cta = blockIdx.x;
-    const bool whole = ((long long)((RB + G - 1) / G) * CT - T / G) * S < 16;
-    const long long t0 = whole ? bg_start(RB, cta, G) * CT : bg_start(T, cta, G);
-    const long long t1 = whole ? bg_start(RB, cta + 1, G) * CT : bg_start(T, cta + 1, G);
-    const int ntiles = (int)(t1 - t0), first_rb = (int)(t0 / CT);
+    const bool whole = S == 16 || ((long long)((RB + G - 1) / G) * CT - T / G) * S < 16;
+    const long long t0 = whole ? (long long)cta * CT : bg_start(T, cta, G);
+    const int ntiles = whole ? (cta < RB ? (RB - cta + G - 1) / G * CT : 0) : (int)(bg_start(T, cta + 1, G) - t0);
+    const int first_rb = (int)(t0 / CT), rb_step = whole ? G : 1;
     __shared__ int ca_s, cb_s, fin_s;
     if (threadIdx.x == 0) {
         for (int i = 0; i < NST; i++) {
@@ -150,27 +190,24 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
         tmap_acquire(&M.tmap_lo);
         int seq = 0;
         int rb = first_rb, t = (int)(t0 - (long long)rb * CT);
-        {
-            for (int i = 0; i < ntiles; i++) {
-                const int sl = seq % NST;
-                if (seq >= NST && !mbar_wait(&empty[sl], ((seq / NST) - 1) & 1)) {
-                    set_err(st, ERRB_TIMEOUT);
-                    break;
-                }
-                unsigned char *dst = ring + (size_t)sl * SB;
-                mbar_arrive_expect_tx(&full[sl], (unsigned)SB);
-                tma_load_2d(dst, &M.tmap, t * BG_TC, rb * BG_TR, &full[sl]);
-                tma_load_2d(dst + BG_A_B, &M.tmap_lo, t * BG_TC, rb * BG_TR, &full[sl]);
-                for (int j = 0; j < S; j++) {
-                    const long long off = (long long)j * a.ldp + (long long)t * BG_TC;
-                    bulk_load_1d(dst + 2 * BG_A_B + (size_t)j * BG_TC * 4, a.Ph + off, BG_TC * 4, &full[sl]);
-                    bulk_load_1d(dst + 2 * BG_A_B + (size_t)(S + j) * BG_TC * 4, a.Pl + off, BG_TC * 4, &full[sl]);
-                }
-                seq++;
-                if (++t == CT) {
-                    t = 0;
-                    rb++;
-                }
+        for (; seq < ntiles; seq++) {
+            const int sl = seq % NST;
+            if (seq >= NST && !mbar_wait(&empty[sl], ((seq / NST) - 1) & 1)) {
+                set_err(st, ERRB_TIMEOUT);
+                break;
+            }
+            unsigned char *dst = ring + (size_t)sl * SB;
+            mbar_arrive_expect_tx(&full[sl], (unsigned)SB);
+            tma_load_2d(dst, &M.tmap, t * BG_TC, rb * BG_TR, &full[sl]);
+            tma_load_2d(dst + BG_A_B, &M.tmap_lo, t * BG_TC, rb * BG_TR, &full[sl]);
+            for (int j = 0; j < S; j++) {
+                const long long off = (long long)j * a.ldp + (long long)t * BG_TC;
+                bulk_load_1d(dst + 2 * BG_A_B + (size_t)j * BG_TC * 4, a.Ph + off, BG_TC * 4, &full[sl]);
+                bulk_load_1d(dst + 2 * BG_A_B + (size_t)(S + j) * BG_TC * 4, a.Pl + off, BG_TC * 4, &full[sl]);
+            }
+            if (++t == CT) {
+                t = 0;
+                rb += rb_step;
             }
         }
         // no copy may be in flight when the CTA exits
@@ -183,131 +220,93 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
     // warp w: rows w, w + WS, ... of the block (RPW of them); lane g: the
     // 4-column chunks g and g + 32 of each tile
     const int w = threadIdx.x >> 5, g = threadIdx.x & 31;
-    // one row per warp (S <= 8): the two column chunks accumulate apart (two
-    // independent chains per column of P), added at the end of the row block
-    constexpr int NA = RPW == 1 ? 2 : 1;
-    F2 acc[RPW * NA][S];
-#pragma unroll
-    for (int q = 0; q < RPW * NA; q++)
-#pragma unroll
-        for (int j = 0; j < S; j++) acc[q][j] = {0.f, 0.f};
-    int rb = first_rb, t = (int)(t0 - (long long)rb * CT);
+    constexpr int NA = bg_accs<S>() / RPW;
+    int seq = 0;
     bool ok = true;
-    for (int seq = 0; seq < ntiles; seq++) {
-        const int sl = seq % NST;
-        // on a timeout the warp stops waiting and computing but keeps walking
-        // its tiles, so it still meets the others where a row block is shared
-        ok = ok && mbar_wait(&full[sl], (seq / NST) & 1);
-        if (!__all_sync(0xffffffffu, ok)) {
-            set_err(st, ERRB_TIMEOUT);
-            ok = false;
-        }
-        if (ok) {
-            const unsigned char *base = ring + (size_t)sl * SB;
-            const float *Ah = reinterpret_cast<const float *>(base);
-            const float *Al = reinterpret_cast<const float *>(base + BG_A_B);
-            const float *Xh = reinterpret_cast<const float *>(base + 2 * BG_A_B);
-            const float *Xl = Xh + S * BG_TC;
+    for (int rb = first_rb; seq < ntiles; rb += rb_step) {
+        F2 acc[RPW * NA][S];
 #pragma unroll
-            for (int k = 0; k < 2; k++) {
-                const int c0 = (k * 32 + g) * 4;
-                float4 ah[RPW], al[RPW];
+        for (int q = 0; q < RPW * NA; q++)
+#pragma unroll
+            for (int j = 0; j < S; j++) acc[q][j] = {0.f, 0.f};
+        const long long rfirst = (long long)rb * CT;
+        const int end = whole ? seq + CT : (int)min((long long)ntiles, rfirst + CT - t0);
+        for (; seq < end; seq++) {
+            const int sl = seq % NST;
+            // on a timeout the warp stops waiting and computing but keeps walking
+            // its tiles, so it still meets the others where a row block is shared
+            ok = ok && mbar_wait(&full[sl], (seq / NST) & 1);
+            if (!__all_sync(0xffffffffu, ok)) {
+                set_err(st, ERRB_TIMEOUT);
+                ok = false;
+            }
+            if (ok) bg_tile<S>(acc, ring + (size_t)sl * SB, w, g);
+            __syncwarp();
+            if (g == 0) mbar_arrive(&empty[sl]);
+        }
+        // this CTA's share of row block rb
+        if constexpr (NA == 2)
+#pragma unroll
+            for (int j = 0; j < S; j++) acc[0][j] = f2_add(acc[0][j], acc[1][j]);
+        // the 32 lanes of a row
+#pragma unroll
+        for (int q = 0; q < RPW; q++)
+#pragma unroll
+            for (int j = 0; j < S; j++) {
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    F2 b;
+                    b.h = __shfl_xor_sync(0xffffffffu, acc[q][j].h, o);
+                    b.l = __shfl_xor_sync(0xffffffffu, acc[q][j].l, o);
+                    acc[q][j] = f2_add(acc[q][j], b);
+                }
+            }
+        if (whole || (t0 <= rfirst && rfirst + CT <= t0 + ntiles)) {
+            if (g == 0)
 #pragma unroll
                 for (int q = 0; q < RPW; q++) {
-                    ah[q] = *reinterpret_cast<const float4 *>(Ah + (w + WS * q) * BG_TC + c0);
-                    al[q] = *reinterpret_cast<const float4 *>(Al + (w + WS * q) * BG_TC + c0);
-                }
-#pragma unroll
-                for (int j = 0; j < S; j++) {
-                    const float4 xh = *reinterpret_cast<const float4 *>(Xh + j * BG_TC + c0);
-                    const float4 xl = *reinterpret_cast<const float4 *>(Xl + j * BG_TC + c0);
-#pragma unroll
-                    for (int q = 0; q < RPW; q++) {
-                        F2 &a2 = acc[NA == 2 ? k : q][j];
-                        f2_mac(a2, ah[q].x, al[q].x, xh.x, xl.x);
-                        f2_mac(a2, ah[q].y, al[q].y, xh.y, xl.y);
-                        f2_mac(a2, ah[q].z, al[q].z, xh.z, xl.z);
-                        f2_mac(a2, ah[q].w, al[q].w, xh.w, xl.w);
-                    }
-                }
-            }
-        }
-        __syncwarp();
-        if (g == 0) mbar_arrive(&empty[sl]);
-        if (t == CT - 1 || seq == ntiles - 1) {
-            // this CTA's share of row block rb
-            if constexpr (NA == 2)
-#pragma unroll
-                for (int j = 0; j < S; j++) acc[0][j] = f2_add(acc[0][j], acc[1][j]);
-            // the 32 lanes of a row
-#pragma unroll
-            for (int q = 0; q < RPW; q++)
-#pragma unroll
-                for (int j = 0; j < S; j++) {
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        F2 b;
-                        b.h = __shfl_xor_sync(0xffffffffu, acc[q][j].h, o);
-                        b.l = __shfl_xor_sync(0xffffffffu, acc[q][j].l, o);
-                        acc[q][j] = f2_add(acc[q][j], b);
-                    }
-                }
-            const long long rfirst = (long long)rb * CT;
-            if (t0 <= rfirst && rfirst + CT <= t1) {
-                if (g == 0)
-#pragma unroll
-                    for (int q = 0; q < RPW; q++) {
-                        const int row = rb * BG_TR + w + WS * q;
-                        if (row < n)
-#pragma unroll
-                            for (int j = 0; j < S; j++)
-                                if (j < a.s) a.Q[(long long)j * a.ldq + row] = (double)acc[q][j].h + (double)acc[q][j].l;
-                    }
-            } else {
-                // shared with neighbouring CTAs: publish the partial sums; the last of
-                // the sharing CTAs adds them in CTA order
-                double *fix = a.scr->fix + (size_t)(2 * blockIdx.x + (rb == first_rb ? 0 : 1)) * BG_TR * S;
-                if (g == 0) {
-#pragma unroll
-                    for (int q = 0; q < RPW; q++)
+                    const int row = rb * BG_TR + w + WS * q;
+                    if (row < n)
 #pragma unroll
                         for (int j = 0; j < S; j++)
-                            fix[(w + WS * q) * S + j] = (double)acc[q][j].h + (double)acc[q][j].l;
-                    __threadfence();
+                            if (j < a.s) a.Q[(long long)j * a.ldq + row] = (double)acc[q][j].h + (double)acc[q][j].l;
                 }
-                named_bar(1, BG_C);
-                if (threadIdx.x == 0) {
-                    ca_s = bg_owner(rfirst, T, gridDim.x);
-                    cb_s = bg_owner(rfirst + CT - 1, T, gridDim.x);
-                    int ncov = 0;
-                    for (int c = ca_s; c <= cb_s; c++) ncov += bg_start(T, c, gridDim.x) < bg_start(T, c + 1, gridDim.x);
-                    fin_s = atomicAdd(&a.scr->bticket[ca_s], 1u) == (unsigned)ncov - 1;
-                    if (fin_s) atomicExch(&a.scr->bticket[ca_s], 0u);
-                }
-                named_bar(1, BG_C);
-                if (fin_s) {
-                    __threadfence();
-                    for (int e = threadIdx.x; e < BG_TR * S; e += BG_C) {
-                        const int row = rb * BG_TR + e / S, j = e % S;
-                        double sum = 0.0;
-                        for (int c = ca_s; c <= cb_s; c++) {
-                            const long long a0 = bg_start(T, c, gridDim.x);
-                            if (bg_start(T, c + 1, gridDim.x) <= a0) continue;   // empty CTA
-                            const int slot = rb == (int)(a0 / CT) ? 0 : 1;
-                            sum += __ldcg(&a.scr->fix[(size_t)(2 * c + slot) * BG_TR * S + e]);
-                        }
-                        if (row < n && j < a.s) a.Q[(long long)j * a.ldq + row] = sum;
+        } else {
+            // shared with neighbouring CTAs: publish the partial sums; the last of
+            // the sharing CTAs adds them in CTA order
+            double *fix = a.scr->fix + (size_t)(2 * blockIdx.x + (rb == first_rb ? 0 : 1)) * BG_TR * S;
+            if (g == 0) {
+#pragma unroll
+                for (int q = 0; q < RPW; q++)
+#pragma unroll
+                    for (int j = 0; j < S; j++)
+                        fix[(w + WS * q) * S + j] = (double)acc[q][j].h + (double)acc[q][j].l;
+                __threadfence();
+            }
+            named_bar(1, BG_C);
+            if (threadIdx.x == 0) {
+                ca_s = bg_owner(rfirst, T, gridDim.x);
+                cb_s = bg_owner(rfirst + CT - 1, T, gridDim.x);
+                int ncov = 0;
+                for (int c = ca_s; c <= cb_s; c++) ncov += bg_start(T, c, gridDim.x) < bg_start(T, c + 1, gridDim.x);
+                fin_s = atomicAdd(&a.scr->bticket[ca_s], 1u) == (unsigned)ncov - 1;
+                if (fin_s) atomicExch(&a.scr->bticket[ca_s], 0u);
+            }
+            named_bar(1, BG_C);
+            if (fin_s) {
+                __threadfence();
+                for (int e = threadIdx.x; e < BG_TR * S; e += BG_C) {
+                    const int row = rb * BG_TR + e / S, j = e % S;
+                    double sum = 0.0;
+                    for (int c = ca_s; c <= cb_s; c++) {
+                        const long long a0 = bg_start(T, c, gridDim.x);
+                        if (bg_start(T, c + 1, gridDim.x) <= a0) continue;   // empty CTA
+                        const int slot = rb == (int)(a0 / CT) ? 0 : 1;
+                        sum += __ldcg(&a.scr->fix[(size_t)(2 * c + slot) * BG_TR * S + e]);
                     }
+                    if (row < n && j < a.s) a.Q[(long long)j * a.ldq + row] = sum;
                 }
             }
-#pragma unroll
-            for (int q = 0; q < RPW * NA; q++)
-#pragma unroll
-                for (int j = 0; j < S; j++) acc[q][j] = {0.f, 0.f};
-        }
-        if (++t == CT) {
-            t = 0;
-            rb++;
         }
     }
 }
