@@ -118,7 +118,8 @@ typedef struct {
     double rel_res;      /* last recursive (or Givens-estimated) relative residual       */
     double true_rel_res; /* ||b - A x|| / ||b|| recomputed in FP64 at exit               */
     double time_ms;      /* device time of the solve (CUDA events on the context stream) */
-    double bytes_moved;  /* algorithmic bytes of A streamed (sum over all products; a
+    double bytes_moved;  /* algorithmic bytes of A streamed (sum over all products; one
+                            triangle where CG reads that of an exactly symmetric A; a
                             fused solve streams A once)                                  */
     long long launches;  /* kernels executed on the device for this call                 */
 } ls_info;
@@ -315,8 +316,9 @@ int ls_block_gmres_solve(ls_ctx *ctx, int n, int s, const double *A, int64_t lda
  * 0).  A zero pivot returns LS_BREAKDOWN with x unchanged; a residual that
  * is not finite returns LS_ERR_NAN.  A row-major n x n (host or device), b
  * and x n vectors; opts may be NULL; opts->precision must be LS_F64.  The
- * elimination is n^3 / 3 updates of two FP64 instructions each, bound by the
- * FP64 pipe; the trailing block crosses HBM once per panel.
+ * elimination is n^3 / 3 updates, a product and a difference each rounded; the
+ * products are formed by integer instructions, the differences by the FP64
+ * pipe, which bounds it.  The trailing block crosses HBM once per panel.
  */
 int ls_lu_solve(ls_ctx *ctx, int n, const double *A, int64_t lda, const double *b, double *x,
                 const ls_opts *opts, ls_info *info);
@@ -549,8 +551,8 @@ int ls_tune_lookup(int n, int nrhs, int num_sms, int *ks32, int *tensor_cores);
  * positive definite) or NaN returns LS_BREAKDOWN with x unchanged; a residual
  * that is not finite returns LS_ERR_NAN.  A row-major n x n (host or device),
  * b and x n vectors; opts may be NULL; opts->precision must be LS_F64.  The
- * factorization is n^3 / 6 updates of two FP64 instructions each, bound by
- * the FP64 pipe.
+ * factorization is n^3 / 6 updates, formed as ls_lu_solve's and bound by the
+ * FP64 pipe.
  */
 int ls_chol_solve(ls_ctx *ctx, int n, const double *A, int64_t lda, const double *b, double *x,
                   const ls_opts *opts, ls_info *info);
