@@ -29,11 +29,11 @@
 // n = 4000 to 16384), below it the tile loop (1.3 us a tile and SM, the FP32 pipe 44 %
 // busy) and the latency of the barrier and the final sums.  A CG step (product and
 // update) at n = 16384 took 317 us with the general product and takes 187; n = 4000
-// 48 -> 28, n = 1024 28 -> 19; BF16 inside the flexible CG at n =
-// 32768 331 -> 192 ms a solve.  Packing: 0.93 ms at n = 16384 against 1.35 for the split
-// of all of A.  Tried and no faster: mbarrier hand-over to reducing warps instead of the
-// barrier a tile (192 us), 16 consumer warps of 8 rows (193), fetching the next
-// product's first tiles into L2 during the update (191 to 196).
+// 48 -> 28, n = 1024 28 -> 19; BF16 inside the flexible CG at n = 32768 331 -> 192 ms
+// a solve.  Packing: 0.71 ms at n = 16384, as long as the split of all of A.  Tried and
+// no faster: mbarrier hand-over to reducing warps instead of the barrier a tile (192 us
+// a step where this form took 191), 16 consumer warps of 8 rows (193), fetching the
+// next product's first tiles into L2 during the update (191 to 196).
 #include <cuda_bf16.h>
 
 #include "ls_device.cuh"
