@@ -28,6 +28,8 @@
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
+#include <type_traits>
+
 #include "ls_device.cuh"
 #include "ls_ds.cuh"
 #include "ls_gemv.cuh"
@@ -135,9 +137,21 @@ __device__ __forceinline__ void load_x(const typename Cfg<DT>::X *x, int c0, int
         for (int k = 0; k < VEC; k++) v[k] = (c0 + k < cols) ? x[c0 + k] : X(0);
     }
 }
-// ... as the operand of the products (the FP32 pair: off the FP64 pipe).
-__device__ __forceinline__ void to_operand(double x, DSV &p) { split_pair(x, p.h, p.l); }
+// ... as the operand of the products.  The FP32 pair: by integer instructions where the
+// chain of a tile counts (whole row tiles; Jacobi, n = 2500: 23.6 -> 21.0 us a step), by
+// the FP64 pipe, idle otherwise, where HBM binds (n = 16384: 316 -> 313).
+template <bool INT>
+__device__ __forceinline__ void to_operand(double x, DSV &p) {
+    if constexpr (INT) {
+        split_pair(x, p.h, p.l);
+    } else {
+        const float h = __double2float_rn(x);
+        p = DSV{h, __double2float_rn(x - (double)h)};
+    }
+}
+template <bool INT>
 __device__ __forceinline__ void to_operand(double x, double &p) { p = x; }
+template <bool INT>
 __device__ __forceinline__ void to_operand(float x, float &p) { p = x; }
 
 // acc0 + acc1 += a[0:VEC] . p[0:VEC] (two independent FMA chains); `a` points
@@ -360,113 +374,121 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
 
         // With one CTA on most SMs (whole row tiles) x of a tile is asked for while the tile before
         // it is worked on (Jacobi, n = 2500: 0.53 -> 0.47 ms); with two the other
-        // CTA hides that latency, and asking early costs 3 % at n = 16384.
-        X xv[VEC];
-        if (whole && ntiles > 0) load_x<DT>(x, lane_col, cols, xv);
-        for (int i = 0; i < ntiles; i++) {
-            V p[VEC];
-            if (!whole) load_x<DT>(x, ct * TC + lane_col, cols, xv);
+        // CTA hides that latency, and asking early costs 3 % at n = 16384.  Two copies of
+        // the loop: deciding inside it cost 1.7 % there.
+        auto tiles = [&](auto ahead) {
+            constexpr bool AHEAD = decltype(ahead)::value;
+            X xv[VEC];
+            if constexpr (AHEAD)
+                if (ntiles > 0) load_x<DT>(x, lane_col, cols, xv);
+            for (int i = 0; i < ntiles; i++) {
+                V p[VEC];
+                if constexpr (!AHEAD) load_x<DT>(x, ct * TC + lane_col, cols, xv);
 #pragma unroll
-            for (int k = 0; k < VEC; k++) to_operand(xv[k], p[k]);
-            if (whole && i + 1 < ntiles) load_x<DT>(x, (ct + 1) * TC + lane_col, cols, xv);
-            if (TMA) {
-                // On a timeout the warp stops waiting and computing but keeps
-                // walking the tile sequence, so it still meets the other
-                // consumer warps at every named barrier below.
-                const int s = i % NST;
-                if (!*(volatile int *)&abort_s && !mbar_wait(&full[s], (i / NST) & 1)) {
-                    set_err(args.st, ERRB_TIMEOUT);
-                    abort_s = 1;
-                }
-                if (!*(volatile int *)&abort_s) {
-                    const T *tile = ring + (size_t)s * STAGE_ELEMS;
-#pragma unroll
-                    for (int r = 0; r < RW; r++)
-                        dot_tile<DT>(tile + (wr * RW + r) * TC + lane_col, p, acc[r], acc1[r]);
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&empty[s]);
-            } else {
-#pragma unroll
-                for (int r = 0; r < RW; r++) {
-                    const int row = rt * TR + wr * RW + r;
-                    if (row < rows)
-                        dot_global<DT>(Ag, Agl, M.lda, row, ct * TC + lane_col, cols, p, acc[r], acc1[r]);
-                }
-            }
-            if (ct == CT - 1 || i == ntiles - 1) {
-                // this CTA's share of row tile rt is done: reduce it over the warp
-#pragma unroll
-                for (int r = 0; r < RW; r++) {
-                    acc[r] += acc1[r];
-                    acc1[r] = V{};
-                }
-                butterfly<RW, 16>(acc, lane);
-                if ((lane & ((32 >> LGR) - 1)) == 0) red[wc][wr * RW + (lane >> (5 - LGR))] = acc[0];
-#pragma unroll
-                for (int r = 0; r < RW; r++) acc[r] = V{};
-                consumers_sync();
-                const long long rfirst = (long long)rt * CT;
-                const bool complete = (t0 <= rfirst) && (rfirst + CT <= t1);
-                if (complete) {
-                    for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                        V s{};
-#pragma unroll
-                        for (int c = 0; c < WC; c++) s += red[c][tr];
-                        const int row = rt * TR + tr;
-                        if (row < rows) mydot += epilogue<Y>(args, row, scaled<DT>(M, row, (Y)to_double(s)));
+                for (int k = 0; k < VEC; k++) to_operand<AHEAD>(xv[k], p[k]);
+                if constexpr (AHEAD)
+                    if (i + 1 < ntiles) load_x<DT>(x, (ct + 1) * TC + lane_col, cols, xv);
+                if (TMA) {
+                    // On a timeout the warp stops waiting and computing but keeps
+                    // walking the tile sequence, so it still meets the other
+                    // consumer warps at every named barrier below.
+                    const int s = i % NST;
+                    if (!*(volatile int *)&abort_s && !mbar_wait(&full[s], (i / NST) & 1)) {
+                        set_err(args.st, ERRB_TIMEOUT);
+                        abort_s = 1;
                     }
+                    if (!*(volatile int *)&abort_s) {
+                        const T *tile = ring + (size_t)s * STAGE_ELEMS;
+#pragma unroll
+                        for (int r = 0; r < RW; r++)
+                            dot_tile<DT>(tile + (wr * RW + r) * TC + lane_col, p, acc[r], acc1[r]);
+                    }
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&empty[s]);
                 } else {
-                    // A row tile shared with neighbouring CTAs: publish the
-                    // partial sums; the last of the sharing CTAs to arrive adds
-                    // them in CTA order and finishes those rows.
-                    const int slot = (rt == first_rt) ? 0 : 1;
-                    for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                        V s{};
 #pragma unroll
-                        for (int c = 0; c < WC; c++) s += red[c][tr];
-                        args.scr->fix[((size_t)cta * 2 + slot) * TR + tr] = (double)to_double(s);
-                        __threadfence();
+                    for (int r = 0; r < RW; r++) {
+                        const int row = rt * TR + wr * RW + r;
+                        if (row < rows)
+                            dot_global<DT>(Ag, Agl, M.lda, row, ct * TC + lane_col, cols, p, acc[r], acc1[r]);
                     }
-                    consumers_sync();
-                    if (threadIdx.x == 0) {
-                        const int ca = tile_owner(rfirst, T_all, G_);
-                        const int cb = tile_owner(rfirst + CT - 1, T_all, G_);
-                        int ncov = 0;
-                        for (int c = ca; c <= cb; c++)
-                            ncov += tile_start(T_all, c, G_) < tile_start(T_all, c + 1, G_);
-                        const unsigned prev = atomicAdd(&args.scr->bticket[ca], 1u);
-                        fin_s = (prev == (unsigned)ncov - 1);
-                        if (fin_s) atomicExch(&args.scr->bticket[ca], 0u);
-                        ca_s = ca;
-                        cb_s = cb;
+                }
+                if (ct == CT - 1 || i == ntiles - 1) {
+                    // this CTA's share of row tile rt is done: reduce it over the warp
+#pragma unroll
+                    for (int r = 0; r < RW; r++) {
+                        acc[r] += acc1[r];
+                        acc1[r] = V{};
                     }
+                    butterfly<RW, 16>(acc, lane);
+                    if ((lane & ((32 >> LGR) - 1)) == 0) red[wc][wr * RW + (lane >> (5 - LGR))] = acc[0];
+#pragma unroll
+                    for (int r = 0; r < RW; r++) acc[r] = V{};
                     consumers_sync();
-                    if (fin_s) {
-                        __threadfence();
+                    const long long rfirst = (long long)rt * CT;
+                    const bool complete = (t0 <= rfirst) && (rfirst + CT <= t1);
+                    if (complete) {
                         for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                            double s = 0.0;
-                            for (int c = ca_s; c <= cb_s; c++) {
-                                const long long a0 = tile_start(T_all, c, G_);
-                                if (tile_start(T_all, c + 1, G_) <= a0) continue;   // empty CTA
-                                const int sl = (rt == (int)(a0 / CT)) ? 0 : 1;
-                                s += __ldcg(&args.scr->fix[((size_t)c * 2 + sl) * TR + tr]);
-                            }
+                            V s{};
+#pragma unroll
+                            for (int c = 0; c < WC; c++) s += red[c][tr];
                             const int row = rt * TR + tr;
-                            tdot[tr] = row < rows ? epilogue<Y>(args, row, scaled<DT>(M, row, (Y)s)) : 0.0;
+                            if (row < rows) mydot += epilogue<Y>(args, row, scaled<DT>(M, row, (Y)to_double(s)));
+                        }
+                    } else {
+                        // A row tile shared with neighbouring CTAs: publish the
+                        // partial sums; the last of the sharing CTAs to arrive adds
+                        // them in CTA order and finishes those rows.
+                        const int slot = (rt == first_rt) ? 0 : 1;
+                        for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
+                            V s{};
+#pragma unroll
+                            for (int c = 0; c < WC; c++) s += red[c][tr];
+                            args.scr->fix[((size_t)cta * 2 + slot) * TR + tr] = (double)to_double(s);
+                            __threadfence();
                         }
                         consumers_sync();
                         if (threadIdx.x == 0) {
-                            double d = 0.0;
-                            for (int tr = 0; tr < TR; tr++) d += tdot[tr];
-                            args.scr->fixdot[ca_s] = d;
+                            const int ca = tile_owner(rfirst, T_all, G_);
+                            const int cb = tile_owner(rfirst + CT - 1, T_all, G_);
+                            int ncov = 0;
+                            for (int c = ca; c <= cb; c++)
+                                ncov += tile_start(T_all, c, G_) < tile_start(T_all, c + 1, G_);
+                            const unsigned prev = atomicAdd(&args.scr->bticket[ca], 1u);
+                            fin_s = (prev == (unsigned)ncov - 1);
+                            if (fin_s) atomicExch(&args.scr->bticket[ca], 0u);
+                            ca_s = ca;
+                            cb_s = cb;
+                        }
+                        consumers_sync();
+                        if (fin_s) {
+                            __threadfence();
+                            for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
+                                double s = 0.0;
+                                for (int c = ca_s; c <= cb_s; c++) {
+                                    const long long a0 = tile_start(T_all, c, G_);
+                                    if (tile_start(T_all, c + 1, G_) <= a0) continue;   // empty CTA
+                                    const int sl = (rt == (int)(a0 / CT)) ? 0 : 1;
+                                    s += __ldcg(&args.scr->fix[((size_t)c * 2 + sl) * TR + tr]);
+                                }
+                                const int row = rt * TR + tr;
+                                tdot[tr] = row < rows ? epilogue<Y>(args, row, scaled<DT>(M, row, (Y)s)) : 0.0;
+                            }
+                            consumers_sync();
+                            if (threadIdx.x == 0) {
+                                double d = 0.0;
+                                for (int tr = 0; tr < TR; tr++) d += tdot[tr];
+                                args.scr->fixdot[ca_s] = d;
+                            }
                         }
                     }
+                    consumers_sync();
                 }
-                consumers_sync();
+                if (++ct == CT) { ct = 0; ++rt; }
             }
-            if (++ct == CT) { ct = 0; ++rt; }
-        }
+        };
+        if (whole) tiles(std::true_type{});
+        else tiles(std::false_type{});
     }
 
     // ---- per-CTA dot; the last CTA reduces them (all threads, fixed order) ----
