@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(KB) gm_arnoldi_kernel(Vecs v, cudaGraphConditi
             warp_sums(s);
 #pragma unroll
             for (int u = 0; u < U; u++)
-                if (lane == 0 && j0 + u * NW <= k) v.part[(size_t)(j0 + u * NW) * G + blockIdx.x] = s[u];
+                if (lane == 0 && j0 + u * NW <= k) v.part[(size_t)gm_slot(pass, j0 + u * NW) * G + blockIdx.x] = s[u];
         }
         ok = grid_sync(v.bar, st);
         if (!ok) break;
@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(KB) gm_arnoldi_kernel(Vecs v, cudaGraphConditi
             for (int b = lane; b < G; b += 32)
 #pragma unroll
                 for (int u = 0; u < U; u++)
-                    if (j0 + u * NW <= k) s[u] += __ldcg(&v.part[(size_t)(j0 + u * NW) * G + b]);
+                    if (j0 + u * NW <= k) s[u] += __ldcg(&v.part[(size_t)gm_slot(pass, j0 + u * NW) * G + b]);
             warp_sums(s);
 #pragma unroll
             for (int u = 0; u < U; u++)
@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(KB) gm_arnoldi_kernel(Vecs v, cudaGraphConditi
         __syncthreads();
         if (pass == 0 && again_s) continue;
         acc = block_sum(acc, red);
-        publish(v.part, LS_MAX_RESTART + 1, acc);   // a slot that no h uses
+        publish(v.part, GM_SLOT_NORM, acc);
         const unsigned ticket = grid_arrive(v.bar);
         if (blockIdx.x == 0 && warp == 2) {
             // while the others arrive: the earlier rotations on the column.  a_j = -s_j a_(j-1) + c_j h_j
@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(KB) gm_arnoldi_kernel(Vecs v, cudaGraphConditi
         if (threadIdx.x == 96) w0_s = 1e-14 * sqrt(wnorm0);
         ok = grid_wait(v.bar, ticket, st);
         if (ok && warp == 0) {
-            const double t = reduce_slot(v.part, LS_MAX_RESTART + 1, G);
+            const double t = reduce_slot(v.part, GM_SLOT_NORM, G);
             if (lane == 0) wn2_s = t;
         }
         break;

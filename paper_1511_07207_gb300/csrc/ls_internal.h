@@ -206,7 +206,16 @@ struct Vecs {
     GmresSmall *gm;
     double rtol;
 };
-constexpr int PART_SLOTS = LS_MAX_RESTART + 4;
+constexpr int PART_SLOTS = 2 * LS_MAX_RESTART + 4;
+// GMRES's slots in it: h_j of either Gram-Schmidt pass, and ||w||^2.  A slot is written
+// again only after a grid barrier that follows its last read.  Between the
+// first pass's reads and the second pass's writes there is none, so the passes
+// have slots of their own.
+constexpr int gm_slot(int pass, int j) { return pass * LS_MAX_RESTART + j; }
+constexpr int GM_SLOT_NORM = 2 * LS_MAX_RESTART;
+static_assert(gm_slot(0, LS_MAX_RESTART - 1) < gm_slot(1, 0) && gm_slot(1, LS_MAX_RESTART - 1) < GM_SLOT_NORM &&
+                  GM_SLOT_NORM < PART_SLOTS,
+              "disjoint slots");
 
 // ---- mixed-precision vectors (workspace) -------------------------------------------
 struct MixVecs {
