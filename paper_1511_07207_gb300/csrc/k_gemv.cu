@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
     T *ring = reinterpret_cast<T *>(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + (size_t)NST * G::TILE_BYTES * C::PARTS);
     uint64_t *empty = full + NST;
-    __shared__ V red[WC][TR];
+    using S = decltype(as_sum(V{}));          // a row's sums: pairs for the FP32 formats too
+    __shared__ S red[WC][TR];
     __shared__ double dred[GEMV_THREADS / 32];
     __shared__ int abort_s, last_s, fin_s, ca_s, cb_s;
     __shared__ double tdot[TR];
@@ -378,6 +379,16 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
         // the loop: deciding inside it cost 1.7 % there.
         auto tiles = [&](auto ahead) {
             constexpr bool AHEAD = decltype(ahead)::value;
+            // A whole row is a longer chain than an equal piece, so its error is kept down to that
+            // of the pieces: the lanes' sums are added as pairs (settled ones for the
+            // FP32 pair), and the FP32 formats' accumulators go into a sum of their own after every
+            // second tile.  Equal pieces are added in FP64 and need neither.
+            constexpr bool SETTLED = AHEAD && DT == DT_DS;
+            constexpr bool PART = AHEAD && std::is_same<V, float>::value;
+            using L = typename std::conditional<AHEAD, S, V>::type;
+            V part[RW];
+#pragma unroll
+            for (int r = 0; r < RW; r++) part[r] = V{};
             X xv[VEC];
             if constexpr (AHEAD)
                 if (ntiles > 0) load_x<DT>(x, lane_col, cols, xv);
@@ -413,27 +424,36 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
                             dot_global<DT>(Ag, Agl, M.lda, row, ct * TC + lane_col, cols, p, acc[r], acc1[r]);
                     }
                 }
+                if constexpr (PART)
+                    if (i & 1) {
+#pragma unroll
+                        for (int r = 0; r < RW; r++) {
+                            part[r] = part[r] + (acc[r] + acc1[r]);
+                            acc[r] = acc1[r] = V{};
+                        }
+                    }
                 if (ct == CT - 1 || i == ntiles - 1) {
                     // this CTA's share of row tile rt is done: reduce it over the warp
+                    L sum[RW];
 #pragma unroll
                     for (int r = 0; r < RW; r++) {
-                        acc[r] += acc1[r];
-                        acc1[r] = V{};
+                        if constexpr (AHEAD) sum[r] = join<SETTLED>(as_sum(acc[r]), as_sum(acc1[r]));
+                        else sum[r] = acc[r] + acc1[r];
+                        if constexpr (PART) sum[r] = join<SETTLED>(as_sum(part[r]), sum[r]);
+                        acc[r] = acc1[r] = part[r] = V{};
                     }
-                    butterfly<RW, 16>(acc, lane);
-                    if ((lane & ((32 >> LGR) - 1)) == 0) red[wc][wr * RW + (lane >> (5 - LGR))] = acc[0];
-#pragma unroll
-                    for (int r = 0; r < RW; r++) acc[r] = V{};
+                    butterfly<RW, 16, SETTLED>(sum, lane);
+                    if ((lane & ((32 >> LGR) - 1)) == 0) red[wc][wr * RW + (lane >> (5 - LGR))] = as_sum(sum[0]);
                     consumers_sync();
                     const long long rfirst = (long long)rt * CT;
                     const bool complete = (t0 <= rfirst) && (rfirst + CT <= t1);
                     if (complete) {
                         for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                            V s{};
+                            S s{};
 #pragma unroll
-                            for (int c = 0; c < WC; c++) s += red[c][tr];
+                            for (int c = 0; c < WC; c++) s = join<SETTLED>(s, red[c][tr]);
                             const int row = rt * TR + tr;
-                            if (row < rows) mydot += epilogue<Y>(args, row, scaled<DT>(M, row, (Y)to_double(s)));
+                            if (row < rows) mydot += epilogue<Y>(args, row, scaled<DT>(M, row, (Y)pair_value(s)));
                         }
                     } else {
                         // A row tile shared with neighbouring CTAs: publish the
@@ -441,10 +461,10 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
                         // them in CTA order and finishes those rows.
                         const int slot = (rt == first_rt) ? 0 : 1;
                         for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                            V s{};
+                            S s{};
 #pragma unroll
-                            for (int c = 0; c < WC; c++) s += red[c][tr];
-                            args.scr->fix[((size_t)cta * 2 + slot) * TR + tr] = (double)to_double(s);
+                            for (int c = 0; c < WC; c++) s = join<SETTLED>(s, red[c][tr]);
+                            args.scr->fix[((size_t)cta * 2 + slot) * TR + tr] = pair_value(s);
                             __threadfence();
                         }
                         consumers_sync();

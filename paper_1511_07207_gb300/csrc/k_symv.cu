@@ -247,6 +247,10 @@ __global__ void __launch_bounds__(S_T, 1) symv_kernel(SymMat M, GemvArgs args) {
                 const T *tile = ring + (size_t)s * (G_::BYTES / sizeof(T)) + (warp * S_RW) * TC + lane * VEC;
 #pragma unroll
                 for (int r = 0; r < S_RW; r++) both<DT>(tile + r * TC, p, xrow[warp * S_RW + r], acc[r], col);
+                if (DT == DT_DS && (J & 3) == 3) {
+#pragma unroll
+                    for (int r = 0; r < S_RW; r++) acc[r] = settled(acc[r]);
+                }
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(&empty[s]);
@@ -257,13 +261,13 @@ __global__ void __launch_bounds__(S_T, 1) symv_kernel(SymMat M, GemvArgs args) {
             if (xg == i % G_::GROUPS) {   // one group adds the eight warps' column sums
                 V c = colbuf[(par * SW) * TC + xc];
 #pragma unroll
-                for (int w = 1; w < SW; w++) c += colbuf[(par * SW + w) * TC + xc];
+                for (int w = 1; w < SW; w++) c = settled_sum(c, colbuf[(par * SW + w) * TC + xc]);
                 pcol[(t0 + i) * TC + xc] = c;
             }
             if (row_ends || i == nt - 1) {
                 // this CTA's share of row block I
                 constexpr int LGR = log2i<S_RW>();
-                butterfly<S_RW, 16>(acc, lane);
+                butterfly<S_RW, 16, true>(acc, lane);
                 if ((lane & ((32 >> LGR) - 1)) == 0)
                     prow[(size_t)(cta + I) * S_TR + warp * S_RW + (lane >> (5 - LGR))] = acc[0];
 #pragma unroll
@@ -319,8 +323,8 @@ __global__ void __launch_bounds__(S_T, 1) symv_kernel(SymMat M, GemvArgs args) {
                 }
 #pragma unroll
                 for (int u = 0; u < U; u++) {
-                    s0 += wide(a0[u]);
-                    s1 += wide(a1[u]);
+                    s0 = settled_sum(s0, wide(a0[u]));
+                    s1 = settled_sum(s1, wide(a1[u]));
                 }
             }
             comb[it & 1][warp][2 * lane] = s0;
@@ -330,7 +334,7 @@ __global__ void __launch_bounds__(S_T, 1) symv_kernel(SymMat M, GemvArgs args) {
             if (threadIdx.x < S_CB && row < n) {
                 DSV s = comb[it & 1][0][threadIdx.x];
 #pragma unroll
-                for (int w = 1; w < SW; w++) s += comb[it & 1][w][threadIdx.x];
+                for (int w = 1; w < SW; w++) s = settled_sum(s, comb[it & 1][w][threadIdx.x]);
                 mydot += epilogue<X>(args, row, (X)to_double(s));
             }
         }

@@ -26,6 +26,18 @@ __device__ __forceinline__ DSV operator+(DSV a, DSV b) {
     return DSV{s, __fadd_rn(e, __fadd_rn(a.l, b.l))};
 }
 __device__ __forceinline__ DSV &operator+=(DSV &a, DSV b) { return a = a + b; }
+// The same value with |lo| at most half an ulp of hi (a fast two-sum).  A long chain
+// of products leaves rounding errors in lo that outgrow an ulp of hi many times, and every
+// further addition to lo is then rounded at that larger size.
+__device__ __forceinline__ DSV settled(DSV a) {
+    const float s = __fadd_rn(a.h, a.l);
+    return DSV{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
+}
+__device__ __forceinline__ float settled(float a) { return a; }
+__device__ __forceinline__ double settled(double a) { return a; }
+// Sums of finished partial sums.
+template <class V>
+__device__ __forceinline__ V settled_sum(V a, V b) { return settled(a + b); }
 __device__ __forceinline__ double to_double(DSV v) { return (double)v.h + (double)v.l; }
 __device__ __forceinline__ double to_double(double v) { return v; }
 __device__ __forceinline__ float to_double(float v) { return v; }

@@ -9,11 +9,25 @@
 
 namespace lsi {
 
+// a + b of two partial sums; SETTLED: of pairs, settled (ls_ds.cuh).  Pairs that stand for
+// FP32 sums are left unsettled, so that hi is what FP32 additions alone would give
+// (an infinity stays one: pair_value).
+template <bool SETTLED, class V>
+__device__ __forceinline__ V join(V a, V b) {
+    if constexpr (SETTLED) return settled_sum(a, b);
+    else return a + b;
+}
+__device__ __forceinline__ DSV as_sum(float v) { return DSV{v, 0.0f}; }
+__device__ __forceinline__ DSV as_sum(DSV v) { return v; }
+__device__ __forceinline__ double as_sum(double v) { return v; }
+__device__ __forceinline__ double pair_value(double v) { return v; }
+__device__ __forceinline__ double pair_value(DSV v) { return isfinite(v.h) ? to_double(v) : (double)v.h; }
+
 // Butterfly transpose-reduction of RW per-lane row accumulators over the warp:
 // each round a lane keeps half of its rows and adds the partner's copy of
 // them, so RW - 1 + (5 - log2 RW) additions replace RW full reductions.
 // Afterwards lane l holds the warp total of row (l >> (5 - log2 RW)).
-template <int N, int OFF, class V, int RW>
+template <int N, int OFF, bool SETTLED, class V, int RW>
 __device__ __forceinline__ void butterfly(V (&acc)[RW], int lane) {
     if constexpr (OFF >= 1) {
         if constexpr (N > 1) {
@@ -23,12 +37,12 @@ __device__ __forceinline__ void butterfly(V (&acc)[RW], int lane) {
             for (int i = 0; i < H; i++) {
                 const V send = upper ? acc[i] : acc[i + H];
                 const V keep = upper ? acc[i + H] : acc[i];
-                acc[i] = keep + shfl_xor_v(send, OFF);
+                acc[i] = join<SETTLED>(keep, shfl_xor_v(send, OFF));
             }
-            butterfly<H, OFF / 2>(acc, lane);
+            butterfly<H, OFF / 2, SETTLED>(acc, lane);
         } else {
-            acc[0] += shfl_xor_v(acc[0], OFF);
-            butterfly<1, OFF / 2>(acc, lane);
+            acc[0] = join<SETTLED>(acc[0], shfl_xor_v(acc[0], OFF));
+            butterfly<1, OFF / 2, SETTLED>(acc, lane);
         }
     }
 }
