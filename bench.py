@@ -138,13 +138,14 @@ def fp32_issue_peak():
 def gemv_source_hash():
     """Hash of the GEMV kernel's device source: k_gemv.cu up to its host-side
     section, the device helpers (ls_device.cuh, the double-single arithmetic of
-    ls_ds.cuh, the shared epilogues of ls_gemv.cuh, the split of x in split_pair.h)
+    ls_ds.cuh, the shared epilogues of ls_gemv.cuh, the split of x in split_pair.h,
+    the rule of gemv_split.h)
     and the GEMV_* constants of ls_internal.h."""
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1511_07207_gb300", "csrc")
     with open(os.path.join(csrc, "k_gemv.cu"), "rb") as fh:
         h.update(fh.read().split(b"// ---- host side", 1)[0])
-    for name in ("ls_device.cuh", "ls_ds.cuh", "ls_gemv.cuh", "split_pair.h"):
+    for name in ("ls_device.cuh", "ls_ds.cuh", "ls_gemv.cuh", "split_pair.h", "gemv_split.h"):
         with open(os.path.join(csrc, name), "rb") as fh:
             h.update(fh.read())
     with open(os.path.join(csrc, "ls_internal.h")) as fh:

@@ -10,7 +10,8 @@
 // Design (GB300):
 //  * persistent grid of 2 CTAs per SM; the (row-tile, column-tile) sequence
 //    of A is cut into equal contiguous pieces, one per CTA, so every SM gets
-//    the same number of bytes whatever n is;
+//    the same number of bytes whatever n is, or a CTA takes a whole row tile where
+//    that costs less (gemv_split.h);
 //  * one producer warp streams TR x TC tiles of A with 2-D TMA bulk copies
 //    (cp.async.bulk.tensor) into a 6-deep (3 for FP32 pairs) shared-memory ring with
 //    mbarrier completion; four consumer warps read the tiles with 128-bit
@@ -30,6 +31,7 @@
 
 #include <type_traits>
 
+#include "gemv_split.h"
 #include "ls_device.cuh"
 #include "ls_ds.cuh"
 #include "ls_gemv.cuh"
@@ -99,6 +101,11 @@ struct Geo {
 // two CTAs per SM.
 template <int DT>
 __host__ __device__ constexpr int stages() { return Cfg<DT>::PARTS > 1 ? 3 : GEMV_STAGES; }
+
+template <int DT>
+__device__ constexpr GemvCosts costs() {
+    return DT == DT_DS ? GEMV_COSTS_PAIR : DT == DT_BF16 ? GEMV_COSTS_BF16 : DT == DT_FP8 ? GEMV_COSTS_FP8 : GEMV_COSTS_F32;
+}
 
 int gemv_tile_rows(int dtype) {
     switch (dtype) {
@@ -294,12 +301,10 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
     const int RT = (rows + TR - 1) / TR, CT = (cols + TC - 1) / TC;
     const long long T_all = (long long)RT * CT;
     const int G_ = gridDim.x, cta = blockIdx.x;
-    // Equal pieces, except when there are at most as many row tiles as CTAs (up to n =
-    // 4864 for the FP32 pair): then a CTA takes one whole row tile, and none of them waits to
-    // add partial sums with its neighbours (2 us each time; n = 2000: half of the kernel's time).
-    // The native FP64 product is bound by the FP64 pipe and keeps the equal pieces, which
-    // use every SM.
-    const bool whole = DT != DT_F64 && RT <= G_;
+    // Equal pieces, or one whole row tile a CTA where the meetings of equal pieces cost more than
+    // the SMs that stay idle (gemv_split.h).  The native FP64 product is bound by the
+    // FP64 pipe and keeps the equal pieces, which use every SM.
+    const bool whole = DT != DT_F64 && gemv_whole_tiles(costs<DT>(), RT, CT, G_);
     const long long t0 = whole ? (long long)min(cta, RT) * CT : tile_start(T_all, cta, G_);
     const long long t1 = whole ? (long long)min(cta + 1, RT) * CT : tile_start(T_all, cta + 1, G_);
     const int ntiles = (int)(t1 - t0);
