@@ -111,7 +111,7 @@ __device__ __forceinline__ void gram_reduce(const BcgVecs &v, double *G) {
 
 __device__ __forceinline__ bool all_pass(const BcgVecs &v, const double *rho) {
     bool ok = true;
-    for (int j = 0; j < v.s; j++) ok = ok && sqrt(rho[j + j * v.s]) <= v.rtol * v.sm->bn[j];
+    for (int j = 0; j < v.s; j++) ok = ok && sqrt(rho[j + j * v.s]) <= v.st->rtol * v.sm->bn[j];
     return ok;
 }
 
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(BK) bcg_check_kernel(BcgVecs v, cudaGraphCondi
         for (int j = 0; j < s; j++) {
             const double r2 = *(volatile double *)&sm->r2[j];
             nan = nan || !isfinite(r2);
-            pass = pass && sqrt(r2) <= v.rtol * sm->bn[j];
+            pass = pass && sqrt(r2) <= v.st->rtol * sm->bn[j];
         }
         int restart = 0;
         if (*(volatile int *)&st->err || nan) {
@@ -648,7 +648,7 @@ __device__ bool coop_orth(const BcgVecs &v, const double *W, long long lo, long 
 // Every column's ||R_j|| <= rtol ||B_j|| (r2 = the squared norms).
 __device__ __forceinline__ bool cols_pass(const BcgVecs &v, const double *r2) {
     bool ok = true;
-    for (int j = 0; j < v.s; j++) ok = ok && sqrt(r2[j]) <= v.rtol * v.sm->bn[j];
+    for (int j = 0; j < v.s; j++) ok = ok && sqrt(r2[j]) <= v.st->rtol * v.sm->bn[j];
     return ok;
 }
 
@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(BK) bcgd_step_kernel(BcgVecs v, cudaGraphCondi
     if (threadIdx.x < 32) {
         const double x = (int)threadIdx.x < s ? r2[threadIdx.x] : 0.0;
         const bool nan = __any_sync(0xffffffffu, !isfinite(x));
-        const bool pass = __all_sync(0xffffffffu, (int)threadIdx.x >= s || sqrt(x) <= v.rtol * __ldcg(&sm->bn[threadIdx.x & 15]));
+        const bool pass = __all_sync(0xffffffffu, (int)threadIdx.x >= s || sqrt(x) <= v.st->rtol * __ldcg(&sm->bn[threadIdx.x & 15]));
         if (threadIdx.x == 0) flag_s = nan ? -1 : pass ? 0 : 1;
     }
     __syncthreads();
@@ -828,7 +828,7 @@ __global__ void __launch_bounds__(BK) bcgd_check_kernel(BcgVecs v, cudaGraphCond
         for (int j = 0; j < s; j++) {
             const double r2 = *(volatile double *)&sm->r2[j];
             nan = nan || !isfinite(r2);
-            pass = pass && sqrt(r2) <= v.rtol * sm->bn[j];
+            pass = pass && sqrt(r2) <= v.st->rtol * sm->bn[j];
         }
         int restart = 0;
         if (*(volatile int *)&st->err || nan) {

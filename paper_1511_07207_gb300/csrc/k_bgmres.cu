@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(GT) bgm_start_kernel(BgmVecs v, cudaGraphCondi
             for (int b = 0; b < (int)gridDim.x; b++) r2 += __ldcg(&v.part[(size_t)b * v.part_stride + c]);
             if (blockIdx.x == 0) v.r2[c] = r2;
             nan = nan || !isfinite(r2);
-            pass = pass && sqrt(r2) <= v.rtol * v.bn[c];
+            pass = pass && sqrt(r2) <= v.st->rtol * v.bn[c];
         }
         int d = 0;   // 0 run a cycle, 1 stop
         if (*(volatile int *)&st->err || nan) {
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(GT) bgm_orth_kernel(BgmVecs v, cudaGraphCondit
     if (lane < s) {
         double e2 = 0.0;
         for (int r = kc; r < kc + s; r++) e2 += Gs[r + lane * L] * Gs[r + lane * L];
-        pass = sqrt(e2) <= v.rtol * v.bn[lane];
+        pass = sqrt(e2) <= v.st->rtol * v.bn[lane];
     }
     const bool conv = __all_sync(0xffffffffu, pass);
     if (lane == 0) {

@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(KB) cg_init_kernel(Vecs v, int x0_given,
         if (threadIdx.x == 0) {
             const double bn = sqrt(b2);
             st->bnorm = bn;
-            st->tol_abs = v.rtol * bn;
+            st->tol_abs = v.st->rtol * bn;
             st->rho = r2;
             st->rnorm = sqrt(r2);
             st->true_rnorm = sqrt(r2);
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(KB) gm_init_kernel(Vecs v, int x0_given,
         {
             const double bn = sqrt(b2);
             st->bnorm = bn;
-            st->tol_abs = v.rtol * bn;
+            st->tol_abs = v.st->rtol * bn;
             if (!x0_given) st->true_rnorm = bn;
             int go = 1;
             if (!isfinite(b2)) {
@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(KB) bs_init_kernel(Vecs v, int x0_given,
         if (threadIdx.x == 0) {
             const double bn = sqrt(b2);
             st->bnorm = bn;
-            st->tol_abs = v.rtol * bn;
+            st->tol_abs = v.st->rtol * bn;
             st->rho = r2;              // r^ = r
             st->alpha = 1.0;
             st->omega = 1.0;
@@ -895,7 +895,7 @@ __global__ void __launch_bounds__(KB) ja_init_kernel(Vecs v, int x0_given,
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const double bn = sqrt(b2);
         st->bnorm = bn;
-        st->tol_abs = v.rtol * bn;
+        st->tol_abs = v.st->rtol * bn;
         st->skip = 0;
         int go = 1;
         if (!isfinite(b2)) {

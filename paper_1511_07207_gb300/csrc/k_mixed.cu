@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(MB) mx_init_kernel(MixVecs v, int x0_given,
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const double bn = sqrt(b2);
         st->bnorm = bn;
-        st->tol_abs = v.rtol * bn;
+        st->tol_abs = v.st->rtol * bn;
         st->rnorm = sqrt(r2);
         st->true_rnorm = sqrt(r2);
         int go = 1;

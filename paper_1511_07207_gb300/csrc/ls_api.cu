@@ -432,7 +432,7 @@ void fill_info(ls_info *info, const State &s, int status, float ms, double bytes
     info->launches = launches;
 }
 
-Vecs make_vecs(ls_ctx *c, const F64Layout &L, int n, double rtol) {
+Vecs make_vecs(ls_ctx *c, const F64Layout &L, int n) {
     Vecs v{};
     v.n = n;
     v.x = L.x;
@@ -450,7 +450,6 @@ Vecs make_vecs(ls_ctx *c, const F64Layout &L, int n, double rtol) {
     v.bar = c->bar;
     v.st = c->st;
     v.gm = c->gm;
-    v.rtol = rtol;
     return v;
 }
 
@@ -749,12 +748,13 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
     rc = upload_desc(c, 0);
     State *hs = c->h_st;
     state_init(hs, max_iter);
+    hs->rtol = o.rtol;
     hs->m = m;
     hs->reorth = o.reorth;
     if (!rc) rc = upload_state(c);
     if (rc) return rc;
 
-    Vecs v = make_vecs(c, L, n, o.rtol);
+    Vecs v = make_vecs(c, L, n);
     const int dt = split ? DT_DS : DT_F64;
     GemvLaunch GL = gemv_plan(dt, hd->use_tma != 0, EPI_DOT, c->num_sms);
     // CG: the packed triangle takes the place of the pair when A is exactly symmetric

@@ -194,6 +194,7 @@ extern "C" int ls_block_cg_solve(ls_ctx *c, int n, int s, const double *A, int64
     rc = upload_desc(c, 0);
     State *hs = c->h_st;
     state_init(hs, max_iter);
+    hs->rtol = o.rtol;
     if (!rc) rc = upload_state(c);
     if (rc) return rc;
 
@@ -213,7 +214,6 @@ extern "C" int ls_block_cg_solve(ls_ctx *c, int n, int s, const double *A, int64
     v.sm = L.sm;
     v.bar = c->bar;
     v.st = c->st;
-    v.rtol = o.rtol;
     const int dt = split ? DT_DS : DT_F64;
     GemvLaunch GL = gemv_plan(dt, hd->use_tma != 0, EPI_DOT, c->num_sms);
     const int deflate = o.deflate ? 1 : 0;

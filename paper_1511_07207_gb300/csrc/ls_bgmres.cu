@@ -198,6 +198,7 @@ extern "C" int ls_block_gmres_solve(ls_ctx *c, int n, int s, const double *A, in
     rc = upload_desc(c, 0);
     State *hs = c->h_st;
     state_init(hs, max_iter);
+    hs->rtol = o.rtol;
     hs->m = m;
     if (!rc) rc = upload_state(c);
     if (rc) return rc;
@@ -227,7 +228,6 @@ extern "C" int ls_block_gmres_solve(ls_ctx *c, int n, int s, const double *A, in
     v.dead = L.dead;
     v.bar = c->bar;
     v.st = c->st;
-    v.rtol = o.rtol;
     v.deflate = o.deflate ? 1 : 0;
     long long key[8] = {300 + s + 50 * v.deflate, n, (long long)(uintptr_t)c->ws, m, o.x0_given, L.ld,
                         (long long)(uintptr_t)c->stream, DT_DS};

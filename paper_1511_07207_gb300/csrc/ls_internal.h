@@ -53,6 +53,7 @@ struct State {
     double omega;        // BiCGSTAB stabilisation step
     double pq;           // p.Ap
     double bnorm;        // ||b||
+    double rtol;         // set by the host for every solve (the cached graphs hold no tolerance)
     double tol_abs;      // rtol * ||b||
     double rnorm;        // recursive residual norm
     double true_rnorm;   // ||b - A x|| at the last check
@@ -204,7 +205,6 @@ struct Vecs {
     GridBar *bar;
     State *st;
     GmresSmall *gm;
-    double rtol;
 };
 constexpr int PART_SLOTS = 2 * LS_MAX_RESTART + 4;
 // GMRES's slots in it: h_j of either Gram-Schmidt pass, and ||w||^2.  A slot is written
@@ -229,7 +229,6 @@ struct MixVecs {
     double *part;
     GridBar *bar;
     State *st;
-    double rtol;
 };
 
 struct MixedKernels {
@@ -292,7 +291,6 @@ struct BcgVecs {
     BcgSmall *sm;
     GridBar *bar;
     State *st;
-    double rtol;
 };
 struct BcgKernels {
     void *init, *step, *check;             // O'Leary's form
@@ -390,7 +388,6 @@ struct BgmVecs {
     int *dead;                    // the dependent columns of the last starting block (s)
     GridBar *bar;
     State *st;
-    double rtol;
     int deflate;                  // replace dependent starting columns (else a breakdown)
 };
 struct BgmKernels {

@@ -236,6 +236,7 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     rc = upload_desc(c, 0);
     if (!rc) rc = upload_desc(c, 1);
     state_init(hs, 0);
+    hs->rtol = o.rtol;
     hs->max_outer = max_outer;
     hs->m = m;
     hs->in_max = o.inner_iters;
@@ -250,7 +251,7 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     v.x = L.x; v.b = L.b; v.r = L.r; v.q = L.q; v.P = L.P; v.W = L.W; v.ldp = L.ldp;
     v.dvals = L.dvals;
     v.rf = L.rf; v.zf = L.zf; v.pf = L.pf; v.qf = L.qf;
-    v.part = c->part; v.bar = c->bar; v.st = c->st; v.rtol = o.rtol;
+    v.part = c->part; v.bar = c->bar; v.st = c->st;
     P64.gemv = gemv_plan(split ? DT_DS : DT_F64, h64->use_tma != 0, EPI_DOT, c->num_sms);
     Plo.gemv = gemv_plan(dtype, hlo->use_tma != 0, EPI_DOT, c->num_sms);
     P64.dA = c->dA;
