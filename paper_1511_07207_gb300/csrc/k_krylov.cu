@@ -298,6 +298,8 @@ __global__ void __launch_bounds__(KB) gm_start_kernel(Vecs v, cudaGraphCondition
         if (go == -1) set_err(st, ERRB_NAN);
         if (go == 0) st->status = LS_OK;
         if (go == -2) st->status = LS_NOT_CONVERGED;
+        // no new cycle: with x0, the gm_finish node that follows must not apply
+        // the previous cycle's correction a second time
         if (go != 1) st->k = 0;
         if (go == 1) {
             GmresSmall *gm = v.gm;

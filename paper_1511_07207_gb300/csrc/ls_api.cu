@@ -646,7 +646,9 @@ static int build_gs_graph(ls_ctx *c, const Vecs &v, const F64Layout &L, const Ge
     return finish_graph(c, c->graph_gs, R, key);
 }
 
-// Builds: gm_init, [resid GEMV if x0] gm_start, while(outer){ while(inner){GEMV, arnoldi}, gm_finish, resid GEMV, gm_start }
+// Builds: gm_init, and without x0 gm_start, while(outer){ while(inner){GEMV, arnoldi}, gm_finish, resid GEMV, gm_start };
+// with x0 while(outer){ resid GEMV, gm_start, while(inner){GEMV, arnoldi}, gm_finish }: gm_init
+// looks at b first, and no product is made when b = 0.
 static int build_gmres_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int x0_given,
                              const long long *key) {
     Root R;
@@ -676,9 +678,12 @@ static int build_gmres_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int 
         void *args[] = {&vv, &x0, &ho};
         top.kernel(c->K.gm_init, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
-    if (x0_given) residual(top);
-    start(top);
+    if (!x0_given) start(top);
     Chain outer = top.loop(ho);
+    if (x0_given) {
+        residual(outer);
+        start(outer);
+    }
     Chain inner = outer.loop(hi);
     {
         GemvArgs a{};
@@ -695,8 +700,10 @@ static int build_gmres_graph(ls_ctx *c, const Vecs &v, const GemvLaunch &L, int 
         void *args[] = {&vv};
         outer.kernel(c->K.gm_finish, vec_grid(c, v.n), c->K.block, 0, args, true);
     }
-    residual(outer);
-    start(outer);
+    if (!x0_given) {
+        residual(outer);
+        start(outer);
+    }
     if (top.err != cudaSuccess || inner.err != cudaSuccess || outer.err != cudaSuccess) {
         R.discard();
         return LS_ERR_CUDA;
@@ -857,7 +864,7 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
     } else if (method == LS_METHOD_CG || method == LS_METHOD_BICGSTAB) {
         passes = s.iter + s.cycles + (o.x0_given ? 1 : 0);
     } else {
-        passes = s.total + s.cycles + (o.x0_given ? 1 : 0);
+        passes = s.total + s.cycles + (o.x0_given && s.bnorm != 0.0 ? 1 : 0);
         sc.iter = s.total;
         sc.rnorm = s.est;   // the Givens estimate of the last step
     }
