@@ -58,20 +58,20 @@ cudaError_t set_smem_limit(const void *func, size_t smem) {
 
 
 // ---- workspace ----------------------------------------------------------------
+// Every cached graph (they hold pointers into the workspace).
+static void reset_graphs(ls_ctx *c) {
+    for (GraphCache *g : {&c->graph_cg, &c->graph_cg_sym, &c->graph_gm, &c->graph_mx, &c->graph_mx_sym, &c->graph_bs,
+                          &c->graph_ja, &c->graph_gs, &c->graph_bcg, &c->graph_bgm})
+        g->reset();
+}
+
 int ws_reserve(ls_ctx *c, size_t bytes) {
     if (bytes <= c->ws_bytes) return LS_OK;
     if (c->ws_user) return LS_ERR_NOMEM;
     if (c->ws) cudaFree(c->ws);
     c->ws = nullptr;
     c->ws_bytes = 0;
-    c->graph_cg.reset();
-    c->graph_gm.reset();
-    c->graph_mx.reset();
-    c->graph_bs.reset();
-    c->graph_ja.reset();
-    c->graph_gs.reset();
-    c->graph_bcg.reset();
-    c->graph_bgm.reset();
+    reset_graphs(c);
     cudaError_t e = cudaMalloc(&c->ws, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -315,14 +315,7 @@ extern "C" int ls_destroy(ls_ctx *c) {
     cudaSetDevice(c->device);
     if (c->stream) cudaStreamSynchronize(c->stream);
     else cudaDeviceSynchronize();
-    c->graph_cg.reset();
-    c->graph_gm.reset();
-    c->graph_mx.reset();
-    c->graph_bs.reset();
-    c->graph_ja.reset();
-    c->graph_gs.reset();
-    c->graph_bcg.reset();
-    c->graph_bgm.reset();
+    reset_graphs(c);
     extra_destroy(c);
     if (c->ws && !c->ws_user) cudaFree(c->ws);
     if (c->fixed) cudaFree(c->fixed);
@@ -340,14 +333,7 @@ extern "C" int ls_set_workspace(ls_ctx *c, void *ptr, size_t bytes) {
     cudaSetDevice(c->device);
     cudaStreamSynchronize(c->stream);
     if (c->ws && !c->ws_user) cudaFree(c->ws);
-    c->graph_cg.reset();
-    c->graph_gm.reset();
-    c->graph_mx.reset();
-    c->graph_bs.reset();
-    c->graph_ja.reset();
-    c->graph_gs.reset();
-    c->graph_bcg.reset();
-    c->graph_bgm.reset();
+    reset_graphs(c);
     c->ws = static_cast<char *>(ptr);
     c->ws_bytes = ptr ? bytes : 0;
     c->ws_user = ptr != nullptr;
@@ -507,7 +493,7 @@ static int build_cg_graph(ls_ctx *c, const Vecs &v, const Product &A, int x0_giv
         R.discard();
         return LS_ERR_CUDA;
     }
-    return finish_graph(c, c->graph_cg, R, key);
+    return finish_graph(c, A.sym ? c->graph_cg_sym : c->graph_cg, R, key);
 }
 
 // Builds: [resid GEMV if x0] bs_init, while(outer){ while(inner){GEMV v = A p (r^.v -> alpha),
@@ -782,9 +768,9 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
         if (rc) return rc;
         PR.sym = hs->asym == 0;
     }
-    long long key[8] = {method, n, (long long)(uintptr_t)c->ws, L.ldv, o.x0_given, hd->use_tma + 2 * PR.sym,
+    long long key[8] = {method, n, (long long)(uintptr_t)c->ws, L.ldv, o.x0_given, hd->use_tma,
                         (long long)(uintptr_t)c->stream, dt};
-    GraphCache &gc = method == LS_METHOD_CG         ? c->graph_cg
+    GraphCache &gc = method == LS_METHOD_CG         ? (PR.sym ? c->graph_cg_sym : c->graph_cg)
                      : method == LS_METHOD_BICGSTAB ? c->graph_bs
                      : method == LS_METHOD_JACOBI   ? c->graph_ja
                      : gs                           ? c->graph_gs

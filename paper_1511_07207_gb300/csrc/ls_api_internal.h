@@ -48,8 +48,9 @@ struct ls_ctx {
     char *ws = nullptr;
     size_t ws_bytes = 0;
     bool ws_user = false;
-    // cached executable graphs
-    lsi::GraphCache graph_cg, graph_gm, graph_mx, graph_bs, graph_ja, graph_gs, graph_bcg, graph_bgm;
+    // cached executable graphs (CG with the product from one triangle has its own: a
+    // caller may alternate between matrices of either kind)
+    lsi::GraphCache graph_cg, graph_cg_sym, graph_gm, graph_mx, graph_mx_sym, graph_bs, graph_ja, graph_gs, graph_bcg, graph_bgm;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     long long launches_total = 0;
     lsi::Engine *batch = nullptr;

@@ -158,7 +158,7 @@ static int build_mixed_graph(ls_ctx *c, const MixVecs &v, const Product &A64, co
         R.discard();
         return LS_ERR_CUDA;
     }
-    return finish_graph(c, c->graph_mx, R, key);
+    return finish_graph(c, A64.sym ? c->graph_mx_sym : c->graph_mx, R, key);
 }
 
 int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double *b, double *x,
@@ -257,12 +257,13 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     P64.dA = c->dA;
     Plo.dA = c->dA + 1;
     long long key[8] = {100 + o.refine, n, (long long)(uintptr_t)c->ws, dtype * 2 + (split ? 1 : 0), o.x0_given,
-                        h64->use_tma * 2 + hlo->use_tma + 4 * sym, (long long)(uintptr_t)c->stream, m};
-    if (!c->graph_mx.matches(key)) {
+                        h64->use_tma * 2 + hlo->use_tma, (long long)(uintptr_t)c->stream, m};
+    GraphCache &gc = sym ? c->graph_mx_sym : c->graph_mx;
+    if (!gc.matches(key)) {
         rc = build_mixed_graph(c, v, P64, Plo, o.x0_given, key);
         if (rc) return rc;
     }
-    rc = launch_cached(c, c->graph_mx);
+    rc = launch_cached(c, gc);
     if (rc) return rc;
     e = cudaEventRecord(c->ev1, c->stream);
     if (e != cudaSuccess) return map_cuda(e);
