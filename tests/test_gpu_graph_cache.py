@@ -46,3 +46,36 @@ def test_alternating_symmetry(ctx, gpu, precision):
         call(mats[1])
 
     assert _median(both) <= 1.3 * apart
+
+
+TIMED = {
+    "cg": ("spd", B.ls_cg_solve, {"fused": 0}, 200),
+    "cg_one_triangle": ("spd", B.ls_cg_solve, {"fused": 0}, 1030),
+    "gmres": ("nonsym", B.ls_gmres_solve, {"fused": 0}, 200),
+    "bicgstab": ("nonsym", B.ls_bicgstab_solve, {}, 200),
+    "jacobi": ("nonsym", B.ls_jacobi_solve, {}, 200),
+    "gauss_seidel": ("nonsym", B.ls_gauss_seidel_solve, {}, 200),
+    "mixed": ("spd", B.ls_cg_solve, {"precision": B.LS_F32_IR, "inner_iters": 1}, 200),
+    "mixed_one_triangle": ("spd", B.ls_cg_solve, {"precision": B.LS_F32_IR, "inner_iters": 1}, 1030),
+}
+
+
+@pytest.mark.parametrize("name", list(TIMED))
+def test_time_of_a_call_that_builds_its_graph(ctx, gpu, name):
+    """time_ms of the first call of a size is that of the second; building and instantiating a graph
+    would add 0.2 ms or more to a solve of a step or two (kernels are loaded by a call of another size)."""
+    kind, solve, kw, n = TIMED[name]
+    o = B.make_opts(rtol=1e-10, max_iter=2, **kw)
+    ms = {}
+    for m in (n, n + 8, n, n + 8):
+        A = inputs.spd_matrix(m, 0.1, seed=660) if kind == "spd" else inputs.nonsym_matrix(m, seed=661)
+        Ad = torch.from_numpy(A).to(gpu)
+        b = torch.from_numpy(A @ inputs.solution(m, seed=662)).to(gpu)
+        x = torch.zeros(m, dtype=torch.float64, device=gpu)
+        ms.setdefault(m, [])
+        for _ in range(5):
+            ms[m].append(solve(ctx, Ad, b, x, o)[1]["time_ms"])
+    # every fifth call built a graph: the calls at n + 8 when the kernels had been loaded
+    first = min(ms[n + 8][0], ms[n + 8][5])
+    rest = sorted(ms[n + 8][1:5] + ms[n + 8][6:])[4]
+    assert first <= 1.5 * rest + 0.05
