@@ -241,7 +241,8 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     hs->m = m;
     hs->in_max = o.inner_iters;
     hs->in_tol2 = o.inner_rtol > 0.0 ? (float)(o.inner_rtol * o.inner_rtol) : -1.0f;
-    hs->launches = split ? 2 : 1;   // the quantisation (and split or packing) kernels
+    // the quantisation (and split) kernels, or both packing ones; a packing that found A not symmetric
+    hs->launches = (split ? 2 : 1) + (want_sym && !sym);
     if (!rc) rc = upload_state(c);
     if (rc) return rc;
 
