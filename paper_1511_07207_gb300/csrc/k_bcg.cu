@@ -740,7 +740,6 @@ __global__ void __launch_bounds__(BK) bcgd_step_kernel(BcgVecs v, cudaGraphCondi
     if (!flag_s) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             st->status = LS_BREAKDOWN;
-            sm->ok = 0;
             set_cond(st, h_inner, 0u);
         }
         return;

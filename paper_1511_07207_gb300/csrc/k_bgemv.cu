@@ -66,11 +66,8 @@ __host__ __device__ constexpr int bg_rows_per_warp() {
     return S <= 8 ? 1 : 2;
 }
 // Accumulators a column: one row per warp (S <= 8) keeps the two column chunks apart (two
-// independent chains per column of P), added at the end of the row block.
-template <int S>
-__host__ __device__ constexpr int bg_accs() {
-    return 2;
-}
+// independent chains per column of P), added at the end of the row block; two rows have one each.
+constexpr int BG_ACCS = 2;
 template <int S>
 __host__ __device__ constexpr int bg_consumers() {
     return 32 * 16 / bg_rows_per_warp<S>();
@@ -96,8 +93,8 @@ __host__ __device__ constexpr size_t stage_bytes() {
 
 // A warp's share of one 16 x 256 tile in a ring stage: rows w, w + WS, ..., lane g's 4-column chunks.
 template <int S>
-__device__ __forceinline__ void bg_tile(F2 (&acc)[bg_accs<S>()][S], const unsigned char *base, int w, int g) {
-    constexpr int RPW = bg_rows_per_warp<S>(), WS = 16 / RPW, NA = bg_accs<S>() / RPW;
+__device__ __forceinline__ void bg_tile(F2 (&acc)[BG_ACCS][S], const unsigned char *base, int w, int g) {
+    constexpr int RPW = bg_rows_per_warp<S>(), WS = 16 / RPW, NA = BG_ACCS / RPW;
     const float *Ah = reinterpret_cast<const float *>(base);
     const float *Al = reinterpret_cast<const float *>(base + BG_A_B);
     const float *Xh = reinterpret_cast<const float *>(base + 2 * BG_A_B);
@@ -220,7 +217,7 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
     // warp w: rows w, w + WS, ... of the block (RPW of them); lane g: the
     // 4-column chunks g and g + 32 of each tile
     const int w = threadIdx.x >> 5, g = threadIdx.x & 31;
-    constexpr int NA = bg_accs<S>() / RPW;
+    constexpr int NA = BG_ACCS / RPW;
     int seq = 0;
     bool ok = true;
     for (int rb = first_rb; seq < ntiles; rb += rb_step) {
@@ -271,7 +268,7 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
                         for (int j = 0; j < S; j++)
                             if (j < a.s) a.Q[(long long)j * a.ldq + row] = (double)acc[q][j].h + (double)acc[q][j].l;
                 }
-        } else {
+        } else if constexpr (S < 16) {
             // shared with neighbouring CTAs: publish the partial sums; the last of
             // the sharing CTAs adds them in CTA order
             double *fix = a.scr->fix + (size_t)(2 * blockIdx.x + (rb == first_rb ? 0 : 1)) * BG_TR * S;

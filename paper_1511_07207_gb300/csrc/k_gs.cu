@@ -20,7 +20,7 @@
 //     is in, they publish u_I = T_I^-1 (r_I - sum_j A_{I,j} d_j);
 //   * in every CTA one producer lane streams the CTA's fixed sequence of
 //     64 x 64 tiles (hi and lo) into a ring of shared-memory slots (mbarrier
-//     full/empty), so the tiles arrive ahead of the flags that gate their
+//     full/empty), so the tiles arrive ahead of the words that gate their
 //     use; sixteen consumer warps compute.  Helpers load with 2-D TMA
 //     (128-byte swizzle, zero fill past n); the chain's M_{I,w} sit in a
 //     contiguous panel in its threads' read order, one 32 KB bulk copy per
@@ -341,7 +341,7 @@ __device__ __forceinline__ int gs_owned_list(int g, int H, int nblk, int *I) {
 }
 
 // Producer lane: the CTA's tiles in the order its consumers take them
-// (chain: A_{I,I-1}, A_{I,I-2}, T_I for I = 0, 1, ...; helper: for each owned
+// (chain: M_{I,W} .. M_{I,1} of the panel for I = 0, 1, ...; helper: for each owned
 // block A_{I,0} .. A_{I,I-W-1}, T_I).  Before returning it waits for the
 // copies of the last ring's worth of tiles, so none is in flight at exit.
 __device__ void gs_produce(const GsArgs &a, int nblk, GsShared *S, unsigned char *ring, bool chain) {

@@ -171,9 +171,6 @@ __device__ __forceinline__ int atom_add_acq_rel(int *p, int v) {
     asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
     return old;
 }
-__device__ __forceinline__ void st_release_u32(unsigned *p, unsigned v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
 
 // All blocks of the grid meet here.  Returns false (and sets ERRB_TIMEOUT)
 // if the others did not arrive within WAIT_LIMIT_NS.  The arrivals of one barrier

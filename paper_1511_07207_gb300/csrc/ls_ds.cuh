@@ -34,13 +34,10 @@ __device__ __forceinline__ DSV settled(DSV a) {
     return DSV{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
 }
 __device__ __forceinline__ float settled(float a) { return a; }
-__device__ __forceinline__ double settled(double a) { return a; }
 // Sums of finished partial sums.
 template <class V>
 __device__ __forceinline__ V settled_sum(V a, V b) { return settled(a + b); }
 __device__ __forceinline__ double to_double(DSV v) { return (double)v.h + (double)v.l; }
-__device__ __forceinline__ double to_double(double v) { return v; }
-__device__ __forceinline__ float to_double(float v) { return v; }
 __device__ __forceinline__ float shfl_xor_v(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ double shfl_xor_v(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ DSV shfl_xor_v(DSV v, int o) {

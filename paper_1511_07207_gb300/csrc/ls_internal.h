@@ -93,8 +93,6 @@ struct GmresSmall {
     double H[(LS_MAX_RESTART + 1) * LS_MAX_RESTART];  // rotated Hessenberg, column-major
     double cs[LS_MAX_RESTART], sn[LS_MAX_RESTART];
     double g[LS_MAX_RESTART + 1];
-    double y[LS_MAX_RESTART];
-    double h[LS_MAX_RESTART + 1];                     // current column (projection)
 };
 
 // ---- per-launch scratch of the persistent GEMV --------------------------------
@@ -273,9 +271,7 @@ struct BcgSmall {                 // s x s matrices, column-major, leading dimen
     double bn[BCG_MAX_S];                  // ||B_j||
     double r2[BCG_MAX_S];                  // ||B_j - A X_j||^2 from the residual GEMVs
     int ok, update_p;
-    // deflating form: leading dimension BCG_MAX_S for every small matrix
-    double T[BCG_MAX_S * BCG_MAX_S];       // P = W T (the current orthogonalization pass)
-    double Lg[BCG_MAX_S * BCG_MAX_S];      // Cholesky factor of gamma = P^T Q (rank x rank)
+    // deflating form
     double w2[BCG_MAX_S];                  // ||W_j||^2 of the block being orthogonalized
     int rank;                              // orthonormal directions in P (its first columns)
 };
