@@ -103,7 +103,7 @@ template <int DT>
 __host__ __device__ constexpr int stages() { return Cfg<DT>::PARTS > 1 ? 3 : GEMV_STAGES; }
 
 template <int DT>
-__device__ constexpr GemvCosts costs() {
+constexpr GemvCosts costs() {
     return DT == DT_DS ? GEMV_COSTS_PAIR : DT == DT_BF16 ? GEMV_COSTS_BF16 : DT == DT_FP8 ? GEMV_COSTS_FP8 : GEMV_COSTS_F32;
 }
 
@@ -244,6 +244,12 @@ __device__ __forceinline__ void dot_global(const typename Cfg<DT>::T *A, const t
     }
 }
 
+// A row's sum.
+template <int DT, class S>
+__device__ __forceinline__ double row_value(S s) {
+    if constexpr (DT == DT_DS) return to_double(s);
+    else return pair_value(s);
+}
 // FP8: the row's scale
 template <int DT>
 __device__ __forceinline__ typename Cfg<DT>::Y scaled(const MatDesc &M, int row, typename Cfg<DT>::Y s) {
@@ -264,7 +270,10 @@ __device__ __forceinline__ int tile_owner(long long t, long long T, int G) {
     return (int)(((long long)G * (t + 1) + T - 1) / T) - 1;
 }
 
-template <int DT, bool TMA>
+// WHOLE: a CTA takes one whole row tile instead of an equal piece of the tile sequence
+// (gemv_split.h).  A kernel of its own: with both loops in one, the product in equal
+// pieces took 2 % longer at n = 16384 (332 against 326 us, caches cold).
+template <int DT, bool TMA, bool WHOLE>
 __global__ void __launch_bounds__(GEMV_THREADS, 2)
     gemv_kernel(const MatDesc *__restrict__ dA, GemvArgs args) {
     using C = Cfg<DT>;
@@ -283,7 +292,13 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
     T *ring = reinterpret_cast<T *>(smem_raw);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem_raw + (size_t)NST * G::TILE_BYTES * C::PARTS);
     uint64_t *empty = full + NST;
-    using S = decltype(as_sum(V{}));          // a row's sums: pairs for the FP32 formats too
+    // A row's sums.  A whole row is a longer chain than an equal piece, so its error is kept
+    // down to that of the pieces: the lanes' sums are added as pairs (settled ones
+    // for the FP32 pair), and the FP32 formats' accumulators go into a sum of their own
+    // after every second tile (PART).  Equal pieces are added in FP64 and need neither.
+    using S = typename std::conditional<WHOLE, decltype(as_sum(V{})), V>::type;
+    constexpr bool SETTLED = WHOLE && DT == DT_DS;
+    constexpr bool PART = WHOLE && std::is_same<V, float>::value;
     __shared__ S red[WC][TR];
     __shared__ double dred[GEMV_THREADS / 32];
     __shared__ int abort_s, last_s, fin_s, ca_s, cb_s;
@@ -301,12 +316,8 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
     const int RT = (rows + TR - 1) / TR, CT = (cols + TC - 1) / TC;
     const long long T_all = (long long)RT * CT;
     const int G_ = gridDim.x, cta = blockIdx.x;
-    // Equal pieces, or one whole row tile a CTA where the meetings of equal pieces cost more than
-    // the SMs that stay idle (gemv_split.h).  The native FP64 product is bound by the
-    // FP64 pipe and keeps the equal pieces, which use every SM.
-    const bool whole = DT != DT_F64 && gemv_whole_tiles(costs<DT>(), RT, CT, G_);
-    const long long t0 = whole ? (long long)min(cta, RT) * CT : tile_start(T_all, cta, G_);
-    const long long t1 = whole ? (long long)min(cta + 1, RT) * CT : tile_start(T_all, cta + 1, G_);
+    const long long t0 = WHOLE ? (long long)min(cta, RT) * CT : tile_start(T_all, cta, G_);
+    const long long t1 = WHOLE ? (long long)min(cta + 1, RT) * CT : tile_start(T_all, cta + 1, G_);
     const int ntiles = (int)(t1 - t0);
     count_launch(args.st);
 
@@ -380,140 +391,127 @@ __global__ void __launch_bounds__(GEMV_THREADS, 2)
 
         // With one CTA on most SMs (whole row tiles) x of a tile is asked for while the tile before
         // it is worked on (Jacobi, n = 2500: 0.53 -> 0.47 ms); with two the other
-        // CTA hides that latency, and asking early costs 3 % at n = 16384.  Two copies of
-        // the loop: deciding inside it cost 1.7 % there.
-        auto tiles = [&](auto ahead) {
-            constexpr bool AHEAD = decltype(ahead)::value;
-            // A whole row is a longer chain than an equal piece, so its error is kept down to that
-            // of the pieces: the lanes' sums are added as pairs (settled ones for the
-            // FP32 pair), and the FP32 formats' accumulators go into a sum of their own after every
-            // second tile.  Equal pieces are added in FP64 and need neither.
-            constexpr bool SETTLED = AHEAD && DT == DT_DS;
-            constexpr bool PART = AHEAD && std::is_same<V, float>::value;
-            using L = typename std::conditional<AHEAD, S, V>::type;
-            V part[RW];
+        // CTA hides that latency, and asking early costs 3 % at n = 16384.
+        V part[RW];
 #pragma unroll
-            for (int r = 0; r < RW; r++) part[r] = V{};
-            X xv[VEC];
-            if constexpr (AHEAD)
-                if (ntiles > 0) load_x<DT>(x, lane_col, cols, xv);
-            for (int i = 0; i < ntiles; i++) {
-                V p[VEC];
-                if constexpr (!AHEAD) load_x<DT>(x, ct * TC + lane_col, cols, xv);
+        for (int r = 0; r < RW; r++) part[r] = V{};
+        X xv[VEC];
+        if constexpr (WHOLE)
+            if (ntiles > 0) load_x<DT>(x, lane_col, cols, xv);
+        for (int i = 0; i < ntiles; i++) {
+            V p[VEC];
+            if constexpr (!WHOLE) load_x<DT>(x, ct * TC + lane_col, cols, xv);
 #pragma unroll
-                for (int k = 0; k < VEC; k++) to_operand<AHEAD>(xv[k], p[k]);
-                if constexpr (AHEAD)
-                    if (i + 1 < ntiles) load_x<DT>(x, (ct + 1) * TC + lane_col, cols, xv);
-                if (TMA) {
-                    // On a timeout the warp stops waiting and computing but keeps
-                    // walking the tile sequence, so it still meets the other
-                    // consumer warps at every named barrier below.
-                    const int s = i % NST;
-                    if (!*(volatile int *)&abort_s && !mbar_wait(&full[s], (i / NST) & 1)) {
-                        set_err(args.st, ERRB_TIMEOUT);
-                        abort_s = 1;
-                    }
-                    if (!*(volatile int *)&abort_s) {
-                        const T *tile = ring + (size_t)s * STAGE_ELEMS;
+            for (int k = 0; k < VEC; k++) to_operand<WHOLE>(xv[k], p[k]);
+            if constexpr (WHOLE)
+                if (i + 1 < ntiles) load_x<DT>(x, (ct + 1) * TC + lane_col, cols, xv);
+            if (TMA) {
+                // On a timeout the warp stops waiting and computing but keeps
+                // walking the tile sequence, so it still meets the other
+                // consumer warps at every named barrier below.
+                const int s = i % NST;
+                if (!*(volatile int *)&abort_s && !mbar_wait(&full[s], (i / NST) & 1)) {
+                    set_err(args.st, ERRB_TIMEOUT);
+                    abort_s = 1;
+                }
+                if (!*(volatile int *)&abort_s) {
+                    const T *tile = ring + (size_t)s * STAGE_ELEMS;
 #pragma unroll
-                        for (int r = 0; r < RW; r++)
-                            dot_tile<DT>(tile + (wr * RW + r) * TC + lane_col, p, acc[r], acc1[r]);
-                    }
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&empty[s]);
-                } else {
+                    for (int r = 0; r < RW; r++)
+                        dot_tile<DT>(tile + (wr * RW + r) * TC + lane_col, p, acc[r], acc1[r]);
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&empty[s]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < RW; r++) {
+                    const int row = rt * TR + wr * RW + r;
+                    if (row < rows)
+                        dot_global<DT>(Ag, Agl, M.lda, row, ct * TC + lane_col, cols, p, acc[r], acc1[r]);
+                }
+            }
+            if constexpr (PART)
+                if (i & 1) {
 #pragma unroll
                     for (int r = 0; r < RW; r++) {
-                        const int row = rt * TR + wr * RW + r;
-                        if (row < rows)
-                            dot_global<DT>(Ag, Agl, M.lda, row, ct * TC + lane_col, cols, p, acc[r], acc1[r]);
+                        part[r] = part[r] + (acc[r] + acc1[r]);
+                        acc[r] = acc1[r] = V{};
                     }
                 }
-                if constexpr (PART)
-                    if (i & 1) {
+            if (ct == CT - 1 || i == ntiles - 1) {
+                // this CTA's share of row tile rt is done: reduce it over the warp
+                S sum[RW];
 #pragma unroll
-                        for (int r = 0; r < RW; r++) {
-                            part[r] = part[r] + (acc[r] + acc1[r]);
-                            acc[r] = acc1[r] = V{};
-                        }
-                    }
-                if (ct == CT - 1 || i == ntiles - 1) {
-                    // this CTA's share of row tile rt is done: reduce it over the warp
-                    L sum[RW];
+                for (int r = 0; r < RW; r++) {
+                    if constexpr (WHOLE) sum[r] = join<SETTLED>(as_sum(acc[r]), as_sum(acc1[r]));
+                    else sum[r] = acc[r] + acc1[r];
+                    if constexpr (PART) sum[r] = join<SETTLED>(as_sum(part[r]), sum[r]);
+                    acc[r] = acc1[r] = part[r] = V{};
+                }
+                butterfly<RW, 16, SETTLED>(sum, lane);
+                if ((lane & ((32 >> LGR) - 1)) == 0) red[wc][wr * RW + (lane >> (5 - LGR))] = sum[0];
+                consumers_sync();
+                const long long rfirst = (long long)rt * CT;
+                const bool complete = WHOLE || ((t0 <= rfirst) && (rfirst + CT <= t1));
+                if (complete) {
+                    for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
+                        S s{};
 #pragma unroll
-                    for (int r = 0; r < RW; r++) {
-                        if constexpr (AHEAD) sum[r] = join<SETTLED>(as_sum(acc[r]), as_sum(acc1[r]));
-                        else sum[r] = acc[r] + acc1[r];
-                        if constexpr (PART) sum[r] = join<SETTLED>(as_sum(part[r]), sum[r]);
-                        acc[r] = acc1[r] = part[r] = V{};
+                        for (int c = 0; c < WC; c++) s = join<SETTLED>(s, red[c][tr]);
+                        const int row = rt * TR + tr;
+                        if (row < rows) mydot += epilogue<Y>(args, row, scaled<DT>(M, row, (Y)row_value<DT>(s)));
                     }
-                    butterfly<RW, 16, SETTLED>(sum, lane);
-                    if ((lane & ((32 >> LGR) - 1)) == 0) red[wc][wr * RW + (lane >> (5 - LGR))] = as_sum(sum[0]);
+                } else {
+                    // A row tile shared with neighbouring CTAs: publish the
+                    // partial sums; the last of the sharing CTAs to arrive adds
+                    // them in CTA order and finishes those rows.
+                    const int slot = (rt == first_rt) ? 0 : 1;
+                    for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
+                        S s{};
+#pragma unroll
+                        for (int c = 0; c < WC; c++) s = join<SETTLED>(s, red[c][tr]);
+                        args.scr->fix[((size_t)cta * 2 + slot) * TR + tr] = row_value<DT>(s);
+                        __threadfence();
+                    }
                     consumers_sync();
-                    const long long rfirst = (long long)rt * CT;
-                    const bool complete = (t0 <= rfirst) && (rfirst + CT <= t1);
-                    if (complete) {
+                    if (threadIdx.x == 0) {
+                        const int ca = tile_owner(rfirst, T_all, G_);
+                        const int cb = tile_owner(rfirst + CT - 1, T_all, G_);
+                        int ncov = 0;
+                        for (int c = ca; c <= cb; c++)
+                            ncov += tile_start(T_all, c, G_) < tile_start(T_all, c + 1, G_);
+                        const unsigned prev = atomicAdd(&args.scr->bticket[ca], 1u);
+                        fin_s = (prev == (unsigned)ncov - 1);
+                        if (fin_s) atomicExch(&args.scr->bticket[ca], 0u);
+                        ca_s = ca;
+                        cb_s = cb;
+                    }
+                    consumers_sync();
+                    if (fin_s) {
+                        __threadfence();
                         for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                            S s{};
-#pragma unroll
-                            for (int c = 0; c < WC; c++) s = join<SETTLED>(s, red[c][tr]);
+                            double s = 0.0;
+                            for (int c = ca_s; c <= cb_s; c++) {
+                                const long long a0 = tile_start(T_all, c, G_);
+                                if (tile_start(T_all, c + 1, G_) <= a0) continue;   // empty CTA
+                                const int sl = (rt == (int)(a0 / CT)) ? 0 : 1;
+                                s += __ldcg(&args.scr->fix[((size_t)c * 2 + sl) * TR + tr]);
+                            }
                             const int row = rt * TR + tr;
-                            if (row < rows) mydot += epilogue<Y>(args, row, scaled<DT>(M, row, (Y)pair_value(s)));
-                        }
-                    } else {
-                        // A row tile shared with neighbouring CTAs: publish the
-                        // partial sums; the last of the sharing CTAs to arrive adds
-                        // them in CTA order and finishes those rows.
-                        const int slot = (rt == first_rt) ? 0 : 1;
-                        for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                            S s{};
-#pragma unroll
-                            for (int c = 0; c < WC; c++) s = join<SETTLED>(s, red[c][tr]);
-                            args.scr->fix[((size_t)cta * 2 + slot) * TR + tr] = pair_value(s);
-                            __threadfence();
+                            tdot[tr] = row < rows ? epilogue<Y>(args, row, scaled<DT>(M, row, (Y)s)) : 0.0;
                         }
                         consumers_sync();
                         if (threadIdx.x == 0) {
-                            const int ca = tile_owner(rfirst, T_all, G_);
-                            const int cb = tile_owner(rfirst + CT - 1, T_all, G_);
-                            int ncov = 0;
-                            for (int c = ca; c <= cb; c++)
-                                ncov += tile_start(T_all, c, G_) < tile_start(T_all, c + 1, G_);
-                            const unsigned prev = atomicAdd(&args.scr->bticket[ca], 1u);
-                            fin_s = (prev == (unsigned)ncov - 1);
-                            if (fin_s) atomicExch(&args.scr->bticket[ca], 0u);
-                            ca_s = ca;
-                            cb_s = cb;
-                        }
-                        consumers_sync();
-                        if (fin_s) {
-                            __threadfence();
-                            for (int tr = threadIdx.x; tr < TR; tr += GEMV_CONSUMER_WARPS * 32) {
-                                double s = 0.0;
-                                for (int c = ca_s; c <= cb_s; c++) {
-                                    const long long a0 = tile_start(T_all, c, G_);
-                                    if (tile_start(T_all, c + 1, G_) <= a0) continue;   // empty CTA
-                                    const int sl = (rt == (int)(a0 / CT)) ? 0 : 1;
-                                    s += __ldcg(&args.scr->fix[((size_t)c * 2 + sl) * TR + tr]);
-                                }
-                                const int row = rt * TR + tr;
-                                tdot[tr] = row < rows ? epilogue<Y>(args, row, scaled<DT>(M, row, (Y)s)) : 0.0;
-                            }
-                            consumers_sync();
-                            if (threadIdx.x == 0) {
-                                double d = 0.0;
-                                for (int tr = 0; tr < TR; tr++) d += tdot[tr];
-                                args.scr->fixdot[ca_s] = d;
-                            }
+                            double d = 0.0;
+                            for (int tr = 0; tr < TR; tr++) d += tdot[tr];
+                            args.scr->fixdot[ca_s] = d;
                         }
                     }
-                    consumers_sync();
                 }
-                if (++ct == CT) { ct = 0; ++rt; }
+                consumers_sync();
             }
-        };
-        if (whole) tiles(std::true_type{});
-        else tiles(std::false_type{});
+            if (++ct == CT) { ct = 0; ++rt; }
+        }
     }
 
     // ---- per-CTA dot; the last CTA reduces them (all threads, fixed order) ----
@@ -543,41 +541,46 @@ static size_t gemv_smem() {
     return (size_t)stages<DT>() * Geo<DT>::TILE_BYTES * Cfg<DT>::PARTS + 2 * stages<DT>() * sizeof(uint64_t);
 }
 
-template <int DT, bool TMA>
-static void *gemv_func() {
-    return reinterpret_cast<void *>(&gemv_kernel<DT, TMA>);
+template <int DT>
+static void *gemv_func(bool tma, int rows, int cols, int grid) {
+    if constexpr (DT != DT_F64) {   // the native FP64 product, bound by the FP64 pipe, keeps every SM
+        const int RT = (rows + Geo<DT>::TR - 1) / Geo<DT>::TR, CT = (cols + Geo<DT>::TC - 1) / Geo<DT>::TC;
+        if (gemv_whole_tiles(costs<DT>(), RT, CT, grid))
+            return tma ? reinterpret_cast<void *>(&gemv_kernel<DT, true, true>)
+                       : reinterpret_cast<void *>(&gemv_kernel<DT, false, true>);
+    }
+    return tma ? reinterpret_cast<void *>(&gemv_kernel<DT, true, false>)
+               : reinterpret_cast<void *>(&gemv_kernel<DT, false, false>);
 }
 
-GemvLaunch gemv_plan(int dtype, bool use_tma, int epi, int num_sms) {
-    (void)epi;
+GemvLaunch gemv_plan(int dtype, bool use_tma, int rows, int cols, int num_sms) {
     GemvLaunch L{};
     L.block = GEMV_THREADS;
-    L.grid = 2 * num_sms;
+    L.grid = 2 * num_sms < MAX_GRID ? 2 * num_sms : MAX_GRID;
     switch (dtype) {
         case DT_F64:
-            L.func = use_tma ? gemv_func<DT_F64, true>() : gemv_func<DT_F64, false>();
+            L.func = gemv_func<DT_F64>(use_tma, rows, cols, L.grid);
             L.smem = gemv_smem<DT_F64>();
             break;
         case DT_DS:
-            L.func = use_tma ? gemv_func<DT_DS, true>() : gemv_func<DT_DS, false>();
+            L.func = gemv_func<DT_DS>(use_tma, rows, cols, L.grid);
             L.smem = gemv_smem<DT_DS>();
             break;
         case DT_BF16:
-            L.func = use_tma ? gemv_func<DT_BF16, true>() : gemv_func<DT_BF16, false>();
+            L.func = gemv_func<DT_BF16>(use_tma, rows, cols, L.grid);
             L.smem = gemv_smem<DT_BF16>();
             break;
         case DT_FP8:
-            L.func = use_tma ? gemv_func<DT_FP8, true>() : gemv_func<DT_FP8, false>();
+            L.func = gemv_func<DT_FP8>(use_tma, rows, cols, L.grid);
             L.smem = gemv_smem<DT_FP8>();
             break;
         default:
-            L.func = use_tma ? gemv_func<DT_F32, true>() : gemv_func<DT_F32, false>();
+            L.func = gemv_func<DT_F32>(use_tma, rows, cols, L.grid);
             L.smem = gemv_smem<DT_F32>();
             break;
     }
     if (!use_tma) L.smem = 2 * GEMV_STAGES * sizeof(uint64_t);   // barriers only (no ring)
     set_smem_limit(L.func, L.smem);
-    if (L.grid > MAX_GRID) L.grid = MAX_GRID;
     return L;
 }
 

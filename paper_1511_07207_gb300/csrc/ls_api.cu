@@ -749,7 +749,7 @@ static int krylov_f64(ls_ctx *c, int method, int n, const double *A, int64_t lda
 
     Vecs v = make_vecs(c, L, n);
     const int dt = split ? DT_DS : DT_F64;
-    GemvLaunch GL = gemv_plan(dt, hd->use_tma != 0, EPI_DOT, c->num_sms);
+    GemvLaunch GL = gemv_plan(dt, hd->use_tma != 0, n, n, c->num_sms);
     // CG: the packed triangle takes the place of the pair when A is exactly symmetric
     Product PR{};
     PR.gemv = GL;
@@ -980,7 +980,7 @@ extern "C" int ls_gemv(ls_ctx *c, int dtype, int rows, int cols, const void *A, 
     state_init(c->h_st, 0);
     rc = upload_state(c);
     if (rc) return rc;
-    GemvLaunch L = gemv_plan(dtype, hd->use_tma != 0, EPI_STORE, c->num_sms);
+    GemvLaunch L = gemv_plan(dtype, hd->use_tma != 0, rows, cols, c->num_sms);
     GemvArgs a{};
     a.x = x;
     a.y = y;
@@ -1013,7 +1013,7 @@ extern "C" int ls_gemv_timed(ls_ctx *c, int dtype, int rows, int cols, const voi
     state_init(c->h_st, 0);
     rc = upload_state(c);
     if (rc) return rc;
-    GemvLaunch L = gemv_plan(dtype, hd->use_tma != 0, EPI_STORE, c->num_sms);
+    GemvLaunch L = gemv_plan(dtype, hd->use_tma != 0, rows, cols, c->num_sms);
     GemvArgs a{};
     a.x = x;
     a.y = y;

@@ -215,7 +215,7 @@ extern "C" int ls_block_cg_solve(ls_ctx *c, int n, int s, const double *A, int64
     v.bar = c->bar;
     v.st = c->st;
     const int dt = split ? DT_DS : DT_F64;
-    GemvLaunch GL = gemv_plan(dt, hd->use_tma != 0, EPI_DOT, c->num_sms);
+    GemvLaunch GL = gemv_plan(dt, hd->use_tma != 0, n, n, c->num_sms);
     const int deflate = o.deflate ? 1 : 0;
     long long key[8] = {200 + s + 100 * deflate, n, (long long)(uintptr_t)c->ws, L.ld, o.x0_given, hd->use_tma,
                         (long long)(uintptr_t)c->stream, dt};

@@ -21,6 +21,7 @@ __device__ __forceinline__ DSV as_sum(float v) { return DSV{v, 0.0f}; }
 __device__ __forceinline__ DSV as_sum(DSV v) { return v; }
 __device__ __forceinline__ double as_sum(double v) { return v; }
 __device__ __forceinline__ double pair_value(double v) { return v; }
+__device__ __forceinline__ float pair_value(float v) { return v; }
 __device__ __forceinline__ double pair_value(DSV v) { return isfinite(v.h) ? to_double(v) : (double)v.h; }
 
 // Butterfly transpose-reduction of RW per-lane row accumulators over the warp:

@@ -146,8 +146,8 @@ struct GemvLaunch {
     int grid, block;
     size_t smem;
 };
-// Choose the kernel for a matrix (TMA or plain-load variant) and epilogue.
-GemvLaunch gemv_plan(int dtype, bool use_tma, int epi, int num_sms);
+// Choose the kernel for a matrix (TMA or plain loads; whole row tiles or equal pieces).
+GemvLaunch gemv_plan(int dtype, bool use_tma, int rows, int cols, int num_sms);
 // Raise a kernel's dynamic shared-memory limit to at least smem bytes on the
 // current device.  The attribute is per device: it is set again only for a
 // new (kernel, device) pair or a larger size.  Safe from several host threads.

@@ -155,7 +155,7 @@ extern "C" int ls_lu_solve(ls_ctx *c, int n, const double *A, int64_t lda, const
     rc = upload_desc(c, 1);
     if (rc) return rc;
     cudaError_t e = cudaMemcpyAsync(L.r, b, sizeof(double) * n, cudaMemcpyDefault, c->stream);
-    GemvLaunch GL = gemv_plan(DT_F64, hd->use_tma != 0, EPI_RESID, c->num_sms);
+    GemvLaunch GL = gemv_plan(DT_F64, hd->use_tma != 0, n, n, c->num_sms);
     GemvArgs ga{};
     ga.x = L.x;
     ga.y = L.r;

@@ -253,8 +253,8 @@ int mixed_cg_solve(ls_ctx *c, int n, const double *A, int64_t lda, const double 
     v.dvals = L.dvals;
     v.rf = L.rf; v.zf = L.zf; v.pf = L.pf; v.qf = L.qf;
     v.part = c->part; v.bar = c->bar; v.st = c->st;
-    P64.gemv = gemv_plan(split ? DT_DS : DT_F64, h64->use_tma != 0, EPI_DOT, c->num_sms);
-    Plo.gemv = gemv_plan(dtype, hlo->use_tma != 0, EPI_DOT, c->num_sms);
+    P64.gemv = gemv_plan(split ? DT_DS : DT_F64, h64->use_tma != 0, n, n, c->num_sms);
+    Plo.gemv = gemv_plan(dtype, hlo->use_tma != 0, n, n, c->num_sms);
     P64.dA = c->dA;
     Plo.dA = c->dA + 1;
     long long key[8] = {100 + o.refine, n, (long long)(uintptr_t)c->ws, dtype * 2 + (split ? 1 : 0), o.x0_given,

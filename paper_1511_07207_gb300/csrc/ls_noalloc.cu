@@ -82,7 +82,7 @@ extern "C" int ls_gemv_noalloc(int dtype, int rows, int cols, const void *A, int
     int sms = 0;
     int rc = scratch_for_current_device(&base, &sms);
     if (rc) return rc;
-    GemvLaunch L = gemv_plan(dtype, true, EPI_STORE, sms);
+    GemvLaunch L = gemv_plan(dtype, true, rows, cols, sms);
     if (L.grid > LS_NOALLOC_MAX_CTAS) return LS_ERR_UNSUPPORTED;   // partial sums would not fit
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -95,7 +95,7 @@ extern "C" int ls_gemv_noalloc(int dtype, int rows, int cols, const void *A, int
         make_tensor_map(&hd, dtype, A, rows, cols, lda);
     }
     hd.scale = scale;
-    L = gemv_plan(dtype, hd.use_tma != 0, EPI_STORE, sms);
+    L = gemv_plan(dtype, hd.use_tma != 0, rows, cols, sms);
     MatDesc *dA = reinterpret_cast<MatDesc *>(base + OFF_DESC);
     State *st = reinterpret_cast<State *>(base + OFF_STATE);
     GemvScratch *scr = reinterpret_cast<GemvScratch *>(base + OFF_SCRATCH);
