@@ -1,13 +1,7 @@
-// gemv_split.h -- how the matrix-vector product (k_gemv.cu) deals its tiles to
-// the CTAs: whole row tiles, or equal pieces of the tile sequence.  Host and device
-// share this code (the host side is what the CPU test compiles).
+// gemv_split.h -- how the products (k_gemv.cu, k_bgemv.cu) deal their tiles to the
+// CTAs: whole row tiles, or equal pieces of the tile sequence.  Host code, which the
+// CPU tests compile too.
 #pragma once
-
-#if defined(__CUDACC__)
-#define LS_SPLIT_RULE_FN __host__ __device__ __forceinline__
-#else
-#define LS_SPLIT_RULE_FN inline
-#endif
 
 namespace lsi {
 
@@ -32,7 +26,7 @@ struct GemvCosts {
 // row tiles against equal pieces: n = 1024 10.3 and 16.4 us (pair), 10.3 and 20.5 (FP8);
 // n = 4000 28.9 and 35.9 (pair), 14.7 and 18.5 (BF16), 14.4 and 20.5 (FP32); n = 9500
 // 39.4 and 41.7 (BF16), but 35.4 and 29.1 for FP8, which takes pieces there.
-LS_SPLIT_RULE_FN bool gemv_whole_tiles(GemvCosts c, int RT, int CT, int G) {
+inline bool gemv_whole_tiles(GemvCosts c, int RT, int CT, int G) {
     if (RT < 1 || RT > G) return false;
     const long long share = G / RT < CT ? G / RT : CT;
     return (long long)CT * c.tile * G <= 2ll * RT * CT * c.piece + (c.meet + c.sharer * share) * G;
@@ -42,5 +36,23 @@ constexpr GemvCosts GEMV_COSTS_PAIR = {900, 540, 13000, 1000};
 constexpr GemvCosts GEMV_COSTS_BF16 = {560, 440, 6000, 950};
 constexpr GemvCosts GEMV_COSTS_FP8 = {920, 250, 13000, 1000};
 constexpr GemvCosts GEMV_COSTS_F32 = {520, 250, 5300, 1300};
+
+// ---- the block product -----------------------------------------------------------------
+// One CTA an SM; whole row blocks go to CTA c, c + G, ..., so the longest CTA has
+// ceil(RB / G) CT tiles, in equal pieces RB CT / G.  Pieces win when the tiles they
+// save take longer than the meeting of the CTAs that share a row block.
+struct BgemvCosts {
+    int tile, meet;   // ns
+};
+inline bool bgemv_whole_blocks(BgemvCosts c, long long RB, long long CT, long long G) {
+    const long long idle = (RB + G - 1) / G * CT * G - RB * CT;   // over all CTAs
+    return idle * c.tile < c.meet * G;
+}
+// Fitted to both forms at 20 sizes from n = 300 to 9801 (caches cold): the form chosen is
+// within 2 % of the faster one.  Eight columns: n = 1000 16.9 us whole, 23.8 in pieces; 2001
+// 26.2 and 34.3; 2450 53.2 and 42.0; 4500 87.3 and 92.3; 8000 287.9 and 249.7.
+inline BgemvCosts bgemv_costs(int S) {
+    return S <= 1 ? BgemvCosts{650, 8500} : S <= 2 ? BgemvCosts{870, 6500} : S <= 4 ? BgemvCosts{1370, 10400} : BgemvCosts{2400, 12800};
+}
 
 }  // namespace lsi

@@ -13,13 +13,16 @@
 // double-single (two-sum of the high parts, the low parts and rounding
 // errors summed apart, as the GEMV does), and the 32 lanes of a row add
 // their sums by shuffles at the end of the row block.  The (row block, column
-// tile) sequence is cut into equal pieces, one per CTA (whole row blocks left up to
-// a fifth of the SMs idle in the last round: n = 8192 has 512 of them; S = 16 and
-// small products keep them); the last of the CTAs that share a row block adds
-// their sums in CTA order, so results are deterministic.  Work per element of A is 12 FP32 operations per column of
+// tile) sequence is cut into equal pieces, one per CTA (whole row blocks leave up to
+// a fifth of the SMs idle in the last turn: n = 8192 has 512 of them), and the last of
+// the CTAs that share a row block adds their sums in CTA order, so results are
+// deterministic; where meeting costs more than that, and for S = 16, a CTA takes whole
+// row blocks (gemv_split.h).  Two kernels: with both forms in one, the whole row
+// blocks took up to half as long again.  Work per element of A is 12 FP32 operations per column of
 // P: compute-bound for S >= 4 (HBM-bound below).
 #include <cuda_runtime.h>
 
+#include "gemv_split.h"
 #include "ls_device.cuh"
 #include "ls_internal.h"
 #include "split_pair.h"
@@ -144,7 +147,8 @@ __global__ void bgemv_split_kernel(int n, int s, int S, const double *__restrict
     }
 }
 
-template <int S>
+// WHOLE: whole row blocks, CTA c: c, c + G, ...; else equal pieces (gemv_split.h).
+template <int S, bool WHOLE>
 __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc *__restrict__ dA, BgemvArgs a) {
     constexpr int BG_C = bg_consumers<S>();
     constexpr int RPW = bg_rows_per_warp<S>(), WS = 16 / RPW;   // rows per warp, their stride
@@ -158,17 +162,11 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
     count_launch(st);
     const int n = a.n;
     const int RB = (n + BG_TR - 1) / BG_TR, CT = (n + BG_TC - 1) / BG_TC;
-    // Equal pieces of the (row block, column tile) sequence, or whole row blocks (CTA c: c, c + G,
-    // ...) where those leave less idle time than adding shared ones up takes: a tile is about
-    // 0.3 S us, the sums 4 (n = 2000, s = 3: 5.6 ms a solve with whole blocks, 6.1 with pieces).
-    // Sixteen columns keep whole row blocks, by measurement (block GMRES, s = 16: n = 8192
-    // 40.4 ms a solve with whole blocks, 42.1 with pieces; n = 6000, s = 12 24.7 and 26.5).
     const long long T = (long long)RB * CT;
     const int G = gridDim.x, cta = blockIdx.x;
-    const bool whole = S == 16 || ((long long)((RB + G - 1) / G) * CT - T / G) * S < 16;
-    const long long t0 = whole ? (long long)cta * CT : bg_start(T, cta, G);
-    const int ntiles = whole ? (cta < RB ? (RB - cta + G - 1) / G * CT : 0) : (int)(bg_start(T, cta + 1, G) - t0);
-    const int first_rb = (int)(t0 / CT), rb_step = whole ? G : 1;
+    const long long t0 = WHOLE ? (long long)cta * CT : bg_start(T, cta, G);
+    const int ntiles = WHOLE ? (cta < RB ? (RB - cta + G - 1) / G * CT : 0) : (int)(bg_start(T, cta + 1, G) - t0);
+    const int first_rb = WHOLE ? cta : (int)(t0 / CT), rb_step = WHOLE ? G : 1;
     __shared__ int ca_s, cb_s, fin_s;
     if (threadIdx.x == 0) {
         for (int i = 0; i < NST; i++) {
@@ -227,7 +225,7 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
 #pragma unroll
             for (int j = 0; j < S; j++) acc[q][j] = {0.f, 0.f};
         const long long rfirst = (long long)rb * CT;
-        const int end = whole ? seq + CT : (int)min((long long)ntiles, rfirst + CT - t0);
+        const int end = WHOLE ? seq + CT : (int)min((long long)ntiles, rfirst + CT - t0);
         for (; seq < end; seq++) {
             const int sl = seq % NST;
             // on a timeout the warp stops waiting and computing but keeps walking
@@ -258,7 +256,7 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
                     acc[q][j] = f2_add(acc[q][j], b);
                 }
             }
-        if (whole || (t0 <= rfirst && rfirst + CT <= t0 + ntiles)) {
+        if (WHOLE || (t0 <= rfirst && rfirst + CT <= t0 + ntiles)) {
             if (g == 0)
 #pragma unroll
                 for (int q = 0; q < RPW; q++) {
@@ -268,7 +266,7 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
                         for (int j = 0; j < S; j++)
                             if (j < a.s) a.Q[(long long)j * a.ldq + row] = (double)acc[q][j].h + (double)acc[q][j].l;
                 }
-        } else if constexpr (S < 16) {
+        } else if constexpr (!WHOLE) {
             // shared with neighbouring CTAs: publish the partial sums; the last of
             // the sharing CTAs adds them in CTA order
             double *fix = a.scr->fix + (size_t)(2 * blockIdx.x + (rb == first_rb ? 0 : 1)) * BG_TR * S;
@@ -309,24 +307,33 @@ __global__ void __launch_bounds__(bg_threads<S>(), 1) bgemv_kernel(const MatDesc
 }
 
 namespace {
+// Sixteen columns keep whole row blocks, by measurement (block GMRES, s = 16: n = 8192
+// 40.4 ms a solve with whole blocks, 42.1 with pieces; n = 6000, s = 12 24.7 and 26.5).
 template <int S>
-void *bg_func() {
-    return reinterpret_cast<void *>(&bgemv_kernel<S>);
+void bg_set(BgemvLaunch &L, int n) {
+    L.smem = stages<S>() * stage_bytes<S>() + 1024;
+    if constexpr (S < 16) {
+        if (!bgemv_whole_blocks(bgemv_costs(S), (n + BG_TR - 1) / BG_TR, (n + BG_TC - 1) / BG_TC, L.grid)) {
+            L.func = reinterpret_cast<void *>(&bgemv_kernel<S, false>);
+            return;
+        }
+    }
+    L.func = reinterpret_cast<void *>(&bgemv_kernel<S, true>);
 }
 }  // namespace
 
-BgemvLaunch bgemv_plan(int s, int num_sms) {
+BgemvLaunch bgemv_plan(int n, int s, int num_sms) {
     BgemvLaunch L{};
     L.split = reinterpret_cast<void *>(&bgemv_split_kernel);
     L.grid = num_sms;
     L.S = s <= 1 ? 1 : s <= 2 ? 2 : s <= 4 ? 4 : s <= 8 ? 8 : 16;
     L.block = L.S <= 8 ? bg_threads<8>() : bg_threads<16>();
     switch (L.S) {
-        case 1: L.func = bg_func<1>(); L.smem = stages<1>() * stage_bytes<1>() + 1024; break;
-        case 2: L.func = bg_func<2>(); L.smem = stages<2>() * stage_bytes<2>() + 1024; break;
-        case 4: L.func = bg_func<4>(); L.smem = stages<4>() * stage_bytes<4>() + 1024; break;
-        case 8: L.func = bg_func<8>(); L.smem = stages<8>() * stage_bytes<8>() + 1024; break;
-        default: L.func = bg_func<16>(); L.smem = stages<16>() * stage_bytes<16>() + 1024; break;
+        case 1: bg_set<1>(L, n); break;
+        case 2: bg_set<2>(L, n); break;
+        case 4: bg_set<4>(L, n); break;
+        case 8: bg_set<8>(L, n); break;
+        default: bg_set<16>(L, n); break;
     }
     set_smem_limit(L.func, L.smem);
     return L;

@@ -90,7 +90,7 @@ int build_bcg_graph(ls_ctx *c, const BcgVecs &v, const BcgLayout &L, const GemvL
     Chain inner = outer.loop(hi);
     if (L.Ph) {
         // Q = A P in one pass over the pair of A (P split first)
-        const BgemvLaunch BL = bgemv_plan(v.s, c->num_sms);
+        const BgemvLaunch BL = bgemv_plan(v.n, v.s, c->num_sms);
         int nn = v.n, ss = v.s, SS = BL.S;
         const double *Pp = v.P;
         long long ld = v.ld, ldp = L.ldp;

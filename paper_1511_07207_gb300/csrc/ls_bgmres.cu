@@ -62,7 +62,7 @@ BgmLayout bgm_layout(void *base, int n, int s, int m, int grid, bool stageA) {
 
 int build_bgm_graph(ls_ctx *c, const BgmVecs &v, const BgmLayout &L, int x0_given, const long long *key) {
     const BgmKernels K = bgm_kernels();
-    const BgemvLaunch BL = bgemv_plan(v.s, c->num_sms);
+    const BgemvLaunch BL = bgemv_plan(v.n, v.s, c->num_sms);
     const size_t orth_smem = bgm_orth_smem(v.m, v.s), fin_smem = bgm_finish_smem(v.m, v.s);
     set_smem_limit(K.orth, orth_smem);
     set_smem_limit(K.finish, fin_smem);

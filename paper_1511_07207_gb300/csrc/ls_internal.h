@@ -409,7 +409,7 @@ struct BgemvLaunch {
     int grid, block, S;           // S: the kernel's column count (s rounded up to a power of two)
     size_t smem;
 };
-BgemvLaunch bgemv_plan(int s, int num_sms);
+BgemvLaunch bgemv_plan(int n, int s, int num_sms);
 
 struct KrylovKernels {
     void *cg_init, *cg_update, *cg_check;
