@@ -344,8 +344,8 @@ __device__ __forceinline__ void warp_sums(double (&s)[U]) {
 // second pass) and chains of dependent FP64 instructions between them.  So a warp
 // takes several columns of V at once, square roots and quotients come from one
 // reciprocal square root each, and whether a second pass is needed is read from ||w||^2 -
-// ||h||^2 (V is orthonormal) instead of a norm that every block waits for.  At n = 2000,
-// k = 8, two passes: 46 k cycles before.
+// ||h||^2 (V is orthonormal) instead of a norm that every block waits for.  n = 2000, mean of 17
+// steps, most with two passes (ncu, caches cold): 36.9 us before, 22.6 now; n = 16384 39.1 and 32.2.
 __global__ void __launch_bounds__(KB) gm_arnoldi_kernel(Vecs v, cudaGraphConditionalHandle h_inner) {
     __shared__ double red[KB / 32];
     __shared__ double h[LS_MAX_RESTART + 1];
